@@ -61,7 +61,8 @@ typedef struct {
 /* flags */
 #define LX_CART 0x0        /* Cartesian output, ncart(l) = (l+1)(l+2)/2 per shell */
 #define LX_SOLID 0x1       /* real solid-harmonic output, 2l+1 per shell */
-#define LX_PATH_FP64 0x0   /* every step in FP64 */
+#define LX_PATH_FP64 0x0   /* every step in FP64; quartets large enough take the two transforms through
+                              frames in which they are sparse (the axial form), the rest as GEMMs */
 #define LX_PATH_SPLIT 0x2  /* the two Hermite transforms as Ozaki-style BF16 slice products on the
                               tensor cores (FP32 accumulation, integer recombination); Boys,
                               [r]^(m), E and H stay FP64.  Operands carry 8 bits per digit kept
@@ -87,9 +88,9 @@ typedef struct {
 /* stages timed with LX_TIME_STAGES */
 #define LX_STAGE_NORM 0   /* contraction normalisation */
 #define LX_STAGE_PAIR 1   /* pair scalars and H matrices */
-#define LX_STAGE_BOYS_R 2 /* Boys function and [r]^(0) */
-#define LX_STAGE_GEMM1 3  /* [ab|q] = H_ab [p|q] */
-#define LX_STAGE_GEMM2 4  /* (ab|cd) = [ab|q] H_cd^T */
+#define LX_STAGE_BOYS_R 2 /* Boys function and [r]^(0) (axial form: its tables) */
+#define LX_STAGE_GEMM1 3  /* [ab|q] = H_ab [p|q] (axial form: both transforms, in the pairs' frames) */
+#define LX_STAGE_GEMM2 4  /* (ab|cd) = [ab|q] H_cd^T (axial form: rotation to the lab frame) */
 #define LX_STAGE_SPLIT 5  /* LX_PATH_SPLIT: FP64 operands -> BF16 digit planes */
 #define LX_STAGE_DIGEST 6 /* lx_eri_jk: blocks digested into J and K */
 #define LX_NSTAGE 7
@@ -191,9 +192,9 @@ int lx_eri_pairs(const lx_shell* shells, int32_t nshell, const double* exps, con
  *   quartets[].out_offset is not used (it must still be >= 0).
  *   workspace: as lx_eri_batch, sized by lx_eri_jk_workspace_size / _min.  On the FP64
  *     path J and K are contracted straight from [ab|q] (no second transform, no block
- *     stored); on the split path each quartet's block is written to the workspace by the
- *     second transform and streamed once by the digestion kernel.  Nothing is written to a
- *     caller output.
+ *     stored), or in the axial form from each block, kept in the room of [ab|q]; on the split
+ *     path each quartet's block is written to the workspace by the second transform and
+ *     streamed once by the digestion kernel.  Nothing is written to a caller output.
  * Flags, paths (LX_PATH_SPLIT, LX_PATH_ROUTED), staging and stream semantics as
  * lx_eri_batch; LX_TIME_STAGES times the digestion as LX_STAGE_DIGEST.  nbf <= 2^31 - 1.
  */
@@ -257,7 +258,7 @@ int lx_eri_graph_destroy(void* handle);
  * output kind): for each of the `max_keys` costliest keys of the batch, up to `samples` of its
  * quartets are evaluated with every tile shape (32x64, 64x32, 32x32, 64x64) and the fastest,
  * timed with CUDA events on cuda_stream, is recorded in the library's tuning table, which the
- * planner consults for every later call.  out (DEVICE, out_doubles long) and workspace are
+ * planner consults for every later call (for the quartets that take the GEMMs).  out (DEVICE, out_doubles long) and workspace are
  * scratch.  Synchronises cuda_stream.  The split path has a single tile shape: no-op.
  */
 int lx_eri_autotune(const lx_shell* shells, int32_t nshell, const double* exps, const double* coefs,

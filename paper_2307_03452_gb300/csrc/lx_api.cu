@@ -5,6 +5,8 @@
 //   boys_r  -> per primitive quartet: Boys function and [r]^(0) by Eq. md1
 //   gemm1   -> [ab|q] = H_ab [p|q]                                  (Eq. make-abq)
 //   gemm2   -> (ab|cd) = [ab|q] H_cd^T                              (Eq. make-abcd)
+// On the FP64 path most quartets take the axial form of the two transforms (lx_axial.cu;
+// axial_route says which).
 // The host side only validates, deduplicates shell pairs, lays out the caller's workspace
 // and builds work lists; every arithmetic step of the method runs in the kernels.
 #include <cmath>
@@ -18,6 +20,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "lx_axial.cuh"
 #include "lx_internal.cuh"
 #include "lx_split.cuh"
 
@@ -109,6 +112,7 @@ int ensure_device(unsigned** status) {
         if ((e = init_split_kernels(tuv.data())) != cudaSuccess) return cuda_fail(e);
         if ((e = init_jk_kernels()) != cudaSuccess) return cuda_fail(e);
         if ((e = init_router_kernels()) != cudaSuccess) return cuda_fail(e);
+        if ((e = init_axial(axial_tables())) != cudaSuccess) return cuda_fail(e);
         void* p = nullptr;
         if ((e = cudaGetSymbolAddress(&p, g_status_word)) != cudaSuccess) return cuda_fail(e);
         const unsigned zero = 0;
@@ -250,6 +254,47 @@ size_t pair_bytes(const lx_shell* sh, int sa, int sb, int flags) {
     return bytes;
 }
 
+// Workspace bytes of a quartet and of a pair in the axial form.
+size_t axial_quartet_bytes(const lx_shell* sh, const lx_quartet& q, int flags, bool full) {
+    const bool solid = flags & LX_SOLID;
+    const lx_shell &a = sh[q.s[0]], &b = sh[q.s[1]], &c = sh[q.s[2]], &d = sh[q.s[3]];
+    const int Lb = a.l + b.l, Lk = c.l + d.l;
+    const size_t nab = (size_t)nfun(a.l, solid) * nfun(b.l, solid), ncd = (size_t)nfun(c.l, solid) * nfun(d.l, solid);
+    const size_t prim = (size_t)a.nprim * b.nprim * c.nprim * d.nprim;
+    const size_t nhalf = axial_tables().cls[ax_class_id(a.l, b.l, solid)].nhalf;
+    const size_t items = prim + (nhalf + AX_NR - 1) / AX_NR + (nab + 7) / 8 + (ncd + 7) / 8;
+    size_t bytes = sizeof(AxQuartet) + items * sizeof(WorkItem) + 8 * prim * ax_t_size(Lb, Lk, full) + 256;
+    if (flags & JK_DIGEST) bytes += 8 * nab * ncd + 256;
+    return bytes;
+}
+
+size_t axial_pair_bytes(const lx_shell* sh, int sa, int sb, int flags) {
+    const lx_shell &a = sh[sa], &b = sh[sb];
+    const size_t kab = (size_t)a.nprim * b.nprim;
+    const AxClass& c = axial_tables().cls[ax_class_id(a.l, b.l, flags & LX_SOLID)];
+    return sizeof(AxPair) + kab * sizeof(WorkItem) + 8 * (kab * (4 + c.nh) + ax_rot_size(std::max(a.l, b.l))) + 512;
+}
+
+// How a quartet of the FP64 path is evaluated: 0 = matrix form, 1 = axial form with the
+// factors of the ket blocks in its tables, 2 = axial form with the full blocks.  A rule on its
+// class and contraction degrees alone, so that results do not depend on the batch, the chunk
+// or the workspace.  The matrix form stays for small classes, where it is the faster one
+// (AX_MIN_FMA), and where the axial form's tables (one per primitive quartet) would need more
+// workspace than the matrix form's [r]^(0) and [ab|q], which the workspace sizes are stated for.
+int axial_route(const lx_shell* sh, const lx_quartet& q, int flags) {
+    if (flags & LX_PATH_SPLIT) return 0;
+    const bool solid = flags & LX_SOLID;
+    const int Lb = sh[q.s[0]].l + sh[q.s[1]].l, Lk = sh[q.s[2]].l + sh[q.s[3]].l;
+    const int64_t nab = (int64_t)nfun(sh[q.s[0]].l, solid) * nfun(sh[q.s[1]].l, solid),
+                  ncd = (int64_t)nfun(sh[q.s[2]].l, solid) * nfun(sh[q.s[3]].l, solid);
+    if (nab * pyr(Lk) * (pyr(Lb) + ncd) < (nab < AX_FEW_ROWS ? AX_MIN_FMA_FEW : AX_MIN_FMA)) return 0;
+    if (axial_pair_bytes(sh, q.s[0], q.s[1], flags) > pair_bytes(sh, q.s[0], q.s[1], flags) ||
+        axial_pair_bytes(sh, q.s[2], q.s[3], flags) > pair_bytes(sh, q.s[2], q.s[3], flags))
+        return 0;
+    const size_t room = quartet_bytes(sh, q, flags);
+    return axial_quartet_bytes(sh, q, flags, true) <= room ? 2 : axial_quartet_bytes(sh, q, flags, false) <= room;
+}
+
 constexpr size_t CHUNK_SLACK = 32 * 256;  // alignment padding of the chunk's regions and the work counters
 
 size_t head_bytes(int nshell, int nprim) {
@@ -312,6 +357,13 @@ struct ChunkPlan {
     std::vector<WorkItem> items_sr, items_sB, items_sg1, items_sD, items_sg2;
     size_t off_srd = 0, off_sq = 0, off_sg1 = 0, off_sg2 = 0;
     size_t off_isr = 0, off_isB = 0, off_isg1 = 0, off_isD = 0, off_isg2 = 0;
+    // axial form (FP64 path): its own pairs and quartets
+    std::vector<AxPair> ax_pairs;
+    std::vector<AxQuartet> ax_quartets;
+    std::vector<WorkItem> ax_ip, ax_it, ax_im, ax_irk, ax_irb;  // pairs, tables, main, rotations of ket and bra
+    int ax_counts[AX_NBIN] = {0, 0, 0, 0}, ax_lmax = 0, ax_lanes_k = 16, ax_lanes_b = 16;
+    size_t ax_smem[AX_NBIN] = {0, 0, 0, 0}, ax_rot_k = 0, ax_rot_b = 0;
+    size_t off_axp = 0, off_axq = 0, off_aip = 0, off_ait = 0, off_aim = 0, off_airk = 0, off_airb = 0;
     size_t total = 0;         // bytes from the chunk base
     std::vector<char> blob;   // descriptor bytes [0, off_data)
 };
@@ -337,7 +389,27 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
     P.sg2.clear();
     for (auto* v : {&P.items_sr, &P.items_sB, &P.items_sg1, &P.items_sD, &P.items_sg2})
         v->clear();
-    std::unordered_map<PairKey, int, PairKeyHash> pid;
+    P.ax_pairs.clear();
+    P.ax_quartets.clear();
+    for (auto* v : {&P.ax_ip, &P.ax_it, &P.ax_im, &P.ax_irk, &P.ax_irb}) v->clear();
+    std::vector<int64_t> dense;  // index of each matrix-form quartet in qs
+    std::unordered_map<PairKey, int, PairKeyHash> pid, apid;
+    auto get_ax_pair = [&](int sa, int sb, int side) {
+        const PairKey k{((int64_t)sa << 32 | (uint32_t)sb) * 2 + side};
+        const auto ins = apid.emplace(k, (int)P.ax_pairs.size());
+        if (!ins.second) return ins.first->second;
+        AxPair p{};
+        p.sa = sa;
+        p.sb = sb;
+        p.Kab = sh[sa].nprim * sh[sb].nprim;
+        p.sign = side;
+        p.la = sh[sa].l;
+        p.lb = sh[sb].l;
+        p.cls = ax_class_id(p.la, p.lb, solid);
+        p.nh = axial_tables().cls[p.cls].nh;
+        P.ax_pairs.push_back(p);
+        return ins.first->second;
+    };
     auto get_pair = [&](int sa, int sb, int side) {
         const PairKey k{((int64_t)sa << 32 | (uint32_t)sb) * 2 + side};
         auto f = pid.find(k);
@@ -358,6 +430,27 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
     };
     for (int64_t i = ch.q_begin; i < ch.q_end; ++i) {
         const lx_quartet& q = qs[i];
+        const int route = ov.v1 < 0 ? axial_route(sh, q, flags) : 0;
+        if (route) {
+            const lx_shell &a = sh[q.s[0]], &b = sh[q.s[1]], &c = sh[q.s[2]], &dd = sh[q.s[3]];
+            AxQuartet x{};
+            x.pb = get_ax_pair(q.s[0], q.s[1], 0);
+            x.pk = get_ax_pair(q.s[2], q.s[3], 1);
+            x.kbra = a.nprim * b.nprim;
+            x.kket = c.nprim * dd.nprim;
+            x.Lb = a.l + b.l;
+            x.Lk = c.l + dd.l;
+            x.nab = nfun(a.l, solid) * nfun(b.l, solid);
+            x.ncd = nfun(c.l, solid) * nfun(dd.l, solid);
+            x.cb = ax_class_id(a.l, b.l, solid);
+            x.ck = ax_class_id(c.l, dd.l, solid);
+            x.full = route == 2;
+            x.tab_stride = ax_t_size(x.Lb, x.Lk, x.full);
+            x.out_off = q.out_offset;
+            P.ax_quartets.push_back(x);
+            continue;
+        }
+        dense.push_back(i);
         DQuartet d{};
         d.pb = get_pair(q.s[0], q.s[1], 0);
         d.pk = get_pair(q.s[2], q.s[3], 1);
@@ -372,6 +465,49 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
         d.nr = pyr(d.L);
         d.out_off = q.out_offset;
         P.quartets.push_back(d);
+    }
+    // work lists of the axial form: longest main items first (a rough count of their FMAs),
+    // grouped by the shared memory they need
+    for (int i = 0; i < (int)P.ax_pairs.size(); ++i)
+        for (int kp = 0; kp < P.ax_pairs[i].Kab; ++kp) P.ax_ip.push_back({i, kp, 0, 0});
+    {
+        struct Cost {
+            int bin;
+            int64_t c;
+            WorkItem w;
+        };
+        std::vector<Cost> main;
+        int nmax_k = 0, nmax_b = 0;
+        P.ax_lmax = 0;
+        for (int b = 0; b < AX_NBIN; ++b) {
+            P.ax_counts[b] = 0;
+            P.ax_smem[b] = 0;
+        }
+        for (const AxQuartet& x : P.ax_quartets) {
+            nmax_k = std::max(nmax_k, x.ncd);
+            nmax_b = std::max(nmax_b, x.nab);
+        }
+        P.ax_lanes_k = axial_lanes(nmax_k);
+        P.ax_lanes_b = axial_lanes(nmax_b);
+        P.ax_rot_k = axial_rotate_smem(nmax_k, P.ax_lanes_k);
+        P.ax_rot_b = axial_rotate_smem(nmax_b, P.ax_lanes_b);
+        for (int i = 0; i < (int)P.ax_quartets.size(); ++i) {
+            const AxQuartet& x = P.ax_quartets[i];
+            const int prim = x.kbra * x.kket, nhalf = axial_tables().cls[x.cb].nhalf, bin = axial_bin(x.Lb, x.Lk);
+            P.ax_lmax = std::max(P.ax_lmax, std::max(x.Lb, x.Lk));
+            P.ax_smem[bin] = std::max(P.ax_smem[bin], axial_main_smem(x.Lb, x.Lk));
+            for (int k = 0; k < prim; ++k) P.ax_it.push_back({i, k, 0, 0});
+            for (int r = 0; r < nhalf; r += AX_NR) {
+                const int n = std::min(AX_NR, nhalf - r);
+                main.push_back({bin, (int64_t)prim * pyr(x.Lk) * (2 * nhalf - r), {i, r, n, 0}});
+                ++P.ax_counts[bin];
+            }
+            for (int r = 0; r < x.nab; r += P.ax_lanes_k) P.ax_irk.push_back({i, r, 0, 0});
+            for (int r = 0; r < x.ncd; r += P.ax_lanes_b) P.ax_irb.push_back({i, r, 0, 0});
+        }
+        std::stable_sort(main.begin(), main.end(),
+                         [](const Cost& a, const Cost& b) { return a.bin != b.bin ? a.bin < b.bin : a.c > b.c; });
+        for (const Cost& c : main) P.ax_im.push_back(c.w);
     }
     // work lists
     for (int i = 0; i < (int)P.pairs.size(); ++i)
@@ -395,7 +531,7 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
             // untuned: 64-row tiles once the bra has 128 rows or more (measured on (ii|ii)),
             // 32-row tiles for smaller classes
             int v1 = d.nab >= 128 ? GEMM_V64x32 : GEMM_V32x64, v2 = v1;
-            auto f = g_tune.find(tune_key(sh, qs[ch.q_begin + i], solid));
+            auto f = g_tune.find(tune_key(sh, qs[dense[i]], solid));
             if (f != g_tune.end()) {
                 v1 = f->second.v1;
                 v2 = f->second.v2;
@@ -426,7 +562,7 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
             for (int qc = 16; qc >= 1; qc /= 2) {
                 size_t need = 0;
                 for (int i = 0; i < (int)P.quartets.size(); ++i) {
-                    const lx_quartet& qq = qs[ch.q_begin + i];
+                    const lx_quartet& qq = qs[dense[i]];
                     const int nb_ = nfun(sh[qq.s[1]].l, solid), nc_ = nfun(sh[qq.s[2]].l, solid),
                               nd_ = nfun(sh[qq.s[3]].l, solid);
                     need = std::max(need, jk_direct_smem(P.quartets[i].nab, P.quartets[i].ncd, nb_, nc_, nd_, qc));
@@ -524,6 +660,13 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
     region(P.off_isg1, sizeof(WorkItem) * P.items_sg1.size());
     region(P.off_isD, sizeof(WorkItem) * P.items_sD.size());
     region(P.off_isg2, sizeof(WorkItem) * P.items_sg2.size());
+    region(P.off_axp, sizeof(AxPair) * P.ax_pairs.size());
+    region(P.off_axq, sizeof(AxQuartet) * P.ax_quartets.size());
+    region(P.off_aip, sizeof(WorkItem) * P.ax_ip.size());
+    region(P.off_ait, sizeof(WorkItem) * P.ax_it.size());
+    region(P.off_aim, sizeof(WorkItem) * P.ax_im.size());
+    region(P.off_airk, sizeof(WorkItem) * P.ax_irk.size());
+    region(P.off_airb, sizeof(WorkItem) * P.ax_irb.size());
     P.off_data = o;
     // data regions: FP64 blocks in doubles from the workspace base, digit planes in bytes
     int64_t dw = (int64_t)((chunk_base + o) / 8);
@@ -539,6 +682,15 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
         d.rr_off = take((int64_t)d.kbra * d.kket * d.nr);
         d.x_off = take((int64_t)d.nab * d.kket * d.nq);
         if (jk && split) d.out_off = take((int64_t)d.nab * d.ncd);  // doubles from the workspace base
+    }
+    for (auto& p : P.ax_pairs) {
+        p.info_off = take(4 * (int64_t)p.Kab + ax_rot_size(std::max(p.la, p.lb)));
+        p.rot_off = p.info_off + 4 * (int64_t)p.Kab;
+        p.h_off = take((int64_t)p.Kab * p.nh);
+    }
+    for (auto& x : P.ax_quartets) {
+        x.tab_off = take((int64_t)x.kbra * x.kket * x.tab_stride);
+        if (jk) x.out_off = take((int64_t)x.nab * x.ncd);
     }
     if (split) {
         auto take_bytes = [&](int64_t bytes) { return 8 * take((bytes + 7) / 8); };
@@ -625,6 +777,13 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
     put(P.off_isg1, P.items_sg1.data(), sizeof(WorkItem) * P.items_sg1.size());
     put(P.off_isD, P.items_sD.data(), sizeof(WorkItem) * P.items_sD.size());
     put(P.off_isg2, P.items_sg2.data(), sizeof(WorkItem) * P.items_sg2.size());
+    put(P.off_axp, P.ax_pairs.data(), sizeof(AxPair) * P.ax_pairs.size());
+    put(P.off_axq, P.ax_quartets.data(), sizeof(AxQuartet) * P.ax_quartets.size());
+    put(P.off_aip, P.ax_ip.data(), sizeof(WorkItem) * P.ax_ip.size());
+    put(P.off_ait, P.ax_it.data(), sizeof(WorkItem) * P.ax_it.size());
+    put(P.off_aim, P.ax_im.data(), sizeof(WorkItem) * P.ax_im.size());
+    put(P.off_airk, P.ax_irk.data(), sizeof(WorkItem) * P.ax_irk.size());
+    put(P.off_airb, P.ax_irb.data(), sizeof(WorkItem) * P.ax_irb.size());
 }
 
 // Workspace bytes that plan_chunks needs to keep quartets [b, e) in one chunk (an upper
@@ -692,10 +851,19 @@ int plan_batch(const lx_shell* shells, int32_t nshell, const double* exps, const
         std::memcpy(B.head_blob.data() + B.o_exps, exps, sizeof(double) * (size_t)nprim_total);
         std::memcpy(B.head_blob.data() + B.o_coefs, coefs, sizeof(double) * (size_t)nprim_total);
     }
-    B.chunks.resize(chunks.size());
     for (size_t c = 0; c < chunks.size(); ++c) {
-        build_chunk(shells, quartets, chunks[c], pflags, B.head, B.chunks[c], ov);
-        if (B.head + B.chunks[c].total > workspace_bytes) return LX_ERR_WORKSPACE;
+        B.chunks.emplace_back();
+        build_chunk(shells, quartets, chunks[c], pflags, B.head, B.chunks.back(), ov);
+        if (B.head + B.chunks.back().total <= workspace_bytes) continue;
+        // a pair used by matrix-form and by axial quartets of one chunk is stored in both forms,
+        // which plan_chunks does not count: halve such a chunk
+        Chunk half = chunks[c];
+        if (half.q_end - half.q_begin < 2) return LX_ERR_WORKSPACE;
+        half.q_begin += (half.q_end - half.q_begin) / 2;
+        chunks[c].q_end = half.q_begin;
+        chunks.insert(chunks.begin() + c + 1, half);
+        B.chunks.pop_back();
+        --c;
     }
     return LX_OK;
 }
@@ -749,16 +917,24 @@ int enqueue_batch(const PlannedBatch& B, const char* head_src, const std::vector
         const WorkItem* d_ibr = reinterpret_cast<const WorkItem*>(base + P.off_br);
         const WorkItem* d_ig1 = reinterpret_cast<const WorkItem*>(base + P.off_g1);
         const WorkItem* d_ig2 = reinterpret_cast<const WorkItem*>(base + P.off_g2);
+        const AxPair* d_axp = reinterpret_cast<const AxPair*>(base + P.off_axp);
+        const AxQuartet* d_axq = reinterpret_cast<const AxQuartet*>(base + P.off_axq);
+        auto ax = [&](size_t off) { return reinterpret_cast<const WorkItem*>(base + off); };
+        const bool axial = !P.ax_quartets.empty(), matrix = !P.quartets.empty();
         if ((e = tm.begin()) != cudaSuccess) return cuda_fail(e);
         if ((e = launch_pair_h(d_pairs, d_ih, (int)P.items_h.size(), d_sh, d_exps, d_ncoef, ws, ws, solid, split,
-                               P.fold_lcap, P.fold_qcap, P.fold_wcap, P.fold_gcap, status, st)) != cudaSuccess)
+                               P.fold_lcap, P.fold_qcap, P.fold_wcap, P.fold_gcap, status, st)) != cudaSuccess ||
+            (e = launch_axial_pair(d_axp, ax(P.off_aip), (int)P.ax_ip.size(), d_sh, d_exps, d_ncoef, ws, solid, st)) !=
+                cudaSuccess)
             return cuda_fail(e);
-        if ((e = tm.end(LX_STAGE_PAIR, 1)) != cudaSuccess) return cuda_fail(e);
+        if ((e = tm.end(LX_STAGE_PAIR, matrix + axial)) != cudaSuccess) return cuda_fail(e);
         if ((e = tm.begin()) != cudaSuccess) return cuda_fail(e);
         if ((e = launch_boys_r(d_q, d_pairs, d_ibr, (int)P.items_br.size(), P.br_lmax, ws, status, st)) !=
-            cudaSuccess)
+                cudaSuccess ||
+            (e = launch_axial_boys(d_axq, d_axp, ax(P.off_ait), (int)P.ax_it.size(), ws, st)) != cudaSuccess ||
+            (e = launch_axial_wigner(d_axq, ax(P.off_ait), (int)P.ax_it.size(), P.ax_lmax, ws, st)) != cudaSuccess)
             return cuda_fail(e);
-        if ((e = tm.end(LX_STAGE_BOYS_R, 1)) != cudaSuccess) return cuda_fail(e);
+        if ((e = tm.end(LX_STAGE_BOYS_R, matrix + 2 * axial)) != cudaSuccess) return cuda_fail(e);
         if (split) {
             auto at = [&](size_t off) { return base + off; };
             const SplitRowsDesc* d_srd = reinterpret_cast<const SplitRowsDesc*>(at(P.off_srd));
@@ -789,25 +965,38 @@ int enqueue_batch(const PlannedBatch& B, const char* head_src, const std::vector
                 return cuda_fail(e);
             if ((e = tm.end(LX_STAGE_GEMM2, 1)) != cudaSuccess) return cuda_fail(e);
         } else {
+            int launches1 = 0, launches2 = 0;
+            for (int v = 0; v < GEMM_NVARIANT; ++v) {
+                launches1 += P.g1_counts[v] > 0;
+                launches2 += P.g2_counts[v] > 0;
+            }
+            for (int b = 0; b < AX_NBIN; ++b) launches1 += P.ax_counts[b] > 0;
             if ((e = tm.begin()) != cudaSuccess) return cuda_fail(e);
             int* d_counters = reinterpret_cast<int*>(base + P.off_counters);
-            if ((e = launch_gemm1(d_q, d_pairs, d_ig1, P.g1_counts, ws, d_counters, status, st)) != cudaSuccess)
+            if ((e = launch_gemm1(d_q, d_pairs, d_ig1, P.g1_counts, ws, d_counters, status, st)) != cudaSuccess ||
+                (e = launch_axial_main(d_axq, d_axp, ax(P.off_aim), P.ax_counts, P.ax_smem, ws, out, st)) != cudaSuccess)
                 return cuda_fail(e);
-            if ((e = tm.end(LX_STAGE_GEMM1, 1)) != cudaSuccess) return cuda_fail(e);
+            if ((e = tm.end(LX_STAGE_GEMM1, launches1)) != cudaSuccess) return cuda_fail(e);
+            if ((e = tm.begin()) != cudaSuccess) return cuda_fail(e);
+            // J and K of matrix-form quartets come straight from [ab|q]: no second transform
+            if ((!jk && (e = launch_gemm2(d_q, d_pairs, d_ig2, P.g2_counts, ws, out, d_counters + GEMM_NVARIANT, status,
+                                          st)) != cudaSuccess) ||
+                (e = launch_axial_rotate(1, d_axq, d_axp, ax(P.off_airk), (int)P.ax_irk.size(), P.ax_lanes_k,
+                                         P.ax_rot_k, ws, out, solid, st)) != cudaSuccess ||
+                (e = launch_axial_rotate(0, d_axq, d_axp, ax(P.off_airb), (int)P.ax_irb.size(), P.ax_lanes_b,
+                                         P.ax_rot_b, ws, out, solid, st)) != cudaSuccess)
+                return cuda_fail(e);
+            if ((e = tm.end(LX_STAGE_GEMM2, launches2 + 2 * axial)) != cudaSuccess) return cuda_fail(e);
             if (jk) {
-                // J and K straight from [ab|q]: no second transform, no stored block
                 if ((e = tm.begin()) != cudaSuccess) return cuda_fail(e);
                 if ((e = launch_jk_direct(d_q, d_pairs, d_sh, (int)P.quartets.size(), P.jkd_qc, P.jkd_smem, ws,
-                                          solid, jk->D, jk->nbf, jk->J, jk->K, st)) != cudaSuccess)
+                                          solid, jk->D, jk->nbf, jk->J, jk->K, st)) != cudaSuccess ||
+                    (e = launch_jk_digest(d_axq, d_axp, d_sh, (int)P.ax_quartets.size(), ws, solid, jk->D, jk->nbf,
+                                          jk->J, jk->K, st)) != cudaSuccess)
                     return cuda_fail(e);
-                if ((e = tm.end(LX_STAGE_DIGEST, 1)) != cudaSuccess) return cuda_fail(e);
+                if ((e = tm.end(LX_STAGE_DIGEST, matrix + axial)) != cudaSuccess) return cuda_fail(e);
                 continue;
             }
-            if ((e = tm.begin()) != cudaSuccess) return cuda_fail(e);
-            if ((e = launch_gemm2(d_q, d_pairs, d_ig2, P.g2_counts, ws, out, d_counters + GEMM_NVARIANT, status,
-                                  st)) != cudaSuccess)
-                return cuda_fail(e);
-            if ((e = tm.end(LX_STAGE_GEMM2, 1)) != cudaSuccess) return cuda_fail(e);
         }
         if (jk) {
             if ((e = tm.begin()) != cudaSuccess) return cuda_fail(e);

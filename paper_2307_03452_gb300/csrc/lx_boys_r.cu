@@ -15,6 +15,7 @@
 #include <cstring>
 #include <vector>
 
+#include "lx_axial.cuh"
 #include "lx_internal.cuh"
 
 namespace lx {
@@ -127,6 +128,101 @@ __global__ void __launch_bounds__(32) boys_r_kernel(const DQuartet* __restrict__
     for (int r = lane; r < nr; r += 32) out[r] = R[r];
 }
 
+// Axial form (lx_axial.cu): 8 lanes per primitive quartet (item.q, item.a = kp kket + kq) write
+// the angles of its frames and the table B_kappa(L) Z^L.  Geometry and Boys values are computed
+// alike in the 8 lanes (one instruction serves 4 quartets), powers and table rows are spread
+// over them.
+constexpr int AXB_THREADS = 64, AXB_GROUPS = AXB_THREADS / 8;
+__global__ void __launch_bounds__(AXB_THREADS) axial_boys_kernel(const AxQuartet* __restrict__ qd,
+                                                                 const AxPair* __restrict__ pairs,
+                                                                 const WorkItem* __restrict__ items, int nitems,
+                                                                 double* __restrict__ ws) {
+    __shared__ double F[AXB_GROUPS][LTOT + 1], row[AXB_GROUPS][2][LTOT + 2], zp_[AXB_GROUPS][LTOT + 1];
+    const int g = threadIdx.x >> 3, sub = threadIdx.x & 7;
+    const int item = blockIdx.x * AXB_GROUPS + g;
+    const bool live = item < nitems;
+    const WorkItem it = items[live ? item : nitems - 1];
+    const AxQuartet q = qd[it.q];
+    const AxPair pb = pairs[q.pb], pk = pairs[q.pk];
+    const int kp = it.a / q.kket, kq = it.a - kp * q.kket, Lt = q.Lb + q.Lk;
+    const double* ib = ws + pb.info_off + 4 * (int64_t)kp;
+    const double* ik = ws + pk.info_off + 4 * (int64_t)kq;
+    const double *Fb = ws + pb.rot_off, *Fk = ws + pk.rot_off;
+    const double zp = ib[0], zq = ik[0];
+    const double v[3] = {ib[1] - ik[1], ib[2] - ik[2], ib[3] - ik[3]};
+    const double R2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+    double n[3];
+    const double Z = ax_unit3(v, n);
+    const double rho = zp * zq / (zp + zq), T = rho * R2;
+    const double pref = 2.0 * PI * PI * sqrt(PI) / (zp * zq * sqrt(zp + zq));
+    double* tab = ws + q.tab_off + (int64_t)it.a * q.tab_stride;
+    // bra rotation: PQ in the AB frame (no rotation for P = Q)
+    double c = 1.0, s = 0.0, cg = 1.0, sg = 0.0;
+    if (Z > 0.0) {
+        c = Fb[6] * n[0] + Fb[7] * n[1] + Fb[8] * n[2];
+        s = ax_unit(Fb[0] * n[0] + Fb[1] * n[1] + Fb[2] * n[2], Fb[3] * n[0] + Fb[4] * n[1] + Fb[5] * n[2], cg, sg);
+    }
+    const double nrm = 1.0 / sqrt(c * c + s * s);
+    c *= nrm;
+    s *= nrm;
+    // PQ frame in the lab, and the ket rotation Rm = F_cd F_pq^T = Rz(a) Ry Rz(b)
+    double Fp[9], Rm[9];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const double r0 = cg * Fb[i] + sg * Fb[3 + i];
+        Fp[i] = c * r0 - s * Fb[6 + i];
+        Fp[3 + i] = cg * Fb[3 + i] - sg * Fb[i];
+        Fp[6 + i] = s * r0 + c * Fb[6 + i];
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            Rm[3 * i + j] = Fk[3 * i] * Fp[3 * j] + Fk[3 * i + 1] * Fp[3 * j + 1] + Fk[3 * i + 2] * Fp[3 * j + 2];
+    double cb, sb, c2 = Rm[8], s2 = ax_unit(Rm[6], Rm[7], cb, sb);
+    const double nrm2 = 1.0 / sqrt(c2 * c2 + s2 * s2);
+    c2 *= nrm2;
+    s2 *= nrm2;
+    // a from what Rz(b) and Ry leave of Rm, so that a and b stay consistent when s2 is tiny:
+    // row 0 of Rm Rz(b)^T Ry^T with Rz(b)^T = [[cb, -sb], [sb, cb]], Ry^T = [[c2, 0, s2], [0, 1, 0], [-s2, 0, c2]]
+    double ca = c2 * (Rm[0] * cb + Rm[1] * sb) - s2 * Rm[2], sa = Rm[1] * cb - Rm[0] * sb;
+    const double nrm3 = 1.0 / sqrt(ca * ca + sa * sa);
+    ca *= nrm3;
+    sa *= nrm3;
+    if (live && sub == 0) {
+        tab[0] = c, tab[1] = s, tab[2] = cg, tab[3] = sg, tab[4] = c2, tab[5] = s2;
+        tab[6] = ca, tab[7] = sa, tab[8] = cb, tab[9] = sb;
+        boys_eval(Lt, T, F[g]);
+    }
+    __syncwarp();
+    // 0 Z^L is taken as 0 and the square of Z kept finite: at separations where F_L underflows
+    // the powers of Z may overflow
+    double* bz = tab + AX_T_BZ;
+    const double R2f = fmin(R2, 1e300);
+    const double ex = exp(-T);
+    double* cur = row[g][0];
+    double* nxt = row[g][1];
+    for (int L = sub; L <= Lt; L += 8) {
+        const double pw = (L & 1 ? -pref : pref) * pow(2.0 * rho, (double)L), zl = pow(Z, (double)L);
+        zp_[g][L] = zl;
+        const double b0 = pw * F[g][L];
+        if (live) bz[ax_bz(L) + (L >> 1)] = b0 != 0.0 ? b0 * zl : 0.0;
+        if (L) cur[L - 1] = pw * ex;  // kappa = 1
+    }
+    __syncwarp();
+    for (int ka = 1; 2 * ka <= Lt; ++ka) {
+        for (int L = sub; L <= Lt - 2 * ka; L += 8) {
+            const double x = cur[L];
+            if (live) bz[ax_bz(2 * ka + L) + (L >> 1)] = x != 0.0 ? x * zp_[g][L] : 0.0;
+            if (L <= Lt - 2 * ka - 2) nxt[L] = fma(R2f, cur[L + 2], (2 * L + 3) * cur[L + 1]);
+        }
+        __syncwarp();
+        double* t = cur;
+        cur = nxt;
+        nxt = t;
+    }
+}
+
 __global__ void boys_stage_kernel(int mmax, const double* __restrict__ T, int64_t n, double* __restrict__ F,
                                   unsigned* status) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -198,6 +294,13 @@ cudaError_t launch_boys_r(const DQuartet* qd, const DPair* pairs, const WorkItem
     if (lmax < 0 || lmax > LTOT) return cudaErrorInvalidValue;
     const size_t smem = sizeof(double) * (pyr(lmax) + LTOT + 1);
     boys_r_kernel<<<nitems, 32, smem, st>>>(qd, pairs, items, ws, status);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_axial_boys(const AxQuartet* qd, const AxPair* pairs, const WorkItem* items, int nitems, double* ws,
+                              cudaStream_t st) {
+    if (nitems <= 0) return cudaSuccess;
+    axial_boys_kernel<<<(nitems + AXB_GROUPS - 1) / AXB_GROUPS, AXB_THREADS, 0, st>>>(qd, pairs, items, nitems, ws);
     return cudaGetLastError();
 }
 

@@ -16,6 +16,7 @@
 // outputs with one atomic per entry.
 #include <numeric>
 
+#include "lx_axial.cuh"
 #include "lx_internal.cuh"
 
 namespace lx {
@@ -25,8 +26,9 @@ namespace {
 constexpr int JK_THREADS = 256;
 constexpr int JK_PAIRS = NCART_MAX * NCART_MAX;  // (nu, lam) pairs of one mu, at most
 
-__global__ void __launch_bounds__(JK_THREADS) jk_digest_kernel(const DQuartet* __restrict__ qd,
-                                                               const DPair* __restrict__ pairs,
+template <typename Q, typename P>  // DQuartet and DPair, or their axial counterparts
+__global__ void __launch_bounds__(JK_THREADS) jk_digest_kernel(const Q* __restrict__ qd,
+                                                               const P* __restrict__ pairs,
                                                                const DShell* __restrict__ sh, int nquartet,
                                                                int stride,
                                                                const double* __restrict__ ws, int solid,
@@ -38,8 +40,8 @@ __global__ void __launch_bounds__(JK_THREADS) jk_digest_kernel(const DQuartet* _
     __shared__ double sk[JK_PAIRS];   // k(nu, lam)
     // neighbouring quartets often share a pair, and so the J or K entries they add to: CTAs
     // that run at the same time take quartets a large stride apart
-    const DQuartet q = qd[(int)(((int64_t)blockIdx.x * stride) % nquartet)];
-    const DPair pb = pairs[q.pb], pk = pairs[q.pk];
+    const Q q = qd[(int)(((int64_t)blockIdx.x * stride) % nquartet)];
+    const P pb = pairs[q.pb], pk = pairs[q.pk];
     const DShell sa = sh[pb.sa], sb = sh[pb.sb], sc = sh[pk.sa], sd = sh[pk.sb];
     const int na = solid ? 2 * sa.l + 1 : ncart(sa.l);
     const int nb = solid ? 2 * sb.l + 1 : ncart(sb.l);
@@ -228,15 +230,27 @@ cudaError_t init_jk_kernels() {
     return cudaFuncSetAttribute(jk_direct_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)JKD_SMEM_MAX);
 }
 
-cudaError_t launch_jk_digest(const DQuartet* qd, const DPair* pairs, const DShell* sh, int nquartet,
-                             const double* ws, bool solid, const double* D, int64_t nbf, double* J, double* K,
-                             cudaStream_t st) {
+template <typename Q, typename P>
+static cudaError_t digest(const Q* qd, const P* pairs, const DShell* sh, int nquartet, const double* ws, bool solid,
+                          const double* D, int64_t nbf, double* J, double* K, cudaStream_t st) {
     if (nquartet <= 0 || (!J && !K)) return cudaSuccess;
     int stride = 7919;  // prime; coprime with nquartet, so the map below is a permutation
     while (nquartet > 1 && std::gcd(stride, nquartet) != 1) stride += 2;
     jk_digest_kernel<<<nquartet, JK_THREADS, 0, st>>>(qd, pairs, sh, nquartet, stride, ws, solid ? 1 : 0, D, nbf, J,
                                                       K);
     return cudaGetLastError();
+}
+
+cudaError_t launch_jk_digest(const DQuartet* qd, const DPair* pairs, const DShell* sh, int nquartet,
+                             const double* ws, bool solid, const double* D, int64_t nbf, double* J, double* K,
+                             cudaStream_t st) {
+    return digest(qd, pairs, sh, nquartet, ws, solid, D, nbf, J, K, st);
+}
+
+cudaError_t launch_jk_digest(const AxQuartet* qd, const AxPair* pairs, const DShell* sh, int nquartet,
+                             const double* ws, bool solid, const double* D, int64_t nbf, double* J, double* K,
+                             cudaStream_t st) {
+    return digest(qd, pairs, sh, nquartet, ws, solid, D, nbf, J, K, st);
 }
 
 }  // namespace lx

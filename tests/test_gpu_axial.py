@@ -1,0 +1,94 @@
+"""The FP64 path's axial form at the sizes and geometries where it can go wrong, against the
+oracle: every tail of the 8-half-row and 16-lane tiles (l = 1..7, mixed within a pair), both
+outputs, contraction, directions along and against the frames' axes (no azimuth), coincident
+centers and P = Q, and batches that mix it with the matrix form.
+
+Bound: 1e-11 of the class's largest integral, the FP64 path's own (each class holds a compact
+quartet)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2307_03452_gb300 import inputs, lx
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-11
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _device():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    torch.cuda.set_device(0)
+
+
+def check(basis, quartets, solid, **kw):
+    out, off = lx.eri(basis, quartets, solid=solid, **kw)
+    ref, _ = oracle.eri(basis, quartets, solid=solid)
+    got = out.cpu().numpy()
+    assert np.all(np.isfinite(got))
+    l = np.asarray(basis["l"])
+    classes = {}
+    for i, q in enumerate(np.asarray(quartets)):
+        cls = tuple(int(l[s]) for s in q)
+        n = int(np.prod([2 * x + 1 if solid else (x + 1) * (x + 2) // 2 for x in cls]))
+        classes.setdefault(cls, []).append(np.arange(off[i], off[i] + n))
+    for cls, idx in classes.items():
+        idx = np.concatenate(idx)
+        scale, err = np.abs(ref[idx]).max(), np.abs(got[idx] - ref[idx]).max()
+        assert err <= TOL * scale, f"{cls}: {err:.3e} against {scale:.3e}"
+
+
+@pytest.mark.parametrize("solid", [True, False])
+@pytest.mark.parametrize("cls", [(1, 1, 1, 1), (2, 0, 1, 3), (2, 2, 2, 2), (3, 3, 3, 3), (4, 4, 4, 4), (5, 5, 5, 5),
+                                 (6, 6, 6, 6), (7, 7, 7, 7), (7, 0, 0, 7), (0, 6, 6, 1), (7, 1, 2, 5), (1, 7, 6, 3)])
+def test_classes(cls, solid):
+    kmax = 1 if sum(cls) > 20 else 2
+    basis, quartets = inputs.uniform_class(cls, 2 if sum(cls) > 20 else 5, 61, cube=1.5, exps=(0.2, 5.0), kmin=1, kmax=kmax)
+    check(basis, quartets, solid)
+
+
+@pytest.mark.parametrize("solid", [True, False])
+def test_directions_without_azimuth(solid):
+    # A, B, C, D on the z axis (either order), on the x axis, bra along z and ket along x, tiny
+    # tilts of 1e-9 and 1e-170, A = B, C = D, all coincident, P = Q with A != B
+    z, x, t = np.array([0, 0, 1.0]), np.array([1.0, 0, 0]), 1e-9
+    sets = [[0 * z, z, 2 * z, 3 * z], [3 * z, 2 * z, z, 0 * z], [0 * x, x, 2 * x, 3 * x], [0 * z, z, z + x, z + 2 * x],
+            [0 * z, z + t * x, 2 * z, 3 * z - t * x], [0 * z, z + 1e-170 * x, 2 * z, z], [z, z, 0 * z, x], [x, 0 * z, z, z],
+            [z, z, z, z], [-z, z, -x, x], [-x, x, -z, z], [0 * z, 1e-170 * x, z, z + 1e-160 * x]]
+    n = len(sets)
+    ls = np.tile([3, 2, 2, 3], n).astype(np.int32)
+    basis = {"l": ls, "nprim": np.ones(4 * n, np.int32), "prim_off": np.arange(4 * n, dtype=np.int32),
+             "center": np.concatenate(sets), "exps": np.full(4 * n, 0.7), "coefs": np.ones(4 * n)}
+    check(basis, np.arange(4 * n).reshape(n, 4), solid)
+
+
+def test_mixed_with_the_matrix_form_and_chunked():
+    # s and p pairs and K = 16 shells (too many tables) take the matrix form; pairs used by both
+    # forms; results do not depend on the workspace
+    rng = np.random.default_rng(62)
+    ls = np.array([0, 0, 1, 4, 5, 6, 3, 3], np.int32)
+    K = np.array([1, 2, 1, 1, 2, 1, 16, 16], np.int32)
+    off = np.concatenate([[0], np.cumsum(K)[:-1]]).astype(np.int32)
+    basis = {"l": ls, "nprim": K, "prim_off": off, "center": rng.uniform(0, 1.5, (8, 3)),
+             "exps": np.exp(rng.uniform(-1.0, 1.5, K.sum())), "coefs": 1 - rng.uniform(0, 1, K.sum())}
+    q = [[3, 4, 0, 1], [0, 1, 3, 4], [3, 4, 5, 4], [5, 5, 4, 3], [0, 2, 1, 0], [6, 7, 3, 4], [3, 4, 3, 4], [2, 1, 5, 5]]
+    check(basis, q, True)
+    b = lx.Batch(basis, q, True)
+    outs = []
+    for ws in (b.workspace_size(), b.workspace_min(), (b.workspace_size() + b.workspace_min()) // 2):
+        outs.append(torch.full((b.out_size,), float("nan"), dtype=torch.float64, device="cuda"))
+        b.run(outs[-1], lx.alloc_workspace(ws))
+        lx.sync_status()
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+
+
+def test_far_apart_stays_finite():
+    # separations at which F_m, and the powers of the distance, leave the FP64 range
+    for d in (1e6, 1e12, 1e160):
+        basis, quartets = inputs.uniform_class((6, 5, 6, 7), 1, 63, cube=1.0, exps=(0.5, 2.0))
+        basis["center"][2:] += np.array([d, 0.0, 0.0])
+        out, _ = lx.eri(basis, quartets, solid=True)
+        assert bool(torch.isfinite(out).all()), d

@@ -18,7 +18,7 @@
 // quartet of (ii|ii) in solid functions the bra rotation, T and the ket rotation take about
 // 1.4e6 FMAs where H_ab [p+q] takes 3.5e7, and the ket transform 7e5 where the second transform takes
 // 1.3e7; what remains is 1e6 FMAs per quartet to rotate the functions to the lab frame.  No
-// step leaves FP64.  2,048 (ii|ii) quartets, solid, K = 1: 194.4 -> 18.9 ms; 200 Cartesian ones 169.1 -> 34.1 ms;
+// step leaves FP64.  2,048 (ii|ii) quartets, solid, K = 1: 194.4 -> 15.8 ms; 200 Cartesian ones 169.1 -> 31.9 ms;
 // against 80-bit arithmetic the axial form's errors are at or below the matrix form's.
 //
 // Rows and columns are kept by half rows (AxHalf): the product of functions of orders m_a, m_b >= 0
@@ -405,6 +405,47 @@ __device__ __forceinline__ void r_task(int l, int mm, int mtop, bool first, doub
     }
 }
 
+// The same for a far primitive quartet (AX_FAR): k = k' = 0, 3 FMAs per (l, l', M') instead of
+// (nk + 2) nk'.  With centers in a 20-bohr cube and exponents of 0.05 to 20 half of the primitive
+// quartets are far: main kernel 12.5 -> 9.65 ms for 2,048 (ii|ii), 72.0 -> 45.4 ms for 200 mixed
+// quartets with K = 1..5; within 6 bohr 6.21 -> 6.14 ms.
+__device__ __forceinline__ void t_far(int lp, int Mp, int Lb, int lo, int M, const double* __restrict__ hs,
+                                      const int* __restrict__ hpre, const int* __restrict__ tinfo,
+                                      const double* __restrict__ T, const double* __restrict__ dC,
+                                      const double* __restrict__ dS, double* __restrict__ sc_out,
+                                      double* __restrict__ ss_out) {
+    double sc = 0.0, ss = 0.0;
+    for (int l = Lb; l >= max(lo, Mp); --l) {
+        const int info = tinfo[l * AX_NL + lp];
+        const double I = hs[hpre[l] * AX_NR] * T[(info >> 8) + Mp * (info & 255)];
+        const double c = l >= M ? dC[ax_co(l) + Mp * (l + 1) + M] : 0.0;
+        const double s = l >= M && M && Mp ? dS[ax_so(l) + (Mp - 1) * l + M - 1] : 0.0;
+        sc = fma(c, I, sc);
+        ss = fma(s, I, ss);
+    }
+    *sc_out = sc;
+    if (Mp) *ss_out = ss;
+}
+
+__device__ __forceinline__ void r_far(int l, int mm, int mtop, int nk, bool first, double cM, double sM,
+                                      const double* __restrict__ D, const double* __restrict__ SC,
+                                      const double* __restrict__ SS, double* __restrict__ X) {
+    const double* d = D + mm * (2 * l + 1) + l;
+    double ra = d[0] * SC[0], rb = 0.0;
+    for (int m = 1; m <= mtop; ++m) {
+        ra = fma(d[m], SC[m * nk * AX_NR], ra);
+        rb = fma(d[-m], SS[(m - 1) * nk * AX_NR], rb);
+    }
+    double2 v = make_double2(cM * ra - sM * rb, sM * ra + cM * rb);
+    double2* p = reinterpret_cast<double2*>(X + mm * nk * 2 * AX_NR);
+    if (!first) {
+        const double2 o = *p;
+        v.x += o.x;
+        v.y += o.y;
+    }
+    *p = v;
+}
+
 // One CTA per (quartet item.q, half rows item.a .. item.a + item.b - 1 of the bra class).  Lanes are
 // the 8 half rows (then the 16 rows: cosine, sine), so every table value is a broadcast and
 // every operand row one conflict-free shared access; groups of tasks are taken from shared
@@ -421,6 +462,7 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
     __shared__ int tinfo[AX_NL * AX_NL];
     __shared__ int hpre[AX_NL + 1], scp[AX_NL + 1], ssp[AX_NL + 1], xp[AX_NL + 1];
     __shared__ int ctr[3];
+    __shared__ unsigned farw[LX_KMAX * LX_KMAX / 32];  // far flags of the primitives of one kq
     __shared__ double cg[AX_NR][2];
     __shared__ AxHalf hr[AX_NR];
     const WorkItem it = items[blockIdx.x];
@@ -474,7 +516,20 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
     double* O = out + q.out_off;
 
     for (int kq = 0; kq < q.kket; ++kq) {
-        for (int kp = 0; kp < q.kbra; ++kp) {
+        for (int i = tid; i < (q.kbra + 31) / 32 * 32; i += THREADS) {
+            const bool f = i < q.kbra && ws[q.tab_off + (int64_t)(i * q.kket + kq) * q.tab_stride + AX_T_FAR] != 0.0;
+            const unsigned m = __ballot_sync(0xffffffffu, f);
+            if (lane == 0) farw[i >> 5] = m;
+        }
+        __syncthreads();
+        // near primitives first: a far one only adds to the k' = 0 entries of X, which are all that the
+        // ket transform reads if none is near
+        int done = 0, near = 0;
+        for (int kpp = 0; kpp < 2 * q.kbra; ++kpp) {
+            const int kp = kpp < q.kbra ? kpp : kpp - q.kbra;
+            const bool far = kpp >= q.kbra;
+            if ((farw[kp >> 5] >> (kp & 31) & 1u) != (far ? 1u : 0u)) continue;
+            near += !far;
             const double* tab = ws + q.tab_off + (int64_t)(kp * q.kket + kq) * q.tab_stride;
             const double* h = ws + pb.h_off + (int64_t)kp * pb.nh;
             for (int i = tid; i < ax_bz(Lb + Lk + 1); i += THREADS) BZ[i] = tab[AX_T_BZ + i];
@@ -488,9 +543,13 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
             if (tid == 0) ctr[1] = 0;
             __syncthreads();
             for (int i = tid; i < nT; i += THREADS) {
-                const int e = __ldg(c_ax.tent + t0 + i), n = e >> 23;
+                const int e = __ldg(c_ax.tent + t0 + i), n = e >> 23 & 15;
                 const double* gp = c_ax.g + (e & 0x3FFF);
                 const double* bz = BZ + ((e >> 14) & 0x1FF);
+                if (far) {
+                    if (e >> 27) T[i] = __ldg(gp + n - 1) * bz[n - 1];
+                    continue;
+                }
                 double t = 0.0;
                 for (int s = 0; s < n; ++s) t = fma(__ldg(gp + s), bz[s], t);
                 T[i] = t;
@@ -506,6 +565,10 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
                 const int lp = task & 255, Mp = task >> 8, nk = ax_nk(Lk, lp);
                 double* so = SC + (scp[lp] + Mp * nk) * AX_NR + r8;
                 double* zo = SS + (ssp[lp] + (Mp - 1) * nk) * AX_NR + r8;
+                if (far) {
+                    t_far(lp, Mp, Lb, lo, Mr, hs + r8, hpre, tinfo, T, dC, dS, so, zo);
+                    continue;
+                }
 #define AX_T(N)                                                                                    \
     case N:                                                                                        \
         t_task<N>(lp, Mp, Lb, lo, Mr, hs + r8, hpre, tinfo, T, dC, dS, so, zo);                    \
@@ -523,7 +586,7 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
                 full_blocks(Lk, td, td + 2 * (Lk + 1), C, C + ax_co(Lk + 1), D, tid, THREADS);
             }
             __syncthreads();
-            const bool first = kp == 0;
+            const bool first = done++ == 0;
             const double cM = cg[r8][0], sM = cg[r8][1];
             for (;;) {
                 int gi = 0;
@@ -533,6 +596,11 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
                 const int task = __ldg(c_ax.task_r + tr0 + 4 * gi + sub);
                 if (task < 0) continue;
                 const int l = task & 255, mm = task >> 8, nk = ax_nk(Lk, l), mtop = min(l, Lb);
+                if (far) {
+                    r_far(l, mm, mtop, nk, first, cM, sM, D + ax_do(l), SC + scp[l] * AX_NR + r8,
+                          SS + ssp[l] * AX_NR + r8, X + xp[l] * 2 * AX_NR + 2 * r8);
+                    continue;
+                }
 #define AX_R(N)                                                                                    \
     case N:                                                                                        \
         r_task<N>(l, mm, mtop, first, cM, sM, D + ax_do(l), SC + scp[l] * AX_NR + r8,              \
@@ -562,7 +630,7 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
                 const int nk = ax_nk(Lk, l);
                 const double* xc = X + (xp[l] + (l + M) * nk) * 2 * AX_NR + row;
                 const double* xs = X + (xp[l] + (l - M) * nk) * 2 * AX_NR + row;
-                for (int k = 0; k < nk; ++k) {
+                for (int k = 0; k < (near ? nk : 1); ++k) {
                     const double w = __ldg(hv + k);
                     vc = fma(w, xc[k * 2 * AX_NR], vc);
                     vs = fma(w, xs[k * 2 * AX_NR], vs);

@@ -67,10 +67,16 @@ __host__ __device__ inline int ax_bz(int N) { return (N - 1) * (N - 1) / 4 + N; 
 // Rotation data of a pair: frame (9), cos and sin of m phi (m = 0..LMAX), Y blocks l = 0..LMAX.
 constexpr int AX_ROT_CS = 10, AX_ROT_C = AX_ROT_CS + 2 * (LMAX + 1);
 __host__ __device__ inline int ax_rot_size(int l) { return AX_ROT_C + ax_co(l + 1) + ax_so(l + 1); }
-// Table of a primitive quartet: angles, B Z^L, cos and sin of M gamma, Y blocks of the bra
+// Table of a primitive quartet: angles, a flag (see AX_FAR), B Z^L, cos and sin of M gamma, Y blocks of the bra
 // rotation, and of the ket rotation either the full blocks or, at about half the size, their
 // factors: cos and sin of m a, of m b, Y blocks.
-constexpr int AX_T_BZ = 10;
+constexpr int AX_T_FAR = 10, AX_T_BZ = 12;
+// A primitive quartet is far if every B_kappa(L) Z^L with kappa >= 1 (a polynomial times e^-T) is below
+// AX_FAR of the B_0(N) Z^N of its degree N = 2 kappa + L: only T(l, l', M, 0) is then used, and of
+// it the L = l + l' term, the interaction of multipoles.  AX_FAR = 2^-100: [r]^(0) of degree N reaches
+// at least 2^-21 B_0(N) Z^N (the ratio of (2N-1)!! to N! at N = 24; 2^-25 at 28), so what is left out
+// lies 2^-20 and more below one rounding of the matrix form's entries of the same degree.
+constexpr double AX_FAR = 0x1p-100;
 __host__ __device__ inline int ax_t_cg(int Lb, int Lk) { return AX_T_BZ + ax_bz(Lb + Lk + 1); }
 __host__ __device__ inline int ax_t_c(int Lb, int Lk) { return ax_t_cg(Lb, Lk) + 2 * (Lb + 1); }
 __host__ __device__ inline int ax_t_d(int Lb, int Lk) { return ax_t_c(Lb, Lk) + ax_co(Lb + 1) + ax_so(Lb + 1); }

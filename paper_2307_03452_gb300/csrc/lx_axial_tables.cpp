@@ -168,7 +168,7 @@ void make_axial_tables(AxHost& H) {
                     for (int M = 0; M <= i; ++M)
                         for (int ka = 0; ka < n; ++ka) {
                             const int N = 2 * ka + i + j, L0 = j - i;
-                            H.tent.push_back(goff[i][j][M] | ((ax_bz(N) + (L0 >> 1)) << 14) | ((i + 1) << 23));
+                            H.tent.push_back(goff[i][j][M] | ((ax_bz(N) + (L0 >> 1)) << 14) | ((i + 1) << 23) | (ka ? 0 : 1 << 27));
                             ++at;
                         }
                 }

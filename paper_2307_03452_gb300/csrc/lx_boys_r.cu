@@ -206,14 +206,21 @@ __global__ void __launch_bounds__(AXB_THREADS) axial_boys_kernel(const AxQuartet
         const double pw = (L & 1 ? -pref : pref) * pow(2.0 * rho, (double)L), zl = pow(Z, (double)L);
         zp_[g][L] = zl;
         const double b0 = pw * F[g][L];
-        if (live) bz[ax_bz(L) + (L >> 1)] = b0 != 0.0 ? b0 * zl : 0.0;
+        const double b = b0 != 0.0 ? b0 * zl : 0.0;
+        if (live) bz[ax_bz(L) + (L >> 1)] = b;
+        F[g][L] = AX_FAR * fabs(b);  // each lane's own entries
         if (L) cur[L - 1] = pw * ex;  // kappa = 1
     }
     __syncwarp();
-    for (int ka = 1; 2 * ka <= Lt; ++ka) {
+    bool far = true;
+    // every lane takes the warp's longest loop, for the barriers: the groups' degrees may differ
+    const int Lw = __reduce_max_sync(0xffffffffu, Lt);
+    for (int ka = 1; 2 * ka <= Lw; ++ka) {
         for (int L = sub; L <= Lt - 2 * ka; L += 8) {
             const double x = cur[L];
-            if (live) bz[ax_bz(2 * ka + L) + (L >> 1)] = x != 0.0 ? x * zp_[g][L] : 0.0;
+            const double b = x != 0.0 ? x * zp_[g][L] : 0.0;
+            if (live) bz[ax_bz(2 * ka + L) + (L >> 1)] = b;
+            far = far && fabs(b) <= F[g][2 * ka + L];
             if (L <= Lt - 2 * ka - 2) nxt[L] = fma(R2f, cur[L + 2], (2 * L + 3) * cur[L + 1]);
         }
         __syncwarp();
@@ -221,6 +228,8 @@ __global__ void __launch_bounds__(AXB_THREADS) axial_boys_kernel(const AxQuartet
         cur = nxt;
         nxt = t;
     }
+    const unsigned all = __ballot_sync(0xffffffffu, far) >> (threadIdx.x & 24) & 0xffu;
+    if (live && sub == 0) tab[AX_T_FAR] = all == 0xffu ? 1.0 : 0.0;
 }
 
 __global__ void boys_stage_kernel(int mmax, const double* __restrict__ T, int64_t n, double* __restrict__ F,

@@ -92,3 +92,29 @@ def test_far_apart_stays_finite():
         basis["center"][2:] += np.array([d, 0.0, 0.0])
         out, _ = lx.eri(basis, quartets, solid=True)
         assert bool(torch.isfinite(out).all()), d
+
+
+def test_near_and_far_primitives():
+    # bra and ket 3 to 14 bohr apart, K = 2 with exponents 0.15 and 6: T of the primitive
+    # quartets spans about 1 to 600, so that within one quartet some take the multipole form and
+    # some do not (none at 3 bohr, all but one at 14).  Per quartet: 1e-11 of its own largest
+    # integral plus 20 times the oracle's noise under a rigid translation, as for far-separated
+    # quartets elsewhere.
+    seps = [3.0, 5.0, 6.5, 8.0, 10.0, 14.0]
+    n = len(seps)
+    rng = np.random.default_rng(64)
+    ls = np.array([[6, 6, 6, 6], [5, 4, 6, 6], [6, 5, 3, 4], [7, 6, 5, 7], [4, 4, 4, 4], [6, 6, 5, 5]], np.int32).reshape(-1)
+    K = np.full(4 * n, 2, np.int32)
+    c = rng.uniform(-0.4, 0.4, (n, 4, 3))
+    c[:, 2:] += np.array(seps)[:, None, None] * np.array([0.6, 0.0, 0.8])
+    basis = {"l": ls, "nprim": K, "prim_off": 2 * np.arange(4 * n, dtype=np.int32), "center": c.reshape(-1, 3),
+             "exps": np.tile([0.15, 6.0], 4 * n), "coefs": np.ones(8 * n)}
+    quartets = np.arange(4 * n).reshape(n, 4)
+    out, off = lx.eri(basis, quartets, solid=True)
+    got = out.cpu().numpy()
+    ref, _ = oracle.eri(basis, quartets, solid=True)
+    ref2, _ = oracle.eri(dict(basis, center=basis["center"] + np.array([0.37, -1.1, 0.53])), quartets, solid=True)
+    for i in range(n):
+        sl = slice(off[i], off[i] + int(np.prod(2 * ls[4 * i:4 * i + 4] + 1)))
+        noise = np.abs(ref[sl] - ref2[sl]).max()
+        assert np.abs(got[sl] - ref[sl]).max() <= TOL * np.abs(ref[sl]).max() + 20 * noise, seps[i]

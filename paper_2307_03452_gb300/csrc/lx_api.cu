@@ -816,6 +816,7 @@ int64_t prim_count(const lx_shell* sh, int32_t nshell) {
 // every chunk's descriptors, laid out for a workspace of `workspace_bytes`.
 struct PlannedBatch {
     int flags = 0, nshell = 0, nprim = 0;
+    int kmax = 0;  // largest contraction degree of the shells
     size_t head = 0, o_exps = 0, o_coefs = 0, o_ncoef = 0;
     std::vector<char> head_blob;  // bytes [0, o_ncoef) of the workspace
     std::vector<ChunkPlan> chunks;
@@ -839,6 +840,7 @@ int plan_batch(const lx_shell* shells, int32_t nshell, const double* exps, const
     for (int32_t s = 0; s < nshell; ++s) {
         dsh[s].l = shells[s].l;
         dsh[s].K = shells[s].nprim;
+        B.kmax = std::max(B.kmax, shells[s].nprim);
         dsh[s].prim_off = shells[s].prim_offset;
         dsh[s].bf = bf;
         bf += nfun(shells[s].l, flags & LX_SOLID);
@@ -903,7 +905,8 @@ int enqueue_batch(const PlannedBatch& B, const char* head_src, const std::vector
     double* d_ncoef = reinterpret_cast<double*>(wsb + B.o_ncoef);
     StageTimer tm{time_stages, st};
     if ((e = tm.begin()) != cudaSuccess) return cuda_fail(e);
-    if ((e = launch_norm(d_sh, nshell, d_exps, d_coefs, d_ncoef, status, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = launch_norm(d_sh, nshell, B.kmax, d_exps, d_coefs, d_ncoef, status, st)) != cudaSuccess)
+        return cuda_fail(e);
     if ((e = tm.end(LX_STAGE_NORM, 1)) != cudaSuccess) return cuda_fail(e);
     for (size_t c = 0; c < B.chunks.size(); ++c) {
         const NvtxRange chunk_range("lx_eri chunk");
@@ -1858,7 +1861,7 @@ int lx_hermite_H(const lx_shell* shells, int32_t nshell, const double* exps, con
     const double* d_exps = reinterpret_cast<const double*>(scratch + o_exps);
     const double* d_coefs = reinterpret_cast<const double*>(scratch + o_coefs);
     double* d_ncoef = reinterpret_cast<double*>(scratch + o_ncoef);
-    if ((e = launch_norm(d_sh, nshell, d_exps, d_coefs, d_ncoef, status, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = launch_norm(d_sh, nshell, LX_KMAX, d_exps, d_coefs, d_ncoef, status, st)) != cudaSuccess) return cuda_fail(e);
     int lcap = 0, qcap = 0, wcap = 0, gcap = 0;
     if (solid)
         for (const DPair& pr : dp) {

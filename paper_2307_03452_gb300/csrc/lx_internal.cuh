@@ -80,8 +80,8 @@ cudaError_t init_prep_tables(const double* host_coefs, const int* host_tuv,
                              const void* host_fold);  // lx_prep.cu (host_fold: const FoldHost*)
 cudaError_t init_tuv_table(const int* host_tuv);           // lx_gemm.cu
 
-cudaError_t launch_norm(const DShell* sh, int nshell, const double* exps, const double* coefs, double* ncoef,
-                        unsigned* status, cudaStream_t st);
+cudaError_t launch_norm(const DShell* sh, int nshell, int kmax, const double* exps, const double* coefs, double* ncoef,
+                        unsigned* status, cudaStream_t st);  // kmax: largest contraction degree of the shells
 // H blocks at ws + h_off, pair scalars at ws_info + info_off.
 cudaError_t launch_pair_h(const DPair* pairs, const WorkItem* items, int nitems, const DShell* sh,
                           const double* exps, const double* ncoef, double* ws, double* ws_info, bool solid,

@@ -42,30 +42,51 @@ __device__ inline double dfact_odd(int n) {
     return r;
 }
 
-// Normaliser of x^l exp(-zeta r^2): (2 zeta/pi)^{3/4} (4 zeta)^{l/2} / sqrt((2l-1)!!).
-__device__ inline double prim_norm(int l, double z) {
-    return pow(2.0 * z / PI, 0.75) * pow(4.0 * z, 0.5 * l) / sqrt(dfact_odd(l));
+// x^n for small n >= 0
+__device__ inline double int_power(double x, int n) {
+    double r = 1.0;
+    for (int k = 0; k < n; ++k) r *= x;
+    return r;
 }
 
-// One thread per shell: c'_i = c_i N(zeta_i, l) s, with s making the contracted x^l
-// function unit-normalised: sum_ij c'_i c'_j (2l-1)!! / (2(z_i+z_j))^l (pi/(z_i+z_j))^{3/2} = 1.
-__global__ void norm_kernel(const DShell* __restrict__ sh, int nshell, const double* __restrict__ exps,
-                            const double* __restrict__ coefs, double* __restrict__ ncoef, unsigned* status) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nshell) return;
-    const DShell d = sh[s];
+// Normaliser of x^l exp(-zeta r^2): (2 zeta/pi)^{3/4} (4 zeta)^{l/2} / sqrt((2l-1)!!).
+__device__ inline double prim_norm(int l, double z) {
+    const double s = sqrt(2.0 * z / PI);
+    return s * sqrt(s) * int_power(4.0 * z, l >> 1) * sqrt((l & 1 ? 4.0 * z : 1.0) / dfact_odd(l));
+}
+
+// G lanes per shell: c'_i = c_i N(zeta_i, l) s, with s making the contracted x^l function
+// unit-normalised: sum_ij c'_i c'_j (2l-1)!! / (2(z_i+z_j))^l (pi/(z_i+z_j))^{3/2} = 1.  Each
+// primitive's normaliser is computed once and the K^2 overlaps are spread over the lanes, with
+// square roots and short products for the half-integer powers (pow takes some 150 FP64
+// instructions, which this GPU issues at one per 20 cycles and SM); blocks of one warp
+// spread small batches over the SMs.
+constexpr int NORM_THREADS = 32;
+template <int G>
+__global__ void __launch_bounds__(NORM_THREADS) norm_kernel(const DShell* __restrict__ sh, int nshell,
+                                                            const double* __restrict__ exps,
+                                                            const double* __restrict__ coefs,
+                                                            double* __restrict__ ncoef, unsigned* status) {
+    __shared__ double cn[NORM_THREADS / G][LX_KMAX];
+    const int g = threadIdx.x / G, sub = threadIdx.x % G, s = blockIdx.x * (NORM_THREADS / G) + g;
+    DShell d{};
+    if (s < nshell) d = sh[s];  // a shell past the end has K = 0
     const int l = d.l, K = d.K, o = d.prim_off;
+    for (int i = sub; i < K; i += G) cn[g][i] = coefs[o + i] * prim_norm(l, exps[o + i]);
+    __syncwarp();
     double acc = 0.0;
     const double df = dfact_odd(l);
-    for (int i = 0; i < K; ++i)
-        for (int j = 0; j < K; ++j) {
-            const double zi = exps[o + i], zj = exps[o + j], ab = zi + zj;
-            const double ov = df / pow(2.0 * ab, l) * pow(PI / ab, 1.5);
-            acc += coefs[o + i] * coefs[o + j] * prim_norm(l, zi) * prim_norm(l, zj) * ov;
-        }
-    if (!(acc > 0.0)) set_status(status, ST_BAD_INPUT);
+    for (int e = sub; e < K * K; e += G) {
+        const int i = e / K, j = e - i * K;
+        const double ab = exps[o + i] + exps[o + j], r = PI / ab;
+        acc += cn[g][i] * cn[g][j] * (df / int_power(2.0 * ab, l) * (r * sqrt(r)));
+    }
+#pragma unroll
+    for (int w = G / 2; w > 0; w >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, w);
+    if (s >= nshell) return;
+    if (!(acc > 0.0) && sub == 0) set_status(status, ST_BAD_INPUT);
     const double sc = 1.0 / sqrt(acc);
-    for (int i = 0; i < K; ++i) ncoef[o + i] = coefs[o + i] * prim_norm(l, exps[o + i]) * sc;
+    for (int i = sub; i < K; i += G) ncoef[o + i] = cn[g][i] * sc;
 }
 
 constexpr int PAIR_THREADS = 128;
@@ -397,10 +418,14 @@ cudaError_t init_prep_tables(const double* host_coefs, const int* host_tuv, cons
     return cudaMemcpyToSymbol(g_tuv_prep, host_tuv, sizeof(int) * NHERM_TOT);
 }
 
-cudaError_t launch_norm(const DShell* sh, int nshell, const double* exps, const double* coefs, double* ncoef,
+cudaError_t launch_norm(const DShell* sh, int nshell, int kmax, const double* exps, const double* coefs, double* ncoef,
                         unsigned* status, cudaStream_t st) {
     if (nshell <= 0) return cudaSuccess;
-    norm_kernel<<<(nshell + 127) / 128, 128, 0, st>>>(sh, nshell, exps, coefs, ncoef, status);
+    const int g = kmax > 1 ? 8 : 1, per = NORM_THREADS / g, n = (nshell + per - 1) / per;
+    if (g == 1)
+        norm_kernel<1><<<n, NORM_THREADS, 0, st>>>(sh, nshell, exps, coefs, ncoef, status);
+    else
+        norm_kernel<8><<<n, NORM_THREADS, 0, st>>>(sh, nshell, exps, coefs, ncoef, status);
     return cudaGetLastError();
 }
 

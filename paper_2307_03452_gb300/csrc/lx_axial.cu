@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
     __shared__ double E[(LMAX + 1) * (LMAX + 1)][AXP_NV + 1];
     __shared__ double zpow[32];
     __shared__ double g[AXP_THREADS / 32][8][AXP_NV];
+    __shared__ double wt[AXP_THREADS / 32][16][8];  // weights of one half row: (ja, jb), q
     __shared__ double pw[4 * AX_LP + 2];
     const WorkItem it = items[blockIdx.x];
     const AxPair pr = pairs[it.q];
@@ -242,17 +243,23 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
         const int na = (la - ma) / 2, nb = (lb - mb) / 2, s0 = hr.slot ? min(ma, mb) : 0;
         const int nq = (L - M) / 2 + 1;  // q = 0 .. nq - 1, v = 0 .. L - M - 2q
         const double cf = pref * (ma && mb ? 0.5 : 1.0);
-        for (int e = lane; e < nq * AXP_NV; e += 32) {
-            const int q = e / AXP_NV, v = e - q * AXP_NV;
+        // weights of the terms, then the sums over them for the pairs (q, v) that occur
+        for (int e = lane; e < (na + 1) * 32; e += 32) {
+            const int ja = e >> 5, jb = e >> 3 & 3, q = e & 7, s = ja + jb + s0;
+            if (jb <= nb && q <= s)
+                wt[warp][4 * ja + jb][q] =
+                    cf * fa.alpha[ja] * fb.alpha[jb] * (__ldg(c_ax.tau + (M * 8 + s) * 8 + q) * zpow[s + q + M]);
+        }
+        __syncwarp();
+        const int npair = nq * (L - M + 2 - nq);  // sum over q of L - M - 2q + 1
+        for (int e = lane; e < npair; e += 32) {
+            int q = 0, v = e;
+            for (int nv = L - M + 1; v >= nv; nv -= 2, ++q) v -= nv;
             double t = 0.0;
-            if (v <= L - M - 2 * q)
-                for (int ja = 0; ja <= na; ++ja)
-                    for (int jb = max(0, q - s0 - ja); jb <= nb; ++jb) {
-                        const int s = ja + jb + s0;
-                        const double w = fa.alpha[ja] * fb.alpha[jb] * __ldg(c_ax.tau + (M * 8 + s) * 8 + q) * zpow[s + q + M];
-                        t = fma(w, E[(la - ma - 2 * ja) * (lb + 1) + lb - mb - 2 * jb][v], t);
-                    }
-            g[warp][q][v] = cf * t;
+            for (int ja = 0; ja <= na; ++ja)
+                for (int jb = max(0, q - s0 - ja); jb <= nb; ++jb)
+                    t = fma(wt[warp][4 * ja + jb][q], E[(la - ma - 2 * ja) * (lb + 1) + lb - mb - 2 * jb][v], t);
+            g[warp][q][v] = t;
         }
         __syncwarp();
         // entries (l, k), l = M .. L, k = 0 .. (L - l) / 2, of degree n = 2k + l
@@ -273,26 +280,27 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
 
 // ------------------------------------------------------------------ rotation blocks
 
-// One warp per primitive quartet (item.q, item.a = kp kket + kq): from the angles of the table,
-// cos, sin of M gamma, the Y blocks of the bra rotation and the full blocks of the rotation PQ ->
-// CD (z, y, z).
-__global__ void __launch_bounds__(32) axial_wigner_kernel(const AxQuartet* __restrict__ qd,
-                                                          const WorkItem* __restrict__ items, int lmax,
-                                                          double* __restrict__ ws) {
+// One CTA of two warps per primitive quartet (item.q, item.a = kp kket + kq): from the angles of
+// the table, cos and sin of M gamma and the Y blocks of the bra rotation (warp 0), the Y blocks of
+// the rotation PQ -> CD (warp 1), then the latter's full blocks (or its factors).
+constexpr int AXW_THREADS = 64;
+__global__ void __launch_bounds__(AXW_THREADS) axial_wigner_kernel(const AxQuartet* __restrict__ qd,
+                                                                   const WorkItem* __restrict__ items, int lmax,
+                                                                   double* __restrict__ ws) {
     extern __shared__ double sm[];
+    __shared__ double pw[2][4 * AX_LP + 2], ph[4 * AX_NL];  // ph: cos, sin of m a, then of m b: 4 (Lk + 1)
     double* C = sm;
     double* S = C + ax_co(lmax + 1);
-    double* pw = S + ax_so(lmax + 1);  // 4 AX_LP + 2
-    double* ph = pw + 4 * AX_LP + 2;   // cos, sin of m a, then of m b: 4 (Lk + 1)
     const WorkItem it = items[blockIdx.x];
     const AxQuartet q = qd[it.q];
     double* tab = ws + q.tab_off + (int64_t)it.a * q.tab_stride;
-    const int lane = threadIdx.x, Lb = q.Lb, Lk = q.Lk;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, Lb = q.Lb, Lk = q.Lk;
     auto sync = [] { __syncwarp(); };
-    if (lane < 3) {  // phases: gamma, then a and b of the ket rotation
-        const double c0 = tab[lane == 0 ? 2 : 4 + 2 * lane], s0 = tab[lane == 0 ? 3 : 5 + 2 * lane];
-        double* o = lane == 0 ? tab + ax_t_cg(Lb, Lk) : ph + 2 * (Lk + 1) * (lane - 1);
-        const int n = lane == 0 ? Lb : Lk;
+    if (tid == 31 || tid >= 62) {  // phases: gamma (thread 31), a and b of the ket rotation
+        const int w = tid == 31 ? 0 : tid - 61;
+        const double c0 = tab[w == 0 ? 2 : 4 + 2 * w], s0 = tab[w == 0 ? 3 : 5 + 2 * w];
+        double* o = w == 0 ? tab + ax_t_cg(Lb, Lk) : ph + 2 * (Lk + 1) * (w - 1);
+        const int n = w == 0 ? Lb : Lk;
         double c = 1.0, s = 0.0;
         for (int m = 0; m <= n; ++m) {
             o[2 * m] = c;
@@ -302,19 +310,21 @@ __global__ void __launch_bounds__(32) axial_wigner_kernel(const AxQuartet* __res
             c = cn;
         }
     }
-    double* tc = tab + ax_t_c(Lb, Lk);
-    wigner_y(Lb, tab[0], -tab[1], tc, tc + ax_co(Lb + 1), pw, lane, 32, sync);
-    __syncwarp();
-    wigner_y(Lk, tab[4], -tab[5], C, S, pw, lane, 32, sync);
-    __syncwarp();
+    if (warp == 0) {
+        double* tc = tab + ax_t_c(Lb, Lk);
+        wigner_y(Lb, tab[0], -tab[1], tc, tc + ax_co(Lb + 1), pw[0], lane, 32, sync);
+    } else {
+        wigner_y(Lk, tab[4], -tab[5], C, S, pw[1], lane, 32, sync);
+    }
+    __syncthreads();
     double* D = tab + ax_t_d(Lb, Lk);
     if (q.full) {
-        full_blocks(Lk, ph, ph + 2 * (Lk + 1), C, S, D, lane, 32);
+        full_blocks(Lk, ph, ph + 2 * (Lk + 1), C, S, D, tid, AXW_THREADS);
     } else {
         const int nc = ax_co(Lk + 1), ns = ax_so(Lk + 1), np = 4 * (Lk + 1);
-        for (int i = lane; i < np; i += 32) D[i] = ph[i];
-        for (int i = lane; i < nc; i += 32) D[np + i] = C[i];
-        for (int i = lane; i < ns; i += 32) D[np + nc + i] = S[i];
+        for (int i = tid; i < np; i += AXW_THREADS) D[i] = ph[i];
+        for (int i = tid; i < nc; i += AXW_THREADS) D[np + i] = C[i];
+        for (int i = tid; i < ns; i += AXW_THREADS) D[np + nc + i] = S[i];
     }
 }
 
@@ -823,8 +833,8 @@ cudaError_t launch_axial_pair(const AxPair* pairs, const WorkItem* items, int ni
 cudaError_t launch_axial_wigner(const AxQuartet* qd, const WorkItem* items, int nitems, int lmax, double* ws,
                                 cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
-    const size_t smem = sizeof(double) * (size_t)(ax_co(lmax + 1) + ax_so(lmax + 1) + 4 * AX_LP + 2 + 4 * AX_NL);
-    axial_wigner_kernel<<<nitems, 32, smem, st>>>(qd, items, lmax, ws);
+    const size_t smem = sizeof(double) * (size_t)(ax_co(lmax + 1) + ax_so(lmax + 1));
+    axial_wigner_kernel<<<nitems, AXW_THREADS, smem, st>>>(qd, items, lmax, ws);
     return cudaGetLastError();
 }
 

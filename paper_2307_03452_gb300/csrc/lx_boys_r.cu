@@ -128,16 +128,25 @@ __global__ void __launch_bounds__(32) boys_r_kernel(const DQuartet* __restrict__
     for (int r = lane; r < nr; r += 32) out[r] = R[r];
 }
 
+// One more power: (h, l) = x^n as an unevaluated sum -> x^(n+1), so that the chain rounds once, at
+// h + l.
+__device__ inline void power_step(double x, double& h, double& l) {
+    const double p = h * x;
+    l = (__double2hiint(p) & 0x7FF00000) == 0x7FF00000 ? 0.0 : fma(l, x, fma(h, x, -p));
+    h = p;
+}
+
 // Axial form (lx_axial.cu): 8 lanes per primitive quartet (item.q, item.a = kp kket + kq) write
 // the angles of its frames and the table B_kappa(L) Z^L.  Geometry and Boys values are computed
-// alike in the 8 lanes (one instruction serves 4 quartets), powers and table rows are spread
-// over them.
+// alike in the 8 lanes (one instruction serves 4 quartets), table rows are spread over them.  The
+// powers of 2 rho and Z are one chain of products with their errors carried (7 FP64 instructions
+// per degree for both; pow takes some 150 per power).
 constexpr int AXB_THREADS = 64, AXB_GROUPS = AXB_THREADS / 8;
 __global__ void __launch_bounds__(AXB_THREADS) axial_boys_kernel(const AxQuartet* __restrict__ qd,
                                                                  const AxPair* __restrict__ pairs,
                                                                  const WorkItem* __restrict__ items, int nitems,
                                                                  double* __restrict__ ws) {
-    __shared__ double F[AXB_GROUPS][LTOT + 1], row[AXB_GROUPS][2][LTOT + 2], zp_[AXB_GROUPS][LTOT + 1];
+    __shared__ double F[AXB_GROUPS][LTOT + 1], row[AXB_GROUPS][2][LTOT + 2], zp_[AXB_GROUPS][LTOT + 1], pw_[AXB_GROUPS][LTOT + 1];
     const int g = threadIdx.x >> 3, sub = threadIdx.x & 7;
     const int item = blockIdx.x * AXB_GROUPS + g;
     const bool live = item < nitems;
@@ -194,6 +203,15 @@ __global__ void __launch_bounds__(AXB_THREADS) axial_boys_kernel(const AxQuartet
         tab[6] = ca, tab[7] = sa, tab[8] = cb, tab[9] = sb;
         boys_eval(Lt, T, F[g]);
     }
+    double ph = 1.0, pl = 0.0, zh = 1.0, zl_ = 0.0;
+    for (int L = 0; L <= Lt; ++L) {
+        if ((L & 7) == sub) {
+            pw_[g][L] = ph + pl;
+            zp_[g][L] = zh + zl_;
+        }
+        power_step(2.0 * rho, ph, pl);
+        power_step(Z, zh, zl_);
+    }
     __syncwarp();
     // 0 Z^L is taken as 0 and the square of Z kept finite: at separations where F_L underflows
     // the powers of Z may overflow
@@ -203,8 +221,7 @@ __global__ void __launch_bounds__(AXB_THREADS) axial_boys_kernel(const AxQuartet
     double* cur = row[g][0];
     double* nxt = row[g][1];
     for (int L = sub; L <= Lt; L += 8) {
-        const double pw = (L & 1 ? -pref : pref) * pow(2.0 * rho, (double)L), zl = pow(Z, (double)L);
-        zp_[g][L] = zl;
+        const double pw = (L & 1 ? -pref : pref) * pw_[g][L], zl = zp_[g][L];
         const double b0 = pw * F[g][L];
         const double b = b0 != 0.0 ? b0 * zl : 0.0;
         if (live) bz[ax_bz(L) + (L >> 1)] = b;

@@ -361,8 +361,8 @@ struct ChunkPlan {
     std::vector<AxPair> ax_pairs;
     std::vector<AxQuartet> ax_quartets;
     std::vector<WorkItem> ax_ip, ax_it, ax_im, ax_irk, ax_irb;  // pairs, tables, main, rotations of ket and bra
-    int ax_counts[AX_NBIN] = {0, 0, 0, 0}, ax_lmax = 0, ax_lanes_k = 16, ax_lanes_b = 16;
-    size_t ax_smem[AX_NBIN] = {0, 0, 0, 0}, ax_rot_k = 0, ax_rot_b = 0;
+    int ax_counts[AX_NBIN] = {}, ax_lmax = 0, ax_lanes_k = 16, ax_lanes_b = 16;
+    size_t ax_smem[AX_NBIN] = {}, ax_rot_k = 0, ax_rot_b = 0;
     size_t off_axp = 0, off_axq = 0, off_aip = 0, off_ait = 0, off_aim = 0, off_airk = 0, off_airb = 0;
     size_t total = 0;         // bytes from the chunk base
     std::vector<char> blob;   // descriptor bytes [0, off_data)

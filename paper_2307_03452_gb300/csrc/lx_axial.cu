@@ -18,7 +18,7 @@
 // quartet of (ii|ii) in solid functions the bra rotation, T and the ket rotation take about
 // 1.4e6 FMAs where H_ab [p+q] takes 3.5e7, and the ket transform 7e5 where the second transform takes
 // 1.3e7; what remains is 1e6 FMAs per quartet to rotate the functions to the lab frame.  No
-// step leaves FP64.  2,048 (ii|ii) quartets, solid, K = 1: 194.4 -> 15.8 ms; 200 Cartesian ones 169.1 -> 31.9 ms;
+// step leaves FP64.  2,048 (ii|ii) quartets, solid, K = 1: 194.4 -> 14.4 ms; 200 Cartesian ones 169.1 -> 31.1 ms;
 // against 80-bit arithmetic the axial form's errors are at or below the matrix form's.
 //
 // Rows and columns are kept by half rows (AxHalf): the product of functions of orders m_a, m_b >= 0
@@ -344,9 +344,9 @@ __host__ __device__ inline int ax_count(int L) {  // (k, l) pairs, 2k + l <= L
 template <int NK>
 __device__ __forceinline__ void t_task(int lp, int Mp, int Lb, int lo, int M, const double* __restrict__ hs,
                                        const int* __restrict__ hpre, const int* __restrict__ tinfo,
-                                       const double* __restrict__ T, const double* __restrict__ dC,
-                                       const double* __restrict__ dS, double* __restrict__ sc_out,
+                                       const double* __restrict__ T, const double* __restrict__ tc, double* __restrict__ sc_out,
                                        double* __restrict__ ss_out) {
+    const double* ts = tc + ax_co(Lb + 1);
     double sc[NK], ss[NK];
 #pragma unroll
     for (int j = 0; j < NK; ++j) sc[j] = ss[j] = 0.0;
@@ -354,6 +354,8 @@ __device__ __forceinline__ void t_task(int lp, int Mp, int Lb, int lo, int M, co
         const int nk = ax_nk(Lb, l), info = tinfo[l * AX_NL + lp];
         const double* t = T + (info >> 8) + Mp * (info & 255);
         const double* h = hs + hpre[l] * AX_NR;
+        const double c = l >= M ? __ldg(tc + ax_co(l) + Mp * (l + 1) + M) : 0.0;
+        const double s = l >= M && M && Mp ? __ldg(ts + ax_so(l) + (Mp - 1) * l + M - 1) : 0.0;
         double I[NK];
 #pragma unroll
         for (int j = 0; j < NK; ++j) I[j] = 0.0;
@@ -362,8 +364,6 @@ __device__ __forceinline__ void t_task(int lp, int Mp, int Lb, int lo, int M, co
 #pragma unroll
             for (int j = 0; j < NK; ++j) I[j] = fma(hk, t[k + j], I[j]);
         }
-        const double c = l >= M ? dC[ax_co(l) + Mp * (l + 1) + M] : 0.0;
-        const double s = l >= M && M && Mp ? dS[ax_so(l) + (Mp - 1) * l + M - 1] : 0.0;
 #pragma unroll
         for (int j = 0; j < NK; ++j) {
             sc[j] = fma(c, I[j], sc[j]);
@@ -421,15 +421,15 @@ __device__ __forceinline__ void r_task(int l, int mm, int mtop, bool first, doub
 // quartets with K = 1..5; within 6 bohr 6.21 -> 6.14 ms.
 __device__ __forceinline__ void t_far(int lp, int Mp, int Lb, int lo, int M, const double* __restrict__ hs,
                                       const int* __restrict__ hpre, const int* __restrict__ tinfo,
-                                      const double* __restrict__ T, const double* __restrict__ dC,
-                                      const double* __restrict__ dS, double* __restrict__ sc_out,
+                                      const double* __restrict__ T, const double* __restrict__ tc, double* __restrict__ sc_out,
                                       double* __restrict__ ss_out) {
+    const double* ts = tc + ax_co(Lb + 1);
     double sc = 0.0, ss = 0.0;
     for (int l = Lb; l >= max(lo, Mp); --l) {
         const int info = tinfo[l * AX_NL + lp];
         const double I = hs[hpre[l] * AX_NR] * T[(info >> 8) + Mp * (info & 255)];
-        const double c = l >= M ? dC[ax_co(l) + Mp * (l + 1) + M] : 0.0;
-        const double s = l >= M && M && Mp ? dS[ax_so(l) + (Mp - 1) * l + M - 1] : 0.0;
+        const double c = l >= M ? __ldg(tc + ax_co(l) + Mp * (l + 1) + M) : 0.0;
+        const double s = l >= M && M && Mp ? __ldg(ts + ax_so(l) + (Mp - 1) * l + M - 1) : 0.0;
         sc = fma(c, I, sc);
         ss = fma(s, I, ss);
     }
@@ -462,7 +462,8 @@ __device__ __forceinline__ void r_far(int l, int mm, int mtop, int nk, bool firs
 // counters, the longest first.  Every stage is bound by the FP64 pipe: 87,300 warp FMAs per
 // (ii|ii) quartet, at the 20 cycles each that a plain FMA loop reaches 843 us of one SM; measured
 // 934 us (12.6 ms for 2,048 quartets).
-template <int THREADS, int MINB>
+// KM: the largest k range, Lk / 2 + 1, that the group's shared memory admits.
+template <int THREADS, int MINB, int KM>
 __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuartet* __restrict__ qd,
                                                                    const AxPair* __restrict__ pairs,
                                                                    const WorkItem* __restrict__ items,
@@ -511,10 +512,8 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
     double* SC = hs + nh * AX_NR;         // pyr(Lk) x 8: cosine part, then sine part
     double* SS = SC + nsc * AX_NR;
     double* X = SC + nx * AX_NR;          // pyr(Lk) x 16
-    double* dC = X + nx * 2 * AX_NR;      // bra blocks, then T; or the ket blocks
-    double* dS = dC + ax_co(Lb + 1);
-    double* T = dS + ax_so(Lb + 1);
-    double* D = dC;
+    double* T = X + nx * 2 * AX_NR;       // T and B Z^L, replaced by the ket blocks
+    double* D = T;
     const int t0 = c_ax.tent_off[pair_id], nT = c_ax.tent_off[pair_id + 1] - t0;
     double* BZ = T + nT;
     const int lo = hr[0].M;  // half rows are ordered by M
@@ -544,7 +543,6 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
             const double* h = ws + pb.h_off + (int64_t)kp * pb.nh;
             for (int i = tid; i < ax_bz(Lb + Lk + 1); i += THREADS) BZ[i] = tab[AX_T_BZ + i];
             const double* tc = tab + ax_t_c(Lb, Lk);
-            for (int i = tid; i < ax_co(Lb + 1) + ax_so(Lb + 1); i += THREADS) dC[i] = tc[i];
             for (int i = tid; i < nh * AX_NR; i += THREADS) {
                 const int r = i & (AX_NR - 1), e = i / AX_NR, e0 = hpre[hr[r].M];
                 hs[i] = r < it.b && e >= e0 ? h[hr[r].hoff + e - e0] : 0.0;
@@ -576,12 +574,12 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
                 double* so = SC + (scp[lp] + Mp * nk) * AX_NR + r8;
                 double* zo = SS + (ssp[lp] + (Mp - 1) * nk) * AX_NR + r8;
                 if (far) {
-                    t_far(lp, Mp, Lb, lo, Mr, hs + r8, hpre, tinfo, T, dC, dS, so, zo);
+                    t_far(lp, Mp, Lb, lo, Mr, hs + r8, hpre, tinfo, T, tc, so, zo);
                     continue;
                 }
 #define AX_T(N)                                                                                    \
     case N:                                                                                        \
-        t_task<N>(lp, Mp, Lb, lo, Mr, hs + r8, hpre, tinfo, T, dC, dS, so, zo);                    \
+        if constexpr (N <= KM) t_task<N>(lp, Mp, Lb, lo, Mr, hs + r8, hpre, tinfo, T, tc, so, zo);                    \
         break;
                 switch (nk) { AX_T(1) AX_T(2) AX_T(3) AX_T(4) AX_T(5) AX_T(6) AX_T(7) AX_T(8) }
 #undef AX_T
@@ -613,7 +611,7 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
                 }
 #define AX_R(N)                                                                                    \
     case N:                                                                                        \
-        r_task<N>(l, mm, mtop, first, cM, sM, D + ax_do(l), SC + scp[l] * AX_NR + r8,              \
+        if constexpr (N <= KM) r_task<N>(l, mm, mtop, first, cM, sM, D + ax_do(l), SC + scp[l] * AX_NR + r8,              \
                   SS + ssp[l] * AX_NR + r8, X + xp[l] * 2 * AX_NR + 2 * r8);                       \
         break;
                 switch (nk) { AX_R(1) AX_R(2) AX_R(3) AX_R(4) AX_R(5) AX_R(6) AX_R(7) AX_R(8) }
@@ -784,14 +782,19 @@ constexpr int AX_SMEM_MAX = 227 * 1024;
 size_t axial_main_smem(int Lb, int Lk) {
     const AxHost& H = axial_tables();
     const int id = Lb * AX_NL + Lk, nT = H.tent_off[id + 1] - H.tent_off[id];
-    const int tabs = std::max(ax_co(Lb + 1) + ax_so(Lb + 1) + nT + ax_bz(Lb + Lk + 1), ax_do(Lk + 1));
+    const int tabs = std::max(nT + ax_bz(Lb + Lk + 1), ax_do(Lk + 1));
     return sizeof(double) * (size_t)(ax_count(Lb) * AX_NR + 3 * pyr(Lk) * AX_NR + tabs);
 }
 
-// The groups by shared memory: 8, 4, 2 and 1 CTAs per SM.
+// The groups by shared memory: 1, 2, 3, 4 and 8 CTAs per SM of 512, 256, 256, 256 and 128 threads
+// (CTAs that share an SM fill one another's gaps at barriers and table loads; small classes, with
+// short stages, want the most warps).  (ii|ii) needs 113,896 bytes, two per SM with the bra blocks
+// left in global memory: its main kernel 9.65 -> 8.46 ms for 2,048 quartets against one CTA of 512
+// threads; (gg|gg) with 256 threads 4.41 ms for 8,192, with 128 5.34.
 int axial_bin(int Lb, int Lk) {
     const size_t s = axial_main_smem(Lb, Lk);
-    return s <= 24 * 1024 ? 3 : s <= 52 * 1024 ? 2 : s <= 108 * 1024 ? 1 : 0;
+    const int bin = s <= 25 * 1024 ? 4 : s <= 54 * 1024 ? 3 : s <= 73 * 1024 ? 2 : s <= 113900 ? 1 : 0;
+    return std::min(bin, 8 - (Lk / 2 + 1));  // group b's kernel takes k ranges up to 8 - b
 }
 
 cudaError_t init_axial(const AxHost& H) {
@@ -814,8 +817,9 @@ cudaError_t init_axial(const AxHost& H) {
     for (int l = 0; l <= LMAX; ++l)
         for (int s = 0; s < 2; ++s) d.shell[l][s] = H.shell[l][s];
     if ((e = cudaMemcpyToSymbol(c_ax, &d, sizeof(d))) != cudaSuccess) return e;
-    const void* kernels[] = {(const void*)axial_main_kernel<512, 1>, (const void*)axial_main_kernel<256, 2>,
-                             (const void*)axial_main_kernel<256, 4>, (const void*)axial_main_kernel<128, 8>,
+    const void* kernels[] = {(const void*)axial_main_kernel<512, 1, 8>, (const void*)axial_main_kernel<256, 2, 7>,
+                             (const void*)axial_main_kernel<256, 3, 6>, (const void*)axial_main_kernel<256, 4, 5>,
+                             (const void*)axial_main_kernel<128, 8, 4>,
                              (const void*)axial_rotate_kernel<0>, (const void*)axial_rotate_kernel<1>};
     for (const void* k : kernels)
         if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, AX_SMEM_MAX - 8192)) != cudaSuccess)
@@ -844,10 +848,11 @@ cudaError_t launch_axial_main(const AxQuartet* qd, const AxPair* pairs, const Wo
         const int n = counts[b];
         if (n <= 0) continue;
         switch (b) {
-            case 0: axial_main_kernel<512, 1><<<n, 512, smem[b], st>>>(qd, pairs, items, ws, out); break;
-            case 1: axial_main_kernel<256, 2><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, out); break;
-            case 2: axial_main_kernel<256, 4><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, out); break;
-            default: axial_main_kernel<128, 8><<<n, 128, smem[b], st>>>(qd, pairs, items, ws, out); break;
+            case 0: axial_main_kernel<512, 1, 8><<<n, 512, smem[b], st>>>(qd, pairs, items, ws, out); break;
+            case 1: axial_main_kernel<256, 2, 7><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, out); break;
+            case 2: axial_main_kernel<256, 3, 6><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, out); break;
+            case 3: axial_main_kernel<256, 4, 5><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, out); break;
+            default: axial_main_kernel<128, 8, 4><<<n, 128, smem[b], st>>>(qd, pairs, items, ws, out); break;
         }
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -144,7 +144,7 @@ cudaError_t launch_axial_boys(const AxQuartet* qd, const AxPair* pairs, const Wo
 cudaError_t launch_axial_wigner(const AxQuartet* qd, const WorkItem* items, int nitems, int lmax, double* ws,
                                 cudaStream_t st);
 // Size groups of the main kernel's launches.
-constexpr int AX_NBIN = 4;
+constexpr int AX_NBIN = 5;
 int axial_bin(int Lb, int Lk);
 cudaError_t launch_axial_main(const AxQuartet* qd, const AxPair* pairs, const WorkItem* items, const int* counts,
                               const size_t* smem, const double* ws, double* out, cudaStream_t st);

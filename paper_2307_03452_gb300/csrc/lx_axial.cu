@@ -18,7 +18,7 @@
 // quartet of (ii|ii) in solid functions the bra rotation, T and the ket rotation take about
 // 1.4e6 FMAs where H_ab [p+q] takes 3.5e7, and the ket transform 7e5 where the second transform takes
 // 1.3e7; what remains is 1e6 FMAs per quartet to rotate the functions to the lab frame.  No
-// step leaves FP64.  2,048 (ii|ii) quartets, solid, K = 1: 194.4 -> 14.4 ms; 200 Cartesian ones 169.1 -> 31.1 ms;
+// step leaves FP64.  2,048 (ii|ii) quartets, solid, K = 1: 194.4 -> 14.2 ms; 200 Cartesian ones 169.1 -> 24.8 ms;
 // against 80-bit arithmetic the axial form's errors are at or below the matrix form's.
 //
 // Rows and columns are kept by half rows (AxHalf): the product of functions of orders m_a, m_b >= 0
@@ -665,11 +665,12 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
 // frame to the lab (transposed Y, then z) and, for Cartesian output, expanded over monomials.
 // SIDE = 1: ket indices, `lanes` rows from item.a; SIDE = 0: bra indices, `lanes` columns from item.a.
 // Bound by the FP64 pipe (32,800 warp FMAs per (ii|ii) quartet for both sides, 317 us of one SM;
-// measured 331 us, 4.5 ms for 2,048 quartets); a tile of 16 keeps the accesses of a half warp in
-// 128 bytes and two or more CTAs on an SM.
-constexpr int AXR_THREADS = 256;
-template <int SIDE>
-__global__ void __launch_bounds__(AXR_THREADS) axial_rotate_kernel(const AxQuartet* __restrict__ qd,
+// measured 315 us, 4.24 ms for 2,048 quartets; 200 Cartesian (ii|ii) 14.0 ms).  Neighbouring tasks of
+// a warp take the same function of neighbouring lines, so that loop lengths do not differ within a
+// warp (4.47 and 20.2 ms with neighbouring functions of one line); a tile of 16 lanes keeps the
+// accesses of a half warp in 128 bytes and four CTAs on an SM (32 lanes: 5.64 ms).
+template <int SIDE, int THREADS>
+__global__ void __launch_bounds__(THREADS) axial_rotate_kernel(const AxQuartet* __restrict__ qd,
                                                                    const AxPair* __restrict__ pairs,
                                                                    const WorkItem* __restrict__ items, int lanes,
                                                                    const double* __restrict__ ws,
@@ -679,7 +680,7 @@ __global__ void __launch_bounds__(AXR_THREADS) axial_rotate_kernel(const AxQuart
     const WorkItem it = items[blockIdx.x];
     const AxQuartet q = qd[it.q];
     const AxPair pr = pairs[SIDE ? q.pk : q.pb];
-    const int tid = threadIdx.x, ld = lanes + 1, lane = tid % lanes, t0 = tid / lanes, nt = AXR_THREADS / lanes;
+    const int tid = threadIdx.x, ld = lanes + 1, lane = tid % lanes, t0 = tid / lanes, nt = THREADS / lanes;
     const AxShell s1 = c_ax.shell[pr.la][solid], s2 = c_ax.shell[pr.lb][solid];
     const AxFn *f1 = c_ax.fns + s1.fn0, *f2 = c_ax.fns + s2.fn0;
     const int n1 = s1.ntot, n2 = s2.ntot, n = n1 * n2, lm = max(pr.la, pr.lb);
@@ -687,10 +688,10 @@ __global__ void __launch_bounds__(AXR_THREADS) axial_rotate_kernel(const AxQuart
     double* a = sm;
     double* b = sm + n * ld;
     double* O = out + q.out_off;
-    for (int i = tid; i < ax_rot_size(lm); i += AXR_THREADS) rot[i] = ws[pr.rot_off + i];
+    for (int i = tid; i < ax_rot_size(lm); i += THREADS) rot[i] = ws[pr.rot_off + i];
     const double *cs = rot + AX_ROT_CS, *C = rot + AX_ROT_C, *S = C + ax_co(lm + 1);
     if (SIDE) {
-        for (int i = tid; i < live * n; i += AXR_THREADS) {
+        for (int i = tid; i < live * n; i += THREADS) {
             const int r = i / n, c = i - r * n;
             double v = O[(int64_t)(it.a + r) * n + c];
             for (int p = 0; p + 1 < q.nsplit; ++p) v += ws[q.part_off + ((int64_t)p * q.nab + it.a + r) * n + c];
@@ -721,7 +722,7 @@ __global__ void __launch_bounds__(AXR_THREADS) axial_rotate_kernel(const AxQuart
     auto turn = [&](const double* src, double* dst, const AxFn* fn, int nfn, int no, int so, int sf) {
         if (lane < live)
             for (int i = t0; i < no * nfn; i += nt) {
-                const int o = i / nfn, f = i - o * nfn;
+                const int f = i / no, o = i - f * no;
                 const AxFn& F = fn[f];
                 const int lam = F.lam, m = F.m, mid = F.plus - m;
                 const double* v = src + (o * so + mid * sf) * ld + lane;
@@ -744,7 +745,7 @@ __global__ void __launch_bounds__(AXR_THREADS) axial_rotate_kernel(const AxQuart
     auto expand = [&](const double* src, double* dst, const AxShell& s, int no, int so, int sf) {
         if (lane < live)
             for (int i = t0; i < no * s.ntot; i += nt) {
-                const int o = i / s.ntot, c = i - o * s.ntot;
+                const int c = i / no, o = i - c * no;
                 const int b0 = __ldg(c_ax.wc_row + s.wc0 + c), b1 = __ldg(c_ax.wc_row + s.wc0 + c + 1);
                 double t = 0.0;
                 for (int e = b0; e < b1; ++e)
@@ -760,7 +761,7 @@ __global__ void __launch_bounds__(AXR_THREADS) axial_rotate_kernel(const AxQuart
         expand(b, a, s1, n2, 1, n2);
     }
     if (SIDE) {
-        for (int i = tid; i < live * n; i += AXR_THREADS) {
+        for (int i = tid; i < live * n; i += THREADS) {
             const int r = i / n, c = i - r * n;
             O[(int64_t)(it.a + r) * n + c] = a[c * ld + r];
         }
@@ -824,7 +825,8 @@ cudaError_t init_axial(const AxHost& H) {
     const void* kernels[] = {(const void*)axial_main_kernel<512, 1, 8>, (const void*)axial_main_kernel<256, 2, 7>,
                              (const void*)axial_main_kernel<256, 3, 6>, (const void*)axial_main_kernel<256, 4, 5>,
                              (const void*)axial_main_kernel<128, 8, 4>,
-                             (const void*)axial_rotate_kernel<0>, (const void*)axial_rotate_kernel<1>};
+                             (const void*)axial_rotate_kernel<0, 256>, (const void*)axial_rotate_kernel<1, 256>,
+                             (const void*)axial_rotate_kernel<0, 1024>, (const void*)axial_rotate_kernel<1, 1024>};
     for (const void* k : kernels)
         if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, AX_SMEM_MAX - 8192)) != cudaSuccess)
             return e;
@@ -868,10 +870,15 @@ cudaError_t launch_axial_main(const AxQuartet* qd, const AxPair* pairs, const Wo
 cudaError_t launch_axial_rotate(int side, const AxQuartet* qd, const AxPair* pairs, const WorkItem* items, int nitems,
                                 int lanes, size_t smem, const double* ws, double* out, bool solid, cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
-    if (side)
-        axial_rotate_kernel<1><<<nitems, AXR_THREADS, smem, st>>>(qd, pairs, items, lanes, ws, out, solid ? 1 : 0);
-    else
-        axial_rotate_kernel<0><<<nitems, AXR_THREADS, smem, st>>>(qd, pairs, items, lanes, ws, out, solid ? 1 : 0);
+    // at least 32 warps per SM: 256 threads where four CTAs fit, 1,024 otherwise
+    const int s = solid ? 1 : 0;
+    if (smem <= 54 * 1024) {
+        if (side) axial_rotate_kernel<1, 256><<<nitems, 256, smem, st>>>(qd, pairs, items, lanes, ws, out, s);
+        else axial_rotate_kernel<0, 256><<<nitems, 256, smem, st>>>(qd, pairs, items, lanes, ws, out, s);
+    } else {
+        if (side) axial_rotate_kernel<1, 1024><<<nitems, 1024, smem, st>>>(qd, pairs, items, lanes, ws, out, s);
+        else axial_rotate_kernel<0, 1024><<<nitems, 1024, smem, st>>>(qd, pairs, items, lanes, ws, out, s);
+    }
     return cudaGetLastError();
 }
 

@@ -212,6 +212,7 @@ size_t quartet_bytes(const lx_shell* sh, const lx_quartet& q, int flags) {
     const int L = a.l + b.l + c.l + d.l, np = pyr(a.l + b.l), nq = pyr(c.l + d.l);
     const int64_t kbra = (int64_t)a.nprim * b.nprim, kket = (int64_t)c.nprim * d.nprim;
     const int64_t nab = (int64_t)nfun(a.l, solid) * nfun(b.l, solid), ncd = (int64_t)nfun(c.l, solid) * nfun(d.l, solid);
+    constexpr int64_t TB = 32;  // B row tile the bound on the split GEMMs' work items is stated for
     const int64_t n1 = kket * nq;
     int64_t items = kbra * kket;
     // + 256 bytes per data block: each block starts on a 256-byte boundary
@@ -228,8 +229,8 @@ size_t quartet_bytes(const lx_shell* sh, const lx_quartet& q, int flags) {
         const int k1 = (int)(kbra * np), k2 = (int)n1;
         const int ra1 = split_rowpad(k2, SPLIT_TA), ra2 = split_rowpad((int)nab, SPLIT_TA);
         items += (ra1 + ra2) / 8;
-        items += (ra1 / SPLIT_TA) * ((nab + SPLIT_TB - 1) / SPLIT_TB);
-        items += (ra2 / SPLIT_TA) * ((ncd + SPLIT_TB - 1) / SPLIT_TB);
+        items += (ra1 / SPLIT_TA) * ((nab + TB - 1) / TB);
+        items += (ra2 / SPLIT_TA) * ((ncd + TB - 1) / TB);
         bytes += sizeof(SplitQuartet) + 2 * sizeof(SplitGemmDesc) + sizeof(SplitRowsDesc);
         bytes += (size_t)split_dig_bytes(k2, k1, SPLIT_TA) + (size_t)split_dig_bytes((int)nab, k2, SPLIT_TA);
         bytes += 4 * ((size_t)ra1 + (size_t)ra2 * split_nseg(split_nkb(k2))) + 4 * 256;
@@ -245,9 +246,9 @@ size_t pair_bytes(const lx_shell* sh, int sa, int sb, int flags) {
     const int64_t k = kab * pyr(a.l + b.l);
     size_t bytes = sizeof(DPair) + kab * sizeof(WorkItem) + 8 * (size_t)(kab * 4 + rows * k) + 512;
     if (split) {
-        // H's digit planes (rows padded to at most SPLIT_TB), row exponents, column scales
-        const int rp = split_rowpad((int)rows, SPLIT_TB);
-        bytes += sizeof(SplitRowsDesc) + (size_t)split_dig_bytes((int)rows, (int)k, SPLIT_TB);
+        // H's digit planes (a bound: rows padded to 32), row exponents, column scales
+        const int rp = split_rowpad((int)rows, 32);
+        bytes += sizeof(SplitRowsDesc) + (size_t)split_dig_bytes((int)rows, (int)k, 32);
         bytes += 4 * (size_t)(rp + k) + 3 * 256;
         bytes += sizeof(WorkItem) * (size_t)(rp / 8);
     }
@@ -356,6 +357,7 @@ struct ChunkPlan {
     std::vector<WorkItem> items_h, items_br, items_g1, items_g2;
     int br_lmax = 0;  // largest L of the chunk's quartets
     int digits = 6;   // split path: BF16 digits kept per value (one count per batch)
+    bool wide1 = false, wide2 = false;  // some B row tile of GEMM1 (GEMM2) has more than 32 rows
     int fold_lcap = 0, fold_qcap = 0, fold_wcap = 0, fold_gcap = 0;  // solid fold: largest l, Q, W and G of the chunk's pairs
     int jkd_qc = 0;          // J/K on the FP64 path: chunk width of jk_direct_kernel
     size_t jkd_smem = 0;     // and its shared memory
@@ -386,6 +388,7 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
     const bool solid = flags & LX_SOLID, split = flags & LX_PATH_SPLIT, jk = flags & JK_DIGEST;
     const int nd_flag = (flags & LX_SPLIT_DIGITS_MASK) >> 4, nd = nd_flag ? nd_flag : SPLIT_NSLICE;
     P.digits = nd;
+    P.wide1 = P.wide2 = false;
     P.pairs.clear();
     P.quartets.clear();
     P.items_h.clear();
@@ -618,7 +621,8 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
             const DPair& pr = P.pairs[p];
             const int k = pr.Kab * pr.np, tb = split_tb(pr.nrow);
             // columns scaled into (-1, 1): one pass, e = 0 per row
-            P.srd.push_back(SplitRowsDesc{0, 0, 0, 0, k, pr.nrow, k, tb, split_nkb(k), -1, 1, 0, nd, 0});
+            P.srd.push_back(
+                SplitRowsDesc{0, 0, 0, 0, k, pr.nrow, k, tb, split_nkb(k), -1, 1, 0, nd, split_trim(pr.nrow)});
             // digit kernels: one item per 8 consecutive rows, up to nrow rounded to 8 (the GEMMs
             // drop the output columns of B rows past nrow, so the rest of the last row tile is
             // never written)
@@ -635,8 +639,11 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
             q.gidx_off = gidx_offset(sh[pb.sa].l + sh[pb.sb].l, sh[pk.sa].l + sh[pk.sb].l);
             P.sq.push_back(q);
             const int tb1 = split_tb(d.nab), tb2 = split_tb(d.ncd);
+            P.wide1 = P.wide1 || tb1 > 32;
+            P.wide2 = P.wide2 || tb2 > 32;
             // A2: X, one exponent per row and segment (the rows up to nab rounded to 8 are used)
-            P.srd.push_back(SplitRowsDesc{0, 0, 0, 0, k2, d.nab, k2, SPLIT_TA, q.nkb2, +1, 2, split_nseg(q.nkb2), nd, 0});
+            P.srd.push_back(SplitRowsDesc{0, 0, 0, 0, k2, d.nab, k2, SPLIT_TA, q.nkb2, +1, 2, split_nseg(q.nkb2), nd,
+                                          SPLIT_NO_TRIM});
             for (int row = 0; row < split_rowpad(k2, 8); row += 8) P.items_sr.push_back({i, row, 0, 0});
             // X's digit planes only after GEMM1
             for (int row = 0; row < split_rowpad(d.nab, 8); row += 8) P.items_sD.push_back({npair + i, row, 0, 0});
@@ -713,11 +720,11 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
         const int npair = (int)P.pairs.size();
         for (int p = 0; p < npair; ++p) {
             const DPair& pr = P.pairs[p];
-            const int k = pr.Kab * pr.np, tb = split_tb(pr.nrow);
+            const int k = pr.Kab * pr.np;
             SplitRowsDesc& r = P.srd[p];
             r.src_off = pr.h_off;
-            r.dig_off = take_bytes(split_dig_bytes(pr.nrow, k, tb));
-            r.exp_off = take_bytes(4 * (int64_t)split_rowpad(pr.nrow, tb));
+            r.dig_off = take_bytes(split_dig_bytes_b(pr.nrow, k));
+            r.exp_off = take_bytes(4 * (int64_t)split_trim(pr.nrow));
             r.shift_off = take_bytes(4 * (int64_t)k);
             P.pairs[p].cs_off = r.shift_off;  // written by the pair's H kernel
         }
@@ -970,7 +977,7 @@ int enqueue_batch(const PlannedBatch& B, const char* head_src, const std::vector
             if ((e = tm.end(LX_STAGE_SPLIT, 1)) != cudaSuccess) return cuda_fail(e);
             if ((e = tm.begin()) != cudaSuccess) return cuda_fail(e);
             if ((e = launch_split_gemm(d_sg1, items(P.off_isg1), (int)P.items_sg1.size(), wsb, ws, status, st,
-                                       false, P.digits)) != cudaSuccess)
+                                       false, P.digits, P.wide1)) != cudaSuccess)
                 return cuda_fail(e);
             if ((e = tm.end(LX_STAGE_GEMM1, 1)) != cudaSuccess) return cuda_fail(e);
             // the other operand of GEMM2: digit planes of [ab|q], one exponent per row and segment
@@ -980,7 +987,7 @@ int enqueue_batch(const PlannedBatch& B, const char* head_src, const std::vector
             if ((e = tm.end(LX_STAGE_SPLIT, 1)) != cudaSuccess) return cuda_fail(e);
             if ((e = tm.begin()) != cudaSuccess) return cuda_fail(e);
             if ((e = launch_split_gemm(d_sg2, items(P.off_isg2), (int)P.items_sg2.size(), wsb, out, status, st,
-                                       true, P.digits)) != cudaSuccess)
+                                       true, P.digits, P.wide2)) != cudaSuccess)
                 return cuda_fail(e);
             if ((e = tm.end(LX_STAGE_GEMM2, 1)) != cudaSuccess) return cuda_fail(e);
         } else {
@@ -1908,10 +1915,10 @@ int lx_split_gemm(int32_t M, int32_t N, int32_t K, const double* A, int32_t lda,
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int nkb = split_nkb(K);
     const int tb = split_tb(N);
-    const int ra = split_rowpad(M, SPLIT_TA), rb = split_rowpad(N, tb);
+    const int ra = split_rowpad(M, SPLIT_TA), rb = split_trim(N);
     std::vector<SplitRowsDesc> rd(2);
-    rd[0] = SplitRowsDesc{0, 0, 0, -1, lda, M, K, SPLIT_TA, nkb, 0, 0, 0, digits, 0};
-    rd[1] = SplitRowsDesc{0, 0, 0, -1, ldb, N, K, tb, nkb, 0, 0, 0, digits, 0};
+    rd[0] = SplitRowsDesc{0, 0, 0, -1, lda, M, K, SPLIT_TA, nkb, 0, 0, 0, digits, SPLIT_NO_TRIM};
+    rd[1] = SplitRowsDesc{0, 0, 0, -1, ldb, N, K, tb, nkb, 0, 0, 0, digits, rb};
     std::vector<WorkItem> ia, ib, ig;
     for (int r = 0; r < ra; r += 8) ia.push_back({0, r, 0, 0});
     for (int r = 0; r < rb; r += 8) ib.push_back({1, r, 0, 0});
@@ -1929,7 +1936,7 @@ int lx_split_gemm(int32_t M, int32_t N, int32_t K, const double* A, int32_t lda,
     const size_t blob_bytes = o;
     rd[0].dig_off = (int64_t)region((size_t)split_dig_bytes(M, K, SPLIT_TA));
     rd[0].exp_off = (int64_t)region(4 * (size_t)ra);
-    rd[1].dig_off = (int64_t)region((size_t)split_dig_bytes(N, K, tb));
+    rd[1].dig_off = (int64_t)region((size_t)split_dig_bytes_b(N, K));
     rd[1].exp_off = (int64_t)region(4 * (size_t)rb);
     SplitGemmDesc g{};
     g.a_dig = rd[0].dig_off;
@@ -1963,7 +1970,7 @@ int lx_split_gemm(int32_t M, int32_t N, int32_t K, const double* A, int32_t lda,
         return cuda_fail(e);
     if ((e = launch_split_gemm(reinterpret_cast<const SplitGemmDesc*>(scratch + o_g),
                                reinterpret_cast<const WorkItem*>(scratch + o_ig), (int)ig.size(), scratch, C, status,
-                               st, false, digits)) != cudaSuccess)
+                               st, false, digits, tb > 32)) != cudaSuccess)
         return cuda_fail(e);
     if ((e = cudaFreeAsync(scratch, st)) != cudaSuccess) return cuda_fail(e);
     return LX_OK;

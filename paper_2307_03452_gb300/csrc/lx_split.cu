@@ -17,12 +17,13 @@
 //   split_operands_kernel  rows q of the [p|q] operand gathered from [r]^(0), and the H
 //                      rows, -> digit planes + row exponents (GEMM1 operands, H_ket)
 //   split_rows_kernel  FP64 row-major matrix rows ([ab|q]) -> digit planes + row exponents
-//   split_gemm_kernel  D = A B^T on tcgen05 (M tile 128, N tile <= 32, K blocks of 32),
+//   split_gemm_kernel  D = A B^T on tcgen05 (M tile 128, N tile <= 40, K blocks of 32),
 //                      persistent, operand blocks streamed by bulk TMA copies into a
 //                      3-stage mbarrier ring, one thread issuing the MMAs, two TMEM
 //                      accumulator sets drained by eight warps.
 #include <cstdint>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "lx_internal.cuh"
@@ -136,7 +137,7 @@ __device__ inline void umma_commit(uint64_t* bar) {
                  : "memory");
 }
 
-__device__ inline void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+__device__ inline void tmem_ld(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
@@ -144,9 +145,15 @@ __device__ inline void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         : "r"(taddr)
         : "memory");
 }
-__device__ inline void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+__device__ inline void tmem_ld(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+}
+__device__ inline void tmem_ld(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(taddr)
                  : "memory");
 }
@@ -213,8 +220,8 @@ __device__ inline void digits_of(long long q, uint32_t (&f)[SPLIT_NSLICE]) {
 
 // Digits of 8 consecutive values (k0 .. k0+7, k0 a multiple of 8) of one row, written as one
 // 16-byte store per slice (one row of a core matrix), for the first nd slices.
-__device__ inline int64_t dig_index(int row, int k, int s, int T, int nkb);
-__device__ inline void store_digit_group(__nv_bfloat16* dig, int row, int k0, int T, int nkb,
+__device__ inline int64_t dig_index(int row, int k, int s, int T, int nkb, int trim);
+__device__ inline void store_digit_group(__nv_bfloat16* dig, int row, int k0, int T, int nkb, int trim,
                                          const long long (&q)[8], int nd) {
     // w[s][i]: BF16 pair of slice s, element 2i in the low half and 2i + 1 in the high half
     uint32_t w[SPLIT_NSLICE][4];
@@ -229,17 +236,18 @@ __device__ inline void store_digit_group(__nv_bfloat16* dig, int row, int k0, in
 #pragma unroll
     for (int s = 0; s < SPLIT_NSLICE; ++s)  // slices past nd are never read
         if (s < nd)
-            *reinterpret_cast<uint4*>(dig + dig_index(row, k0, s, T, nkb)) =
+            *reinterpret_cast<uint4*>(dig + dig_index(row, k0, s, T, nkb, trim)) =
                 make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
 }
 
 // Offset (in BF16 elements) of element (row, k) of slice s inside an operand stored as
-// row tiles of T rows and K blocks of SPLIT_KB: block (rt, kb) holds NSLICE slice-blocks of
-// T x KB elements, each in core matrices (8 rows x 8 elements) ordered (row/8, k/8).
-__device__ inline int64_t dig_index(int row, int k, int s, int T, int nkb) {
+// row tiles of T rows (the last one trimmed) and K blocks of SPLIT_KB: block (rt, kb) holds NSLICE
+// slice-blocks of T x KB elements, each in core matrices (8 rows x 8 elements) ordered (row/8, k/8).
+__device__ inline int64_t dig_index(int row, int k, int s, int T, int nkb, int trim) {
     const int rt = row / T, r = row - rt * T, kb = k / SPLIT_KB, kk = k - kb * SPLIT_KB;
-    const int64_t block = ((int64_t)rt * nkb + kb) * SPLIT_NSLICE + s;
-    return block * (T * SPLIT_KB) + ((r >> 3) * (SPLIT_KB / 8) + (kk >> 3)) * 64 + (r & 7) * 8 + (kk & 7);
+    const int64_t tile = (int64_t)rt * nkb * SPLIT_NSLICE * (T * SPLIT_KB);
+    return tile + (int64_t)(kb * SPLIT_NSLICE + s) * (min(T, trim - rt * T) * SPLIT_KB) +
+           ((r >> 3) * (SPLIT_KB / 8) + (kk >> 3)) * 64 + (r & 7) * 8 + (kk & 7);
 }
 
 // split_rows_kernel gives one warp 8 consecutive rows r0 .. r0+7 (r0 a multiple of 8), taken
@@ -260,7 +268,7 @@ __device__ inline int row_max16(int mx) {
 // they are scaled by; zeros outside the matrix): digit planes of row tile T with nkb K blocks
 // and one int exponent per row (the modes of SplitRowsDesc::fixed).
 template <bool SEGMENTS, typename Value>
-__device__ __forceinline__ void split_8rows(int r0, int nkb, int T, int fixed, int nseg, int nd,
+__device__ __forceinline__ void split_8rows(int r0, int nkb, int T, int trim, int fixed, int nseg, int nd,
                                             __nv_bfloat16* __restrict__ dig, int* __restrict__ exps, Value value) {
     const int lane = threadIdx.x & 31, c8 = 8 * (lane & 15);
     static_assert(SPLIT_SEG_KB * SPLIT_KB == 128, "one pass of a row pair covers one segment");
@@ -284,7 +292,7 @@ __device__ __forceinline__ void split_8rows(int r0, int nkb, int T, int fixed, i
                     long long q[8];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) q[i] = mx > 0 ? fixed_of(v[i], sh[i], e) : 0ll;
-                    store_digit_group(dig, row, k0, T, nkb, q, nd);
+                    store_digit_group(dig, row, k0, T, nkb, trim, q, nd);
                 }
                 if ((lane & 15) == 0) exps[(int64_t)row * nseg + sg] = e;
             }
@@ -309,7 +317,7 @@ __device__ __forceinline__ void split_8rows(int r0, int nkb, int T, int fixed, i
             long long q[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) q[i] = mx > 0 ? fixed_of(v[i], sh[i], e) : 0ll;
-            store_digit_group(dig, row, k0, T, nkb, q, nd);
+            store_digit_group(dig, row, k0, T, nkb, trim, q, nd);
         }
         if ((lane & 15) == 0) exps[row] = e;
     }
@@ -323,7 +331,7 @@ __device__ __forceinline__ void split_rows_item(const SplitRowsDesc* __restrict_
     const SplitRowsDesc d = descs[it.q];
     const double* src = src_base + d.src_off;
     const int* shift = d.shift_off >= 0 ? reinterpret_cast<const int*>(ws + d.shift_off) : nullptr;
-    split_8rows<SEGMENTS>(it.a, d.nkb, d.T, d.fixed, d.nseg, d.nd, reinterpret_cast<__nv_bfloat16*>(ws + d.dig_off),
+    split_8rows<SEGMENTS>(it.a, d.nkb, d.T, d.trim, d.fixed, d.nseg, d.nd, reinterpret_cast<__nv_bfloat16*>(ws + d.dig_off),
                 reinterpret_cast<int*>(ws + d.exp_off), [&](int row, int k0, double (&v)[8], int (&sh)[8]) {
                     const bool live = row < d.rows;
                     const double* sr = src + (int64_t)row * d.ld;
@@ -423,7 +431,7 @@ __device__ __forceinline__ void split_r_item(const DQuartet* __restrict__ qd, co
         long long qv[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) qv[i] = mx > 0 ? fixed_of(v[i], sh[i], e) : 0ll;
-        store_digit_group(dig, row, SPLIT_KB * kb + c8, SPLIT_TA, s.nkb1, qv, s.nd);
+        store_digit_group(dig, row, SPLIT_KB * kb + c8, SPLIT_TA, s.nkb1, SPLIT_NO_TRIM, qv, s.nd);
     }
     if ((lane & 3) == 0) reinterpret_cast<int*>(ws + s.a1_exp)[row] = e;
 }
@@ -431,7 +439,7 @@ __device__ __forceinline__ void split_r_item(const DQuartet* __restrict__ qd, co
 // The operands of GEMM1 and the H operand of GEMM2 in one launch: split_r items ([p|q]^T rows,
 // issue-bound gathers) and split_rows items (H rows, load-latency bound) in alternating blocks,
 // so that the two kinds share the SMs.  8 warps (items) per block.
-__global__ void __launch_bounds__(256) split_operands_kernel(const DQuartet* __restrict__ qd,
+__global__ void __launch_bounds__(256, 4) split_operands_kernel(const DQuartet* __restrict__ qd,
                                                              const SplitQuartet* __restrict__ sq,
                                                              const WorkItem* __restrict__ items_r, int n_r,
                                                              const SplitRowsDesc* __restrict__ descs,
@@ -463,16 +471,21 @@ constexpr int A_BLOCK = SPLIT_NSLICE * SPLIT_TA * SPLIT_KB * 2;  // bytes of one
 constexpr int B_BLOCK_MAX = SPLIT_NSLICE * SPLIT_TB * SPLIT_KB * 2;
 constexpr int A_SLICE = SPLIT_TA * SPLIT_KB * 2;
 constexpr int STAGE_BYTES = A_BLOCK + B_BLOCK_MAX;
-constexpr int BUF_COLS = SPLIT_NSLICE * SPLIT_TB;  // TMEM columns of one accumulator set
+// TMEM columns of one accumulator set: 6 diagonals of a tile's columns, and up to 8 more that the
+// N of an MMA, a multiple of 16, runs past them (B rows of the next slice; never read)
+__host__ __device__ constexpr int buf_cols(int dc) { return dc > 16 ? 256 : 192; }
 constexpr uint32_t TMEM_COLS = 512;
-static_assert(NBUF * BUF_COLS <= (int)TMEM_COLS, "accumulator sets exceed TMEM");
+static_assert(SPLIT_NSLICE * SPLIT_TB + 8 <= buf_cols(20) && SPLIT_NSLICE * 32 <= buf_cols(16),
+              "an accumulator set holds the diagonals");
+static_assert(NBUF * buf_cols(20) <= (int)TMEM_COLS, "accumulator sets exceed TMEM");
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
 // warp 0 TMA, warp 1 MMA issue + TMEM, warps 2..9 drain / epilogue: two warps per TMEM lane
-// quarter, each owning 16 of the tile's (at most 32) columns
+// quarter, each owning half of the tile's (at most 40) columns
+template <int N>
+using Int = std::integral_constant<int, N>;
 constexpr int DRAIN_WARPS = 8;
-constexpr int DCOLS = 16;  // columns per drain warp
 constexpr int GEMM_THREADS = 32 * (2 + DRAIN_WARPS);
-static_assert(SPLIT_TB == DCOLS * (DRAIN_WARPS / 4), "the drain warps cover the widest column tile");
+static_assert(SPLIT_TB == 20 * (DRAIN_WARPS / 4), "the drain warps cover the widest column tile");
 
 __device__ inline void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -501,12 +514,18 @@ __device__ inline long long shr_round(long long x, int s) {
 // The MMAs of one A slice s and one K step are issued against the B slices 0..nd-1-s at once:
 // slice t lies tb rows after slice t-1 in shared memory and diagonal s + t lies tb TMEM
 // columns after s + t - 1, so A_s [B_0; B_1; ...] lands every product on its diagonal in one
-// MMA of N = (nd - s) tb <= 192.  With nd < NSLICE digits only the first nd slices of each
+// MMA of N = (nd - s) tb <= 240, rounded to a multiple of 16.  With nd < NSLICE digits only the first nd slices of each
 // operand block are loaded, nd MMAs are issued per K step and nd diagonals drained.
-template <bool SEGS, int ND>
+//
+// DC: columns of a drain warp, 20 where a launch holds tiles of 40 columns, else 16 (fewer sums
+// to shift and keep; the drains' instructions compete with the MMA issue).  Tiles of 40 make 5
+// tiles of (ii|ii)'s 169 columns instead of 6, with the last one trimmed to 16: GEMM1 7.43 -> 6.58
+// and GEMM2 4.36 -> 3.75 ms for 4,096 quartets.
+template <bool SEGS, int ND, int DC>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     split_gemm_kernel(const SplitGemmDesc* __restrict__ probs, const WorkItem* __restrict__ items, int nitems,
                       const char* __restrict__ ws, double* __restrict__ cbase, unsigned* status) {
+    constexpr int BUF_COLS = buf_cols(DC);
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte aligned operand stages
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -545,9 +564,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             for (int w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
                 const WorkItem it = items[w];
                 const SplitGemmDesc P = probs[it.q];
-                const int b_block = SPLIT_NSLICE * P.tb * SPLIT_KB * 2;
+                const int tb = min(P.tb, split_trim(P.N) - it.b * P.tb);  // rows of this B tile
+                const int b_block = SPLIT_NSLICE * tb * SPLIT_KB * 2;
                 const char* a_src = ws + P.a_dig + (int64_t)it.a * P.nkb * A_BLOCK;
-                const char* b_src = ws + P.b_dig + (int64_t)it.b * P.nkb * b_block;
+                const char* b_src = ws + P.b_dig + (int64_t)it.b * P.nkb * (SPLIT_NSLICE * P.tb * SPLIT_KB * 2);
                 // rows of this A tile that exist (up to M rounded up to 8): a partial last tile
                 // is copied slice by slice, its first vr rows only; the rows past them hold
                 // whatever the stage held before and only reach output rows >= M, which the
@@ -555,7 +575,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 const int vr = min(SPLIT_TA, ((P.M + 7) & ~7) - it.a * SPLIT_TA);
                 // the first nd digit slices of each block (slices are the outer index of a block)
                 constexpr int nd = ND;  // P.nd equals ND (the launch is chosen by it)
-                const int a_bytes = nd * vr * SPLIT_KB * 2, b_bytes = nd * P.tb * SPLIT_KB * 2;
+                const int a_bytes = nd * vr * SPLIT_KB * 2, b_bytes = nd * tb * SPLIT_KB * 2;
                 for (int kb = 0; kb < P.nkb; ++kb, ++g) {
                     const int st = g % STAGES, use = g / STAGES;
                     if ((use > 0 && !mbar_wait(&empty_bar[st], (use - 1) & 1, status)) || *(volatile int*)&abort_sh) {
@@ -594,11 +614,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             for (int w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
                 const WorkItem it = items[w];
                 const SplitGemmDesc P = probs[it.q];
-                const int tb = P.tb, nkb = P.nkb;
-                constexpr int nd = ND;
+                const int tb = min(P.tb, split_trim(P.N) - it.b * P.tb), nkb = P.nkb;
                 uint32_t idesc[ND];
 #pragma unroll
-                for (int s = 0; s < ND; ++s) idesc[s] = idesc_bf16(SPLIT_TA, (ND - s) * tb);
+                for (int s = 0; s < ND; ++s) idesc[s] = idesc_bf16(SPLIT_TA, ((ND - s) * tb + 15) & ~15);
                 for (int kb0 = 0; kb0 < nkb && ok; kb0 += SPLIT_SEG_KB, ++sgc) {
                     const int buf = sgc & 1, ub = sgc >> 1;
                     if (ub > 0) {
@@ -642,19 +661,21 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             if (!mbar_wait(&final_bar, 0, status)) abort_sh = 1;
         }
     } else {
-        // drain / epilogue: warp w reads TMEM lanes (rows) 32 (w % 4) .. 32 (w % 4) + 31 and the
-        // DCOLS columns c0 .. c0 + DCOLS - 1 of each diagonal
-        const int quarter = warp & 3, c0 = DCOLS * ((warp - 2) >> 2);
-        const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + c0;
+        // drain / epilogue: warp w reads TMEM lanes (rows) 32 (w % 4) .. 32 (w % 4) + 31 and one half of
+        // the tile's columns, c0 .. c0 + nc - 1, of each diagonal
+        const int quarter = warp & 3, half = (warp - 2) >> 2;
         int sgc = 0;
         bool ok = true;
         for (int w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
             const WorkItem it = items[w];
             const SplitGemmDesc P = probs[it.q];
-            const int tb = P.tb, nkb = P.nkb;
+            const int n0 = it.b * P.tb, nkb = P.nkb;
+            const int tb = min(P.tb, split_trim(P.N) - n0);
             constexpr int nd = ND;
-            const int m0 = it.a * SPLIT_TA, n0 = it.b * tb;
+            const int m0 = it.a * SPLIT_TA;
             const int nt = min(tb, P.N - n0);
+            const int nc = DC == 16 ? 16 : (tb / 2 + 3) & ~3, c0 = half * nc;  // nc <= DC
+            const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + c0;
             const bool mine = c0 < nt;  // warp-uniform
             const int xs = max(0, 32 - __clz(nkb * SPLIT_KB - 1) - 14);  // ceil(log2 K) - 14, if positive
             const int row = m0 + quarter * 32 + lane;
@@ -665,9 +686,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             constexpr bool segs = SEGS;
             const int* a_exp = reinterpret_cast<const int*>(ws + P.a_exp) + (int64_t)row * P.a_nseg;
             int E = SPLIT_EXP_NONE, es_next = segs && rlive ? a_exp[0] : SPLIT_EXP_NONE;
-            long long acc[DCOLS];
+            long long acc[DC];
 #pragma unroll
-            for (int j = 0; j < DCOLS; ++j) acc[j] = 0;
+            for (int j = 0; j < DC; ++j) acc[j] = 0;
             for (int kb0 = 0, sg = 0; kb0 < nkb; kb0 += SPLIT_SEG_KB, ++sg, ++sgc) {
                 const int buf = sgc & 1;
                 int sa = 0, sv = 0;  // right shifts of the running sum and of this segment
@@ -683,7 +704,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                     // the running sum's shift is the same for every column: applied here, once
                     if (sa > 0) {
 #pragma unroll
-                        for (int j = 0; j < DCOLS; ++j) acc[j] = shr_round(acc[j], sa);
+                        for (int j = 0; j < DC; ++j) acc[j] = shr_round(acc[j], sa);
                     }
                 }
                 // this segment's shift and its rounding half (sv >= 62: nothing left of it)
@@ -694,19 +715,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 if (!ok) break;
                 tc_fence_after();
                 if (mine) {
-                    // the nd diagonals of HC columns in flight before one wait (the aligned sum
-                    // takes its 16 columns in two halves, to stay within the registers)
-                    constexpr int HC = SEGS ? 8 : DCOLS;
-#pragma unroll
-                    for (int h = 0; h < DCOLS / HC; ++h) {
+                    // the nd diagonals of some columns in flight before one wait: 16, or 8, 8 (and 4) for
+                    // the aligned sum and the wide tiles, to stay within the registers
+                    auto take = [&](auto width, auto at) {
+                        constexpr int HC = decltype(width)::value, first = decltype(at)::value;
                         uint32_t r[ND][HC];
 #pragma unroll
-                        for (int dg = 0; dg < ND; ++dg) {
-                            if constexpr (HC == 16)
-                                tmem_ld16(lane_base + buf * BUF_COLS + dg * tb, r[dg]);
-                            else
-                                tmem_ld8(lane_base + buf * BUF_COLS + dg * tb + HC * h, r[dg]);
-                        }
+                        for (int dg = 0; dg < ND; ++dg) tmem_ld(lane_base + buf * BUF_COLS + dg * tb + first, r[dg]);
                         tmem_ld_wait();
                         // v = sum_d G_d 2^(BETA (nd-2-d)) (>> xs); the last diagonal is rounded down BETA bits
 #pragma unroll
@@ -721,14 +736,22 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                                     v += (gv + (1ll << (SPLIT_BETA - 1))) >> SPLIT_BETA;
                             }
                             if (xs) v = (v + (1ll << (xs - 1))) >> xs;
-                            const int j = HC * h + jj;
+                            long long& a = acc[first + jj];
                             if (segs) {
-                                if (seg_live) acc[j] += (v + seg_half) >> sv;
+                                if (seg_live) a += (v + seg_half) >> sv;
                             } else {
-                                acc[j] += v;
+                                a += v;
                             }
                         }
+                    };
+                    if constexpr (!SEGS && DC == 16) {
+                        take(Int<16>{}, Int<0>{});
+                    } else {
+                        take(Int<8>{}, Int<0>{});
+                        if (DC == 16 || nc > 8) take(Int<8>{}, Int<8>{});
                     }
+                    if constexpr (DC > 16)
+                        if (nc > 16) take(Int<4>{}, Int<16>{});
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -739,9 +762,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 const int ea = segs ? E : reinterpret_cast<const int*>(ws + P.a_exp)[row];
                 const int* eb_tab = reinterpret_cast<const int*>(ws + P.b_exp);
 #pragma unroll
-                for (int j = 0; j < DCOLS; ++j) {
+                for (int j = 0; j < DC; ++j) {
                     const int col = n0 + c0 + j;
-                    if (c0 + j < nt) {
+                    if ((DC == 16 || j < nc) && c0 + j < nt) {
                         // D = 2^(eA + eB - BETA nd + xs) * acc: one rounding (int64 -> FP64, to
                         // nearest even), then an exact power-of-two scaling (acc = 0 gives 0)
                         const int scale = ea + eb_tab[col] - SPLIT_BETA * nd + xs;
@@ -811,9 +834,11 @@ cudaError_t init_split_kernels(const int* host_tuv) {
         return e;
     const uint16_t* p = static_cast<const uint16_t*>(dev_table);
     if ((e = cudaMemcpyToSymbol(g_gidx, &p, sizeof(p))) != cudaSuccess) return e;
-    const void* kernels[] = {(const void*)split_gemm_kernel<false, 4>, (const void*)split_gemm_kernel<false, 5>,
-                             (const void*)split_gemm_kernel<false, 6>, (const void*)split_gemm_kernel<true, 4>,
-                             (const void*)split_gemm_kernel<true, 5>,  (const void*)split_gemm_kernel<true, 6>};
+#define LX_K(D)                                                                                    \
+    (const void*)split_gemm_kernel<false, D, 16>, (const void*)split_gemm_kernel<false, D, 20>,    \
+        (const void*)split_gemm_kernel<true, D, 16>, (const void*)split_gemm_kernel<true, D, 20>
+    const void* kernels[] = {LX_K(4), LX_K(5), LX_K(6)};
+#undef LX_K
     for (const void* k : kernels)
         if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess)
             return e;
@@ -827,7 +852,7 @@ cudaError_t launch_wait_selftest(unsigned* status, unsigned long long limit, cud
 }
 
 cudaError_t launch_split_gemm(const SplitGemmDesc* probs, const WorkItem* items, int nitems, const char* ws,
-                              double* cbase, unsigned* status, cudaStream_t st, bool segments, int digits) {
+                              double* cbase, unsigned* status, cudaStream_t st, bool segments, int digits, bool wide) {
     if (nitems <= 0) return cudaSuccess;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -835,14 +860,19 @@ cudaError_t launch_split_gemm(const SplitGemmDesc* probs, const WorkItem* items,
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     // one CTA per SM (the TMEM allocation and the operand ring take the whole SM)
     const int grid = nitems < sms ? nitems : sms;
-#define LX_SPLIT_GEMM(S, D) split_gemm_kernel<S, D><<<grid, GEMM_THREADS, SMEM_BYTES, st>>>(probs, items, nitems, ws, cbase, status)
-    switch ((segments ? 8 : 0) + digits) {
-        case 4: LX_SPLIT_GEMM(false, 4); break;
-        case 5: LX_SPLIT_GEMM(false, 5); break;
-        case 6: LX_SPLIT_GEMM(false, 6); break;
-        case 12: LX_SPLIT_GEMM(true, 4); break;
-        case 13: LX_SPLIT_GEMM(true, 5); break;
-        case 14: LX_SPLIT_GEMM(true, 6); break;
+#define LX_SPLIT_GEMM(D)                                                                               \
+    case D:                                                                                            \
+        if (segments)                                                                                  \
+            (wide ? split_gemm_kernel<true, D, 20> : split_gemm_kernel<true, D, 16>)<<<grid, GEMM_THREADS, SMEM_BYTES, st>>>( \
+                probs, items, nitems, ws, cbase, status);                                              \
+        else                                                                                           \
+            (wide ? split_gemm_kernel<false, D, 20> : split_gemm_kernel<false, D, 16>)<<<grid, GEMM_THREADS, SMEM_BYTES, st>>>( \
+                probs, items, nitems, ws, cbase, status);                                              \
+        break;
+    switch (digits) {
+        LX_SPLIT_GEMM(4)
+        LX_SPLIT_GEMM(5)
+        LX_SPLIT_GEMM(6)
         default: return cudaErrorInvalidValue;
     }
 #undef LX_SPLIT_GEMM

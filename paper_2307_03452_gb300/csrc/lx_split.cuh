@@ -13,11 +13,16 @@ constexpr int SPLIT_BETA = 8;                        // bits per digit
 constexpr int SPLIT_W = SPLIT_NSLICE * SPLIT_BETA;   // fixed-point bits kept (48)
 constexpr int SPLIT_KB = 32;                         // K block (elements) of one pipeline stage
 constexpr int SPLIT_TA = 128;                        // A row tile = MMA M
-constexpr int SPLIT_TB = 32;                         // largest B row tile (2 sets x 6 diagonals x 32 TMEM columns)
+constexpr int SPLIT_TB = 40;                         // largest B row tile (2 sets x 6 diagonals x 40 TMEM columns)
 constexpr int SPLIT_SEG_KB = 4;                      // K blocks accumulated in TMEM between int64 drains
 
 // Exponent of an all-zero row segment (below any real exponent; its digits are zero).
 constexpr int SPLIT_EXP_NONE = -(1 << 29);
+
+// B operands are stored in row tiles of split_tb(N) rows, the last one trimmed to N rounded to 8:
+// trim = split_trim(N) rows in all.  (A operands keep whole tiles of SPLIT_TA rows: SPLIT_NO_TRIM.)
+__host__ __device__ inline int split_trim(int N) { return (N + 7) / 8 * 8; }
+constexpr int SPLIT_NO_TRIM = 1 << 30;
 
 // One matrix whose rows are split: src at (double*)base + src_off, row stride ld.  Before
 // splitting, column k is multiplied by 2^(shift_sign * shift[k]) (exact; shift_off < 0: none).
@@ -32,7 +37,8 @@ struct SplitRowsDesc {
     int64_t exp_off;    // bytes from the workspace base (int per padded row, times nseg if fixed = 2)
     int64_t shift_off;  // bytes from the workspace base (int per column), or -1
     int ld, rows, K, T, nkb, shift_sign, fixed, nseg;
-    int nd, pad;  // digit slices written (the first nd of the block's NSLICE)
+    int nd;    // digit slices written (the first nd of the block's NSLICE)
+    int trim;  // rows stored: the last row tile has min(T, trim - its first row) of them
 };
 __host__ __device__ inline int split_nseg(int nkb) { return (nkb + SPLIT_SEG_KB - 1) / SPLIT_SEG_KB; }
 
@@ -67,8 +73,8 @@ __host__ __device__ inline int64_t gidx_offset(int lbra, int lket) {
 }
 static_assert(NHERM_TOT < 65536, "[r]^(0) positions fit 16 bits");
 
-// D = A B^T: A digits (row tiles of SPLIT_TA), B digits (row tiles of tb = split_tb(N)), both
-// with nkb K blocks; D written to (double*)C + c_off with row stride ldc (transpose: D[m][n] ->
+// D = A B^T: A digits (row tiles of SPLIT_TA), B digits (row tiles of tb = split_tb(N), the last
+// trimmed), both with nkb K blocks; D written to (double*)C + c_off with row stride ldc (transpose: D[m][n] ->
 // C[n][m]).  B carries one exponent per row; A one per row (a_nseg = 1) or one per row and
 // segment of SPLIT_SEG_KB K blocks (a_nseg = split_nseg(nkb), int[row][a_nseg]).  The A operand
 // is read only up to M rows rounded to 8 (the last row tile is loaded that far).  B rows past
@@ -83,12 +89,11 @@ struct SplitGemmDesc {
 };
 constexpr int SPLIT_MIN_DIGITS = 4;
 
-// B row tile for an operand of N rows: as few tiles as SPLIT_TB rows allow, each a multiple
-// of 16 rows (169 rows -> 6 tiles of 32, 81 -> 3 of 32, 13 -> 1 of 16).
+// B row tile for an operand of N rows: as few tiles as SPLIT_TB rows allow, evenly filled, each a
+// multiple of 8 rows (169 rows -> 4 of 40 and one of 16, 81 -> 2 of 32 and one of 24, 13 -> 1 of 16).
 __host__ __device__ inline int split_tb(int N) {
     const int tiles = (N + SPLIT_TB - 1) / SPLIT_TB;
-    const int t = (N + tiles - 1) / tiles;
-    return (t + 15) / 16 * 16;
+    return split_trim((N + tiles - 1) / tiles);
 }
 
 __host__ __device__ inline int split_rowpad(int rows, int T) { return (rows + T - 1) / T * T; }
@@ -96,6 +101,11 @@ __host__ __device__ inline int split_nkb(int K) { return (K + SPLIT_KB - 1) / SP
 // bytes of the digit planes of an operand (rows padded to T, K padded to SPLIT_KB)
 __host__ __device__ inline int64_t split_dig_bytes(int rows, int K, int T) {
     return (int64_t)split_rowpad(rows, T) * split_nkb(K) * SPLIT_KB * SPLIT_NSLICE * 2;
+}
+
+// bytes of the digit planes of a B operand
+__host__ __device__ inline int64_t split_dig_bytes_b(int rows, int K) {
+    return (int64_t)split_trim(rows) * split_nkb(K) * SPLIT_KB * SPLIT_NSLICE * 2;
 }
 
 cudaError_t init_split_kernels(const int* host_tuv);
@@ -109,8 +119,9 @@ cudaError_t launch_split_operands(const DQuartet* qd, const SplitQuartet* sq, co
 // limit, on an mbarrier nothing arrives on): sets the status word's timeout bit.
 cudaError_t launch_wait_selftest(unsigned* status, unsigned long long limit, cudaStream_t st);
 // segments: some A operands carry one exponent per segment (a_nseg may exceed 1); otherwise
-// every problem has a_nseg = 1.  digits: the nd (4..6) of every problem of the launch.
+// every problem has a_nseg = 1.  digits: the nd (4..6) of every problem of the launch.  wide: some
+// problem has tb > 32.
 cudaError_t launch_split_gemm(const SplitGemmDesc* probs, const WorkItem* items, int nitems, const char* ws,
-                              double* cbase, unsigned* status, cudaStream_t st, bool segments, int digits);
+                              double* cbase, unsigned* status, cudaStream_t st, bool segments, int digits, bool wide);
 
 }  // namespace lx

@@ -15,7 +15,6 @@
 #include <algorithm>
 #include <map>
 #include <mutex>
-#include <unordered_map>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -193,12 +192,57 @@ struct Overrides {
 
 // ------------------------------------------------------------------ planning
 
-struct PairKey {
-    int64_t v;
-    bool operator==(const PairKey& o) const { return v == o.v; }
-};
-struct PairKeyHash {
-    size_t operator()(const PairKey& k) const { return std::hash<int64_t>()(k.v); }
+// Pair ids of one chunk: an open-addressing table keyed by (shells, side), emptied in O(1) by a new
+// generation.  (std::unordered_map took about a third of the planning of small classes.)
+inline int64_t pair_key(int sa, int sb, int side) { return ((int64_t)sa << 32 | (uint32_t)sb) * 2 + side; }
+class PairMap {
+  public:
+    explicit PairMap(int64_t nquartet) {
+        size_t n = 64;
+        while (n < 4 * (size_t)std::min<int64_t>(nquartet, 1 << 20)) n *= 2;
+        slots_.assign(n, Slot{0, 0, 0});
+    }
+    void clear() {
+        ++gen_;
+        used_ = 0;
+    }
+    // The id stored for k, or `id` after storing it (fresh = true).
+    int get(int64_t k, int id, bool& fresh) {
+        if (2 * (used_ + 1) > slots_.size()) grow();
+        Slot& s = find(k);
+        fresh = s.gen != gen_;
+        if (fresh) {
+            s = Slot{k, id, gen_};
+            ++used_;
+        }
+        return s.id;
+    }
+    bool has(int64_t k) { return find(k).gen == gen_; }
+
+  private:
+    struct Slot {
+        int64_t key;
+        int id;
+        unsigned gen;
+    };
+    Slot& find(int64_t k) {
+        uint64_t h = (uint64_t)k * 0x9E3779B97F4A7C15ull;
+        h ^= h >> 32;
+        size_t i = (size_t)h & (slots_.size() - 1);
+        while (slots_[i].gen == gen_ && slots_[i].key != k) i = (i + 1) & (slots_.size() - 1);
+        return slots_[i];
+    }
+    void grow() {
+        std::vector<Slot> old(2 * slots_.size(), Slot{0, 0, 0});
+        old.swap(slots_);
+        const unsigned g = gen_;
+        gen_ = 1;
+        for (const Slot& s : old)
+            if (s.gen == g) find(s.key) = Slot{s.key, s.id, 1};
+    }
+    std::vector<Slot> slots_;
+    size_t used_ = 0;
+    unsigned gen_ = 1;
 };
 
 struct Chunk {
@@ -309,6 +353,39 @@ int axial_route(const lx_shell* sh, const lx_quartet& q, int flags) {
     return axial_quartet_bytes(sh, q, flags, true) <= room ? 2 : axial_quartet_bytes(sh, q, flags, false) <= room;
 }
 
+// What the planner needs of a quartet that depends on its class and contraction degrees alone,
+// computed once per shape of a batch.
+struct Shape {
+    uint64_t key = ~0ull;
+    size_t qbytes = 0, bra_bytes = 0, ket_bytes = 0;
+    int route = 0, nsplit = 1;
+};
+class Shapes {
+  public:
+    Shapes(const lx_shell* sh, int flags) : sh_(sh), flags_(flags), cache_(1024) {}
+    const Shape& of(const lx_quartet& q) {
+        uint64_t k = 0;
+        for (int i = 0; i < 4; ++i) k = k << 8 | (uint64_t)(sh_[q.s[i]].l << 5 | sh_[q.s[i]].nprim);
+        uint64_t h = k * 0x9E3779B97F4A7C15ull;
+        Shape& s = cache_[h >> 54];
+        if (s.key != k) {
+            s.key = k;
+            s.qbytes = quartet_bytes(sh_, q, flags_);
+            s.bra_bytes = pair_bytes(sh_, q.s[0], q.s[1], flags_);
+            s.ket_bytes = pair_bytes(sh_, q.s[2], q.s[3], flags_);
+            s.route = axial_route(sh_, q, flags_);
+            s.nsplit = s.route ? axial_split(sh_, q, flags_, s.route == 2) : 1;
+        }
+        return s;
+    }
+
+  private:
+    const lx_shell* sh_;
+    int flags_;
+    std::vector<Shape> cache_;
+};
+static_assert(LX_LMAX < 8 && LX_KMAX < 32, "a shell's l and degree fit 8 bits of a shape key");
+
 constexpr size_t CHUNK_SLACK = 32 * 256;  // alignment padding of the chunk's regions and the work counters
 
 size_t head_bytes(int nshell, int nprim) {
@@ -316,21 +393,20 @@ size_t head_bytes(int nshell, int nprim) {
 }
 
 // Greedy chunking of the quartet list so that each chunk fits `budget` bytes.
-int plan_chunks(const lx_shell* sh, const lx_quartet* qs, int64_t nq, int flags, size_t budget,
+int plan_chunks(Shapes& shapes, const lx_quartet* qs, int64_t nq, size_t budget, PairMap& seen,
                 std::vector<Chunk>& chunks) {
     chunks.clear();
-    std::unordered_map<PairKey, int, PairKeyHash> seen;
+    seen.clear();
     size_t used = CHUNK_SLACK;
     Chunk cur;
     cur.q_begin = 0;
     for (int64_t i = 0; i < nq; ++i) {
         const lx_quartet& q = qs[i];
-        size_t add = quartet_bytes(sh, q, flags);
-        const PairKey kb{((int64_t)q.s[0] << 32 | (uint32_t)q.s[1]) * 2};
-        const PairKey kk{((int64_t)q.s[2] << 32 | (uint32_t)q.s[3]) * 2 + 1};
-        const bool nb = !seen.count(kb), nk = !seen.count(kk);
-        if (nb) add += pair_bytes(sh, q.s[0], q.s[1], flags);
-        if (nk && !(kk == kb)) add += pair_bytes(sh, q.s[2], q.s[3], flags);
+        const Shape& s = shapes.of(q);
+        const int64_t kb = pair_key(q.s[0], q.s[1], 0), kk = pair_key(q.s[2], q.s[3], 1);
+        size_t add = s.qbytes;
+        if (!seen.has(kb)) add += s.bra_bytes;
+        if (!seen.has(kk)) add += s.ket_bytes;
         if (used + add > budget) {
             if (i == cur.q_begin) return LX_ERR_WORKSPACE;  // one quartet does not fit
             cur.q_end = i;
@@ -342,8 +418,9 @@ int plan_chunks(const lx_shell* sh, const lx_quartet* qs, int64_t nq, int flags,
             continue;
         }
         used += add;
-        seen[kb] = 1;
-        seen[kk] = 1;
+        bool fresh;
+        seen.get(kb, 0, fresh);
+        seen.get(kk, 0, fresh);
     }
     cur.q_end = nq;
     if (nq > 0) chunks.push_back(cur);
@@ -380,11 +457,40 @@ struct ChunkPlan {
     size_t ax_smem[AX_NBIN] = {}, ax_rot_k = 0, ax_rot_b = 0;
     size_t off_axp = 0, off_axq = 0, off_aip = 0, off_ait = 0, off_aim = 0, off_airk = 0, off_airb = 0;
     size_t total = 0;         // bytes from the chunk base
-    std::vector<char> blob;   // descriptor bytes [0, off_data)
+
+    // Write the descriptors and work lists, bytes [0, off_data) of the chunk, to dst.
+    void write(char* dst) const {
+        auto put = [dst](size_t off, const auto& v) {
+            if (!v.empty()) std::memcpy(dst + off, v.data(), sizeof(v[0]) * v.size());
+        };
+        put(off_pairs, pairs);
+        put(off_quartets, quartets);
+        put(off_h, items_h);
+        put(off_br, items_br);
+        put(off_g1, items_g1);
+        put(off_g2, items_g2);
+        std::memset(dst + off_counters, 0, sizeof(int) * 2 * GEMM_NVARIANT);
+        put(off_srd, srd);
+        put(off_sq, sq);
+        put(off_sg1, sg1);
+        put(off_sg2, sg2);
+        put(off_isr, items_sr);
+        put(off_isB, items_sB);
+        put(off_isg1, items_sg1);
+        put(off_isD, items_sD);
+        put(off_isg2, items_sg2);
+        put(off_axp, ax_pairs);
+        put(off_axq, ax_quartets);
+        put(off_aip, ax_ip);
+        put(off_ait, ax_it);
+        put(off_aim, ax_im);
+        put(off_airk, ax_irk);
+        put(off_airb, ax_irb);
+    }
 };
 
 void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int flags, size_t chunk_base,
-                 ChunkPlan& P, const Overrides& ov = Overrides()) {
+                 Shapes& shapes, PairMap& pid, PairMap& apid, ChunkPlan& P, const Overrides& ov) {
     const bool solid = flags & LX_SOLID, split = flags & LX_PATH_SPLIT, jk = flags & JK_DIGEST;
     const int nd_flag = (flags & LX_SPLIT_DIGITS_MASK) >> 4, nd = nd_flag ? nd_flag : SPLIT_NSLICE;
     P.digits = nd;
@@ -409,11 +515,12 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
     P.ax_quartets.clear();
     for (auto* v : {&P.ax_ip, &P.ax_it, &P.ax_im, &P.ax_irk, &P.ax_irb}) v->clear();
     std::vector<int64_t> dense;  // index of each matrix-form quartet in qs
-    std::unordered_map<PairKey, int, PairKeyHash> pid, apid;
+    pid.clear();
+    apid.clear();
     auto get_ax_pair = [&](int sa, int sb, int side) {
-        const PairKey k{((int64_t)sa << 32 | (uint32_t)sb) * 2 + side};
-        const auto ins = apid.emplace(k, (int)P.ax_pairs.size());
-        if (!ins.second) return ins.first->second;
+        bool fresh;
+        const int id = apid.get(pair_key(sa, sb, side), (int)P.ax_pairs.size(), fresh);
+        if (!fresh) return id;
         AxPair p{};
         p.sa = sa;
         p.sb = sb;
@@ -424,12 +531,12 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
         p.cls = ax_class_id(p.la, p.lb, solid);
         p.nh = axial_tables().cls[p.cls].nh;
         P.ax_pairs.push_back(p);
-        return ins.first->second;
+        return id;
     };
     auto get_pair = [&](int sa, int sb, int side) {
-        const PairKey k{((int64_t)sa << 32 | (uint32_t)sb) * 2 + side};
-        auto f = pid.find(k);
-        if (f != pid.end()) return f->second;
+        bool fresh;
+        const int id = pid.get(pair_key(sa, sb, side), (int)P.pairs.size(), fresh);
+        if (!fresh) return id;
         DPair p{};
         p.cs_off = -1;  // set with the data layout on the split path
         p.sa = sa;
@@ -439,14 +546,26 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
         p.np = pyr(sh[sa].l + sh[sb].l);
         p.sign = side;
         p.solid = solid ? 1 : 0;
-        const int id = (int)P.pairs.size();
         P.pairs.push_back(p);
-        pid.emplace(k, id);
         return id;
     };
+    {
+        // room for the lists, so that they are not copied as they grow
+        size_t nax = 0, prims = 0, nmatrix = 0;
+        for (int64_t i = ch.q_begin; i < ch.q_end; ++i) {
+            const lx_quartet& q = qs[i];
+            if (ov.v1 < 0 && shapes.of(q).route) ++nax;
+            else ++nmatrix;
+            prims += (size_t)sh[q.s[0]].nprim * sh[q.s[1]].nprim * sh[q.s[2]].nprim * sh[q.s[3]].nprim;
+        }
+        P.quartets.reserve(nmatrix);
+        dense.reserve(nmatrix);
+        P.ax_quartets.reserve(nax);
+        (nax ? P.ax_it : P.items_br).reserve(prims);
+    }
     for (int64_t i = ch.q_begin; i < ch.q_end; ++i) {
         const lx_quartet& q = qs[i];
-        const int route = ov.v1 < 0 ? axial_route(sh, q, flags) : 0;
+        const int route = ov.v1 < 0 ? shapes.of(q).route : 0;
         if (route) {
             const lx_shell &a = sh[q.s[0]], &b = sh[q.s[1]], &c = sh[q.s[2]], &dd = sh[q.s[3]];
             AxQuartet x{};
@@ -461,7 +580,7 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
             x.cb = ax_class_id(a.l, b.l, solid);
             x.ck = ax_class_id(c.l, dd.l, solid);
             x.full = route == 2;
-            x.nsplit = axial_split(sh, q, flags, x.full);
+            x.nsplit = shapes.of(q).nsplit;
             x.tab_stride = ax_t_size(x.Lb, x.Lk, x.full);
             x.out_off = q.out_offset;
             P.ax_quartets.push_back(x);
@@ -488,12 +607,9 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
     for (int i = 0; i < (int)P.ax_pairs.size(); ++i)
         for (int kp = 0; kp < P.ax_pairs[i].Kab; ++kp) P.ax_ip.push_back({i, kp, 0, 0});
     {
-        struct Cost {
-            int bin;
-            int64_t c;
-            WorkItem w;
-        };
-        std::vector<Cost> main;
+        // (group, ~cost) and position: sorting these keeps the order of equal items
+        std::vector<std::pair<uint64_t, uint32_t>> order;
+        std::vector<WorkItem> main;
         int nmax_k = 0, nmax_b = 0;
         P.ax_lmax = 0;
         for (int b = 0; b < AX_NBIN; ++b) {
@@ -506,26 +622,46 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
         }
         P.ax_lanes_k = axial_lanes(nmax_k);
         P.ax_lanes_b = axial_lanes(nmax_b);
+        size_t nmain = 0, nrk = 0, nrb = 0;
+        for (const AxQuartet& x : P.ax_quartets) {
+            nmain += (size_t)x.nsplit * ((axial_tables().cls[x.cb].nhalf + AX_NR - 1) / AX_NR);
+            nrk += (x.nab + P.ax_lanes_k - 1) / P.ax_lanes_k;
+            nrb += (x.ncd + P.ax_lanes_b - 1) / P.ax_lanes_b;
+        }
+        order.reserve(nmain);
+        main.reserve(nmain);
+        P.ax_irk.reserve(nrk);
+        P.ax_irb.reserve(nrb);
         P.ax_rot_k = axial_rotate_smem(nmax_k, P.ax_lanes_k);
         P.ax_rot_b = axial_rotate_smem(nmax_b, P.ax_lanes_b);
+        int bins[AX_NL][AX_NL];
+        for (auto& r : bins)
+            for (int& b : r) b = -1;
         for (int i = 0; i < (int)P.ax_quartets.size(); ++i) {
             const AxQuartet& x = P.ax_quartets[i];
-            const int prim = x.kbra * x.kket, nhalf = axial_tables().cls[x.cb].nhalf, bin = axial_bin(x.Lb, x.Lk);
-            P.ax_lmax = std::max(P.ax_lmax, std::max(x.Lb, x.Lk));
-            P.ax_smem[bin] = std::max(P.ax_smem[bin], axial_main_smem(x.Lb, x.Lk));
+            const int prim = x.kbra * x.kket, nhalf = axial_tables().cls[x.cb].nhalf;
+            int& bin = bins[x.Lb][x.Lk];
+            if (bin < 0) {
+                bin = axial_bin(x.Lb, x.Lk);
+                P.ax_lmax = std::max(P.ax_lmax, std::max(x.Lb, x.Lk));
+                P.ax_smem[bin] = std::max(P.ax_smem[bin], axial_main_smem(x.Lb, x.Lk));
+            }
             for (int k = 0; k < prim; ++k) P.ax_it.push_back({i, k, 0, 0});
             for (int r = 0; r < nhalf; r += AX_NR) {
                 const int n = std::min(AX_NR, nhalf - r);
-                for (int c = 0; c < x.nsplit; ++c)
-                    main.push_back({bin, (int64_t)prim * pyr(x.Lk) * (2 * nhalf - r) / x.nsplit, {i, r, n, c}});
+                const uint64_t cost = (uint64_t)prim * pyr(x.Lk) * (2 * nhalf - r) / x.nsplit;
+                for (int c = 0; c < x.nsplit; ++c) {
+                    order.push_back({(uint64_t)bin << 60 | ((1ull << 60) - 1 - cost), (uint32_t)main.size()});
+                    main.push_back({i, r, n, c});
+                }
                 P.ax_counts[bin] += x.nsplit;
             }
             for (int r = 0; r < x.nab; r += P.ax_lanes_k) P.ax_irk.push_back({i, r, 0, 0});
             for (int r = 0; r < x.ncd; r += P.ax_lanes_b) P.ax_irb.push_back({i, r, 0, 0});
         }
-        std::stable_sort(main.begin(), main.end(),
-                         [](const Cost& a, const Cost& b) { return a.bin != b.bin ? a.bin < b.bin : a.c > b.c; });
-        for (const Cost& c : main) P.ax_im.push_back(c.w);
+        if (!std::is_sorted(order.begin(), order.end())) std::sort(order.begin(), order.end());
+        P.ax_im.reserve(main.size());
+        for (const auto& o : order) P.ax_im.push_back(main[o.second]);
     }
     // work lists
     for (int i = 0; i < (int)P.pairs.size(); ++i)
@@ -595,18 +731,16 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
     // grouped by tile shape (one persistent launch each), largest tiles first within a shape:
     // the persistent launches hand items out round-robin
     auto lpt = [](std::vector<WorkItem>& items, const std::vector<int64_t>& cost, int* counts) {
-        std::vector<size_t> idx(items.size());
-        for (size_t k = 0; k < idx.size(); ++k) idx[k] = k;
-        std::stable_sort(idx.begin(), idx.end(), [&](size_t x, size_t y) {
-            if (items[x].c != items[y].c) return items[x].c < items[y].c;
-            return cost[x] > cost[y];
-        });
-        std::vector<WorkItem> sorted(items.size());
+        std::vector<std::pair<uint64_t, uint32_t>> order(items.size());  // (shape, ~cost) and position
         for (int v = 0; v < GEMM_NVARIANT; ++v) counts[v] = 0;
-        for (size_t k = 0; k < idx.size(); ++k) {
-            sorted[k] = items[idx[k]];
-            ++counts[sorted[k].c];
+        for (size_t k = 0; k < items.size(); ++k) {
+            order[k] = {(uint64_t)items[k].c << 60 | ((1ull << 60) - 1 - (uint64_t)cost[k]), (uint32_t)k};
+            ++counts[items[k].c];
         }
+        if (std::is_sorted(order.begin(), order.end())) return;
+        std::sort(order.begin(), order.end());
+        std::vector<WorkItem> sorted(items.size());
+        for (size_t k = 0; k < order.size(); ++k) sorted[k] = items[order[k].second];
         items.swap(sorted);
     };
     lpt(P.items_g1, cost1, P.g1_counts);
@@ -623,10 +757,9 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
             // columns scaled into (-1, 1): one pass, e = 0 per row
             P.srd.push_back(
                 SplitRowsDesc{0, 0, 0, 0, k, pr.nrow, k, tb, split_nkb(k), -1, 1, 0, nd, split_trim(pr.nrow)});
-            // digit kernels: one item per 8 consecutive rows, up to nrow rounded to 8 (the GEMMs
-            // drop the output columns of B rows past nrow, so the rest of the last row tile is
-            // never written)
-            for (int row = 0; row < split_rowpad(pr.nrow, 8); row += 8) P.items_sB.push_back({p, row, 0, 0});
+            // digit kernels: one item (a CTA) per 64 consecutive rows, written up to nrow rounded
+            // to 8 (the GEMMs drop the output columns of B rows past nrow)
+            for (int row = 0; row < pr.nrow; row += SPLIT_ITEM_ROWS) P.items_sB.push_back({p, row, 0, 0});
         }
         for (int i = 0; i < (int)P.quartets.size(); ++i) {
             const DQuartet& d = P.quartets[i];
@@ -644,9 +777,9 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
             // A2: X, one exponent per row and segment (the rows up to nab rounded to 8 are used)
             P.srd.push_back(SplitRowsDesc{0, 0, 0, 0, k2, d.nab, k2, SPLIT_TA, q.nkb2, +1, 2, split_nseg(q.nkb2), nd,
                                           SPLIT_NO_TRIM});
-            for (int row = 0; row < split_rowpad(k2, 8); row += 8) P.items_sr.push_back({i, row, 0, 0});
+            for (int row = 0; row < k2; row += SPLIT_ITEM_ROWS) P.items_sr.push_back({i, row, 0, 0});
             // X's digit planes only after GEMM1
-            for (int row = 0; row < split_rowpad(d.nab, 8); row += 8) P.items_sD.push_back({npair + i, row, 0, 0});
+            for (int row = 0; row < d.nab; row += SPLIT_ITEM_ROWS) P.items_sD.push_back({npair + i, row, 0, 0});
             const int mt1 = split_rowpad(k2, SPLIT_TA) / SPLIT_TA, nt1 = (d.nab + tb1 - 1) / tb1;
             const int mt2 = split_rowpad(d.nab, SPLIT_TA) / SPLIT_TA, nt2 = (d.ncd + tb2 - 1) / tb2;
             for (int m = 0; m < mt1; ++m)
@@ -655,10 +788,11 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
                 for (int n = 0; n < nt2; ++n) P.items_sg2.push_back({i, m, n, 0});
         }
         // the persistent split GEMM hands items to CTAs in a fixed stride: longest first
-        std::stable_sort(P.items_sg1.begin(), P.items_sg1.end(),
-                         [&](const WorkItem& x, const WorkItem& y) { return P.sq[x.q].nkb1 > P.sq[y.q].nkb1; });
-        std::stable_sort(P.items_sg2.begin(), P.items_sg2.end(),
-                         [&](const WorkItem& x, const WorkItem& y) { return P.sq[x.q].nkb2 > P.sq[y.q].nkb2; });
+        auto longest = [&](std::vector<WorkItem>& v, auto more) {
+            if (!std::is_sorted(v.begin(), v.end(), more)) std::stable_sort(v.begin(), v.end(), more);
+        };
+        longest(P.items_sg1, [&](const WorkItem& x, const WorkItem& y) { return P.sq[x.q].nkb1 > P.sq[y.q].nkb1; });
+        longest(P.items_sg2, [&](const WorkItem& x, const WorkItem& y) { return P.sq[x.q].nkb2 > P.sq[y.q].nkb2; });
     }
     // byte layout from the chunk base
     size_t o = 0;
@@ -781,48 +915,22 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
         }
     }
     P.total = (size_t)dw * 8 - chunk_base;
-    P.blob.assign(P.off_data, 0);
-    auto put = [&](size_t off, const void* src, size_t bytes) {
-        if (bytes) std::memcpy(P.blob.data() + off, src, bytes);
-    };
-    put(P.off_pairs, P.pairs.data(), sizeof(DPair) * P.pairs.size());
-    put(P.off_quartets, P.quartets.data(), sizeof(DQuartet) * P.quartets.size());
-    put(P.off_h, P.items_h.data(), sizeof(WorkItem) * P.items_h.size());
-    put(P.off_br, P.items_br.data(), sizeof(WorkItem) * P.items_br.size());
-    put(P.off_g1, P.items_g1.data(), sizeof(WorkItem) * P.items_g1.size());
-    put(P.off_g2, P.items_g2.data(), sizeof(WorkItem) * P.items_g2.size());
-    put(P.off_srd, P.srd.data(), sizeof(SplitRowsDesc) * P.srd.size());
-    put(P.off_sq, P.sq.data(), sizeof(SplitQuartet) * P.sq.size());
-    put(P.off_sg1, P.sg1.data(), sizeof(SplitGemmDesc) * P.sg1.size());
-    put(P.off_sg2, P.sg2.data(), sizeof(SplitGemmDesc) * P.sg2.size());
-    put(P.off_isr, P.items_sr.data(), sizeof(WorkItem) * P.items_sr.size());
-    put(P.off_isB, P.items_sB.data(), sizeof(WorkItem) * P.items_sB.size());
-    put(P.off_isg1, P.items_sg1.data(), sizeof(WorkItem) * P.items_sg1.size());
-    put(P.off_isD, P.items_sD.data(), sizeof(WorkItem) * P.items_sD.size());
-    put(P.off_isg2, P.items_sg2.data(), sizeof(WorkItem) * P.items_sg2.size());
-    put(P.off_axp, P.ax_pairs.data(), sizeof(AxPair) * P.ax_pairs.size());
-    put(P.off_axq, P.ax_quartets.data(), sizeof(AxQuartet) * P.ax_quartets.size());
-    put(P.off_aip, P.ax_ip.data(), sizeof(WorkItem) * P.ax_ip.size());
-    put(P.off_ait, P.ax_it.data(), sizeof(WorkItem) * P.ax_it.size());
-    put(P.off_aim, P.ax_im.data(), sizeof(WorkItem) * P.ax_im.size());
-    put(P.off_airk, P.ax_irk.data(), sizeof(WorkItem) * P.ax_irk.size());
-    put(P.off_airb, P.ax_irb.data(), sizeof(WorkItem) * P.ax_irb.size());
 }
 
 // Workspace bytes that plan_chunks needs to keep quartets [b, e) in one chunk (an upper
 // bound of the exact layout built by build_chunk).
-size_t chunk_estimate(const lx_shell* sh, const lx_quartet* qs, int64_t b, int64_t e, int flags) {
-    std::unordered_map<PairKey, int, PairKeyHash> seen;
+size_t chunk_estimate(Shapes& shapes, const lx_quartet* qs, int64_t b, int64_t e, PairMap& seen) {
+    seen.clear();
     size_t used = CHUNK_SLACK;
     for (int64_t i = b; i < e; ++i) {
         const lx_quartet& q = qs[i];
-        used += quartet_bytes(sh, q, flags);
-        const PairKey kb{((int64_t)q.s[0] << 32 | (uint32_t)q.s[1]) * 2};
-        const PairKey kk{((int64_t)q.s[2] << 32 | (uint32_t)q.s[3]) * 2 + 1};
-        if (!seen.count(kb)) used += pair_bytes(sh, q.s[0], q.s[1], flags);
-        if (!seen.count(kk)) used += pair_bytes(sh, q.s[2], q.s[3], flags);
-        seen[kb] = 1;
-        seen[kk] = 1;
+        const Shape& s = shapes.of(q);
+        bool fresh;
+        used += s.qbytes;
+        seen.get(pair_key(q.s[0], q.s[1], 0), 0, fresh);
+        if (fresh) used += s.bra_bytes;
+        seen.get(pair_key(q.s[2], q.s[3], 1), 0, fresh);
+        if (fresh) used += s.ket_bytes;
     }
     return used;
 }
@@ -855,7 +963,9 @@ int plan_batch(const lx_shell* shells, int32_t nshell, const double* exps, const
     if (workspace_bytes < B.head + CHUNK_SLACK) return LX_ERR_WORKSPACE;
     const int pflags = flags & (LX_SOLID | LX_PATH_SPLIT | JK_DIGEST | LX_SPLIT_DIGITS_MASK);
     std::vector<Chunk> chunks;
-    int v = plan_chunks(shells, quartets, nquartet, pflags, workspace_bytes - B.head, chunks);
+    Shapes shapes(shells, pflags);
+    PairMap pid(nquartet), apid(nquartet);
+    int v = plan_chunks(shapes, quartets, nquartet, workspace_bytes - B.head, pid, chunks);
     if (v != LX_OK) return v;
     B.head_blob.assign(B.head, 0);
     DShell* dsh = reinterpret_cast<DShell*>(B.head_blob.data());
@@ -878,7 +988,7 @@ int plan_batch(const lx_shell* shells, int32_t nshell, const double* exps, const
     }
     for (size_t c = 0; c < chunks.size(); ++c) {
         B.chunks.emplace_back();
-        build_chunk(shells, quartets, chunks[c], pflags, B.head, B.chunks.back(), ov);
+        build_chunk(shells, quartets, chunks[c], pflags, B.head, shapes, pid, apid, B.chunks.back(), ov);
         if (B.head + B.chunks.back().total <= workspace_bytes) continue;
         // a pair used by matrix-form and by axial quartets of one chunk is stored in both forms,
         // which plan_chunks does not count: halve such a chunk
@@ -1168,9 +1278,14 @@ int eri_batch_unstaged(const lx_shell* shells, int32_t nshell, const double* exp
     if ((v = plan_batch(shells, nshell, exps, coefs, nprim_total, quartets, nquartet, flags, workspace_bytes,
                         Overrides(), B)) != LX_OK)
         return v;
-    std::vector<const char*> blobs;
-    for (const auto& P : B.chunks) blobs.push_back(P.blob.data());
-    return enqueue_batch(B, B.head_blob.data(), blobs, out, workspace, status, static_cast<cudaStream_t>(cuda_stream),
+    std::vector<std::vector<char>> blobs(B.chunks.size());
+    std::vector<const char*> src;
+    for (size_t c = 0; c < blobs.size(); ++c) {
+        blobs[c].resize(B.chunks[c].off_data);
+        B.chunks[c].write(blobs[c].data());
+        src.push_back(blobs[c].data());
+    }
+    return enqueue_batch(B, B.head_blob.data(), src, out, workspace, status, static_cast<cudaStream_t>(cuda_stream),
                          (flags & LX_TIME_STAGES) != 0, nullptr);
 }
 
@@ -1201,7 +1316,7 @@ int eri_batch_staged(const lx_shell* shells, int32_t nshell, const double* exps,
     if (v != LX_OK) return v;
     // descriptors into a pinned staging buffer, so that the uploads do not wait for the stream
     size_t total = align256(B.head_blob.size());
-    for (const auto& P : B.chunks) total += align256(P.blob.size());
+    for (const auto& P : B.chunks) total += align256(P.off_data);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
@@ -1213,9 +1328,9 @@ int eri_batch_staged(const lx_shell* shells, int32_t nshell, const double* exps,
     size_t o = align256(B.head_blob.size());
     std::vector<const char*> blobs;
     for (const auto& P : B.chunks) {
-        std::memcpy(stage + o, P.blob.data(), P.blob.size());
+        P.write(stage + o);
         blobs.push_back(stage + o);
-        o += align256(P.blob.size());
+        o += align256(P.off_data);
     }
     v = enqueue_batch(B, head_src, blobs, out, workspace, status, st, (flags & LX_TIME_STAGES) != 0, jk);
     const int r = stage_release(dev, idx, st, true);
@@ -1269,11 +1384,11 @@ int64_t workspace_need(const lx_shell* shells, int32_t nshell, const lx_quartet*
     const int32_t solid = (flags & LX_SOLID) | extra;
     // a routed quartet may take either path; the predictions come first
     const bool routed = flags & LX_PATH_ROUTED;
+    Shapes plain(shells, routed ? solid : solid | (flags & LX_PATH_SPLIT)), split(shells, solid | LX_PATH_SPLIT);
+    PairMap seen(least ? 1 : nquartet);
     auto est = [&](int64_t b, int64_t e) {
-        if (routed)
-            return std::max(chunk_estimate(shells, quartets, b, e, solid),
-                            chunk_estimate(shells, quartets, b, e, solid | LX_PATH_SPLIT));
-        return chunk_estimate(shells, quartets, b, e, solid | (flags & LX_PATH_SPLIT));
+        const size_t n = chunk_estimate(plain, quartets, b, e, seen);
+        return routed ? std::max(n, chunk_estimate(split, quartets, b, e, seen)) : n;
     };
     size_t need = CHUNK_SLACK;
     if (!least)
@@ -1482,19 +1597,22 @@ int lx_eri_graph_create(const lx_shell* shells, int32_t nshell, const double* ex
         return code;
     };
     // host bytes the graph's copy nodes read: pinned and owned by the handle
-    auto pin = [&](const std::vector<char>& src, const char** dst) {
+    auto pin = [&](size_t bytes, const char** dst, auto fill) {
         void* p = nullptr;
-        cudaError_t e = cudaHostAlloc(&p, src.size() > 0 ? src.size() : 1, cudaHostAllocDefault);
+        cudaError_t e = cudaHostAlloc(&p, bytes > 0 ? bytes : 1, cudaHostAllocDefault);
         if (e != cudaSuccess) return e;
-        if (!src.empty()) std::memcpy(p, src.data(), src.size());
+        fill(static_cast<char*>(p));
         h->pinned.push_back(p);
         *dst = static_cast<const char*>(p);
         return cudaSuccess;
     };
     const char* head_src = nullptr;
     std::vector<const char*> blobs(B.chunks.size());
-    cudaError_t e = pin(B.head_blob, &head_src);
-    for (size_t c = 0; e == cudaSuccess && c < B.chunks.size(); ++c) e = pin(B.chunks[c].blob, &blobs[c]);
+    cudaError_t e = pin(B.head_blob.size(), &head_src, [&](char* p) {
+        if (!B.head_blob.empty()) std::memcpy(p, B.head_blob.data(), B.head_blob.size());
+    });
+    for (size_t c = 0; e == cudaSuccess && c < B.chunks.size(); ++c)
+        e = pin(B.chunks[c].off_data, &blobs[c], [&](char* p) { B.chunks[c].write(p); });
     if (e != cudaSuccess) return fail(cuda_fail(e));
     cudaStream_t cs = nullptr;
     if ((e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking)) != cudaSuccess) return fail(cuda_fail(e));
@@ -1581,8 +1699,13 @@ int lx_eri_autotune(const lx_shell* shells, int32_t nshell, const double* exps, 
             if ((v = plan_batch(shells, nshell, exps, coefs, nprim_total, sub.data(), (int64_t)sub.size(),
                                 flags & (LX_SOLID | LX_PATH_SPLIT), workspace_bytes, ov, B)) != LX_OK)
                 return v;
+            std::vector<std::vector<char>> bytes(B.chunks.size());
             std::vector<const char*> blobs;
-            for (const auto& P : B.chunks) blobs.push_back(P.blob.data());
+            for (size_t c = 0; c < bytes.size(); ++c) {
+                bytes[c].resize(B.chunks[c].off_data);
+                B.chunks[c].write(bytes[c].data());
+                blobs.push_back(bytes[c].data());
+            }
             double t1 = 1e300, t2 = 1e300;
             for (int rep = 0; rep < 3; ++rep) {  // first repetition warms up
                 if ((v = enqueue_batch(B, B.head_blob.data(), blobs, out, workspace, status, st, true, nullptr)) !=
@@ -1920,8 +2043,8 @@ int lx_split_gemm(int32_t M, int32_t N, int32_t K, const double* A, int32_t lda,
     rd[0] = SplitRowsDesc{0, 0, 0, -1, lda, M, K, SPLIT_TA, nkb, 0, 0, 0, digits, SPLIT_NO_TRIM};
     rd[1] = SplitRowsDesc{0, 0, 0, -1, ldb, N, K, tb, nkb, 0, 0, 0, digits, rb};
     std::vector<WorkItem> ia, ib, ig;
-    for (int r = 0; r < ra; r += 8) ia.push_back({0, r, 0, 0});
-    for (int r = 0; r < rb; r += 8) ib.push_back({1, r, 0, 0});
+    for (int r = 0; r < M; r += SPLIT_ITEM_ROWS) ia.push_back({0, r, 0, 0});
+    for (int r = 0; r < N; r += SPLIT_ITEM_ROWS) ib.push_back({1, r, 0, 0});
     for (int m = 0; m < ra / SPLIT_TA; ++m)
         for (int n = 0; n < (N + tb - 1) / tb; ++n) ig.push_back({0, m, n, 0});
     size_t o = 0;

@@ -250,6 +250,8 @@ __device__ inline int64_t dig_index(int row, int k, int s, int T, int nkb, int t
            ((r >> 3) * (SPLIT_KB / 8) + (kk >> 3)) * 64 + (r & 7) * 8 + (kk & 7);
 }
 
+constexpr int DIGIT_THREADS = 4 * SPLIT_ITEM_ROWS;  // a warp per 8 rows
+
 // split_rows_kernel gives one warp 8 consecutive rows r0 .. r0+7 (r0 a multiple of 8), taken
 // as four pairs.  For a pair, lane (rr, c) = (lane / 16, lane % 16) handles row r0 + 2i + rr and
 // the 8-column groups c, c + 16, c + 32, ... (columns 128 j + 8c .. 128 j + 8c + 7).  A pair is
@@ -323,15 +325,17 @@ __device__ __forceinline__ void split_8rows(int r0, int nkb, int T, int trim, in
     }
 }
 
-// One split_rows item (item.q = descriptor, item.a = r0), by one warp (SEGMENTS: fixed = 2 may
-// occur).
+// One warp's 8 rows from r0 = item.a + 8 warp of a split_rows item (item.q = descriptor; SEGMENTS:
+// fixed = 2 may occur).
 template <bool SEGMENTS>
 __device__ __forceinline__ void split_rows_item(const SplitRowsDesc* __restrict__ descs, const WorkItem& it,
                                                 const double* __restrict__ src_base, char* __restrict__ ws) {
     const SplitRowsDesc d = descs[it.q];
+    const int r0 = it.a + 8 * (threadIdx.x >> 5);
+    if (r0 >= d.rows) return;
     const double* src = src_base + d.src_off;
     const int* shift = d.shift_off >= 0 ? reinterpret_cast<const int*>(ws + d.shift_off) : nullptr;
-    split_8rows<SEGMENTS>(it.a, d.nkb, d.T, d.trim, d.fixed, d.nseg, d.nd, reinterpret_cast<__nv_bfloat16*>(ws + d.dig_off),
+    split_8rows<SEGMENTS>(r0, d.nkb, d.T, d.trim, d.fixed, d.nseg, d.nd, reinterpret_cast<__nv_bfloat16*>(ws + d.dig_off),
                 reinterpret_cast<int*>(ws + d.exp_off), [&](int row, int k0, double (&v)[8], int (&sh)[8]) {
                     const bool live = row < d.rows;
                     const double* sr = src + (int64_t)row * d.ld;
@@ -345,12 +349,10 @@ __device__ __forceinline__ void split_rows_item(const SplitRowsDesc* __restrict_
                 });
 }
 
-__global__ void __launch_bounds__(256) split_rows_kernel(const SplitRowsDesc* __restrict__ descs,
+__global__ void __launch_bounds__(DIGIT_THREADS) split_rows_kernel(const SplitRowsDesc* __restrict__ descs,
                                                          const WorkItem* __restrict__ items, int nitems,
                                                          const double* __restrict__ src_base, char* __restrict__ ws) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (warp >= nitems) return;
-    split_rows_item<true>(descs, items[warp], src_base, ws);
+    if (blockIdx.x < nitems) split_rows_item<true>(descs, items[blockIdx.x], src_base, ws);
 }
 
 // Rows q of the GEMM1 A operand: A[q][k] = [p+q]^(0) of primitive quartet (kp, kq) with
@@ -363,15 +365,16 @@ __global__ void __launch_bounds__(256) split_rows_kernel(const SplitRowsDesc* __
 // within the pair's block, which every group does when K_bra = 1.
 __device__ const uint16_t* g_gidx;
 
-// One split_r item (item.q = quartet, item.a = r0), by one warp.
+// One warp's 8 rows from item.a + 8 warp of a split_r item (item.q = quartet).
 __device__ __forceinline__ void split_r_item(const DQuartet* __restrict__ qd, const SplitQuartet* __restrict__ sq,
                                              const WorkItem& it, const double* __restrict__ wsd,
                                              char* __restrict__ ws) {
     const int lane = threadIdx.x & 31;
     const DQuartet q = qd[it.q];
     const SplitQuartet s = sq[it.q];
-    const int row = it.a + (lane >> 2), c8 = 8 * (lane & 3);
+    const int r0 = it.a + 8 * (threadIdx.x >> 5), row = r0 + (lane >> 2), c8 = 8 * (lane & 3);
     const int nrow = q.kket * q.nq, K = q.kbra * q.np;
+    if (r0 >= nrow) return;
     const bool live = row < nrow;
     const int kq = live ? row / q.nq : 0;
     const double* Rr = wsd + q.rr_off + (int64_t)kq * q.nr;
@@ -438,29 +441,27 @@ __device__ __forceinline__ void split_r_item(const DQuartet* __restrict__ qd, co
 
 // The operands of GEMM1 and the H operand of GEMM2 in one launch: split_r items ([p|q]^T rows,
 // issue-bound gathers) and split_rows items (H rows, load-latency bound) in alternating blocks,
-// so that the two kinds share the SMs.  8 warps (items) per block.
-__global__ void __launch_bounds__(256, 4) split_operands_kernel(const DQuartet* __restrict__ qd,
+// so that the two kinds share the SMs.  One item per block.
+__global__ void __launch_bounds__(DIGIT_THREADS, 8) split_operands_kernel(const DQuartet* __restrict__ qd,
                                                              const SplitQuartet* __restrict__ sq,
                                                              const WorkItem* __restrict__ items_r, int n_r,
                                                              const SplitRowsDesc* __restrict__ descs,
                                                              const WorkItem* __restrict__ items_w, int n_w,
                                                              const double* __restrict__ wsd, char* __restrict__ ws) {
-    const int nb_r = (n_r + 7) / 8, nb_w = (n_w + 7) / 8, m = min(nb_r, nb_w);
+    const int m = min(n_r, n_w);
     const int b = blockIdx.x;
     int kind, idx;  // kind 0: split_r, 1: split_rows
     if (b < 2 * m) {
         kind = b & 1;
         idx = b >> 1;
     } else {
-        kind = nb_r > nb_w ? 0 : 1;
+        kind = n_r > n_w ? 0 : 1;
         idx = m + (b - 2 * m);
     }
-    const int w = idx * 8 + (threadIdx.x >> 5);
-    if (kind == 0) {
-        if (w < n_r) split_r_item(qd, sq, items_r[w], wsd, ws);
-    } else {
-        if (w < n_w) split_rows_item<false>(descs, items_w[w], wsd, ws);  // H rows: fixed = 1
-    }
+    if (kind == 0)
+        split_r_item(qd, sq, items_r[idx], wsd, ws);
+    else
+        split_rows_item<false>(descs, items_w[idx], wsd, ws);  // H rows: fixed = 1
 }
 
 // ------------------------------------------------------------------ tcgen05 GEMM
@@ -789,18 +790,16 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 cudaError_t launch_split_rows(const SplitRowsDesc* descs, const WorkItem* items, int nitems, const double* src_base,
                               char* ws, cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
-    const int warps_per_block = 8;
-    split_rows_kernel<<<(nitems + warps_per_block - 1) / warps_per_block, 32 * warps_per_block, 0, st>>>(
-        descs, items, nitems, src_base, ws);
+    split_rows_kernel<<<nitems, DIGIT_THREADS, 0, st>>>(descs, items, nitems, src_base, ws);
     return cudaGetLastError();
 }
 
 cudaError_t launch_split_operands(const DQuartet* qd, const SplitQuartet* sq, const WorkItem* items_r, int n_r,
                                   const SplitRowsDesc* descs, const WorkItem* items_w, int n_w, const double* wsd,
                                   char* ws, cudaStream_t st) {
-    const int nb = (n_r + 7) / 8 + (n_w + 7) / 8;
+    const int nb = n_r + n_w;
     if (nb <= 0) return cudaSuccess;
-    split_operands_kernel<<<nb, 256, 0, st>>>(qd, sq, items_r, n_r, descs, items_w, n_w, wsd, ws);
+    split_operands_kernel<<<nb, DIGIT_THREADS, 0, st>>>(qd, sq, items_r, n_r, descs, items_w, n_w, wsd, ws);
     return cudaGetLastError();
 }
 

@@ -23,6 +23,10 @@ constexpr int SPLIT_EXP_NONE = -(1 << 29);
 // trim = split_trim(N) rows in all.  (A operands keep whole tiles of SPLIT_TA rows: SPLIT_NO_TRIM.)
 __host__ __device__ inline int split_trim(int N) { return (N + 7) / 8 * 8; }
 constexpr int SPLIT_NO_TRIM = 1 << 30;
+// Rows of one work item of the digit kernels: 4 warps of 8 rows, those past the operand's rows idle
+// (with 8 warps the idle ones cost 2 % of the digit stage).  One item per 32 rows instead of one per 8
+// takes 7 MB of work lists off each 4,096-quartet (ii|ii) call.
+constexpr int SPLIT_ITEM_ROWS = 32;
 
 // One matrix whose rows are split: src at (double*)base + src_off, row stride ld.  Before
 // splitting, column k is multiplied by 2^(shift_sign * shift[k]) (exact; shift_off < 0: none).
@@ -111,7 +115,7 @@ __host__ __device__ inline int64_t split_dig_bytes_b(int rows, int K) {
 cudaError_t init_split_kernels(const int* host_tuv);
 cudaError_t launch_split_rows(const SplitRowsDesc* descs, const WorkItem* items, int nitems, const double* src_base,
                               char* ws, cudaStream_t st);
-// split_r items and split_rows items in one launch (8 items per block, kinds alternating)
+// split_r items and split_rows items in one launch (one per block, kinds alternating)
 cudaError_t launch_split_operands(const DQuartet* qd, const SplitQuartet* sq, const WorkItem* items_r, int n_r,
                                   const SplitRowsDesc* descs, const WorkItem* items_w, int n_w, const double* wsd,
                                   char* ws, cudaStream_t st);

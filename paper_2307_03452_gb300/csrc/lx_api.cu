@@ -1065,12 +1065,12 @@ int enqueue_batch(const PlannedBatch& B, const char* head_src, const std::vector
             return cuda_fail(e);
         if ((e = tm.end(LX_STAGE_PAIR, matrix + axial)) != cudaSuccess) return cuda_fail(e);
         if ((e = tm.begin()) != cudaSuccess) return cuda_fail(e);
-        if ((e = launch_boys_r(d_q, d_pairs, d_ibr, (int)P.items_br.size(), P.br_lmax, ws, status, st)) !=
+        if ((e = launch_boys_r(d_q, d_pairs, d_ibr, (int)P.items_br.size(), P.br_lmax, ws, st)) !=
                 cudaSuccess ||
             (e = launch_axial_boys(d_axq, d_axp, ax(P.off_ait), (int)P.ax_it.size(), ws, st)) != cudaSuccess ||
             (e = launch_axial_wigner(d_axq, ax(P.off_ait), (int)P.ax_it.size(), P.ax_lmax, ws, st)) != cudaSuccess)
             return cuda_fail(e);
-        if ((e = tm.end(LX_STAGE_BOYS_R, matrix + 2 * axial)) != cudaSuccess) return cuda_fail(e);
+        if ((e = tm.end(LX_STAGE_BOYS_R, 2 * matrix + 2 * axial)) != cudaSuccess) return cuda_fail(e);
         if (split) {
             auto at = [&](size_t off) { return base + off; };
             const SplitRowsDesc* d_srd = reinterpret_cast<const SplitRowsDesc*>(at(P.off_srd));

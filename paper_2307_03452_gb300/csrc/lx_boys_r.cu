@@ -98,10 +98,50 @@ __device__ void hermite_r_warp(int L, double X, double Y, double Z, const double
 
 constexpr int BR_WARPS = 4;  // warps per CTA of the stage entry point
 
-// One single-warp CTA per primitive quartet: item.q = quartet, item.a = kpq = kp * kket + kq.
+// One more power: (h, l) = x^n as an unevaluated sum -> x^(n+1), so that the chain rounds once, at
+// h + l.
+__device__ inline void power_step(double x, double& h, double& l) {
+    const double p = h * x;
+    l = (__double2hiint(p) & 0x7FF00000) == 0x7FF00000 ? 0.0 : fma(l, x, fma(h, x, -p));
+    h = p;
+}
+
+// [0]^(m) = (-2 rho)^m 2 pi^{5/2} / (zeta_p zeta_q sqrt(zeta_p + zeta_q)) F_m(T), m = 0..L, of each
+// primitive quartet (item.q = quartet, item.a = kpq = kp kket + kq), into the first L + 1 entries of
+// its [r]^(0).  One thread per primitive quartet: the Boys recursion is serial, with a division
+// per order, so in the recursion kernel's warp it took as many FP64 issues for one quartet as here
+// for 32.
+constexpr int BASE_THREADS = 64;
+__global__ void __launch_bounds__(BASE_THREADS) boys_base_kernel(const DQuartet* __restrict__ qd,
+                                                                 const DPair* __restrict__ pairs,
+                                                                 const WorkItem* __restrict__ items, int nitems,
+                                                                 double* __restrict__ ws) {
+    const int i = blockIdx.x * BASE_THREADS + threadIdx.x;
+    if (i >= nitems) return;
+    const WorkItem it = items[i];
+    const DQuartet q = qd[it.q];
+    const int kp = it.a / q.kket, kq = it.a - kp * q.kket;
+    const double* ib = ws + pairs[q.pb].info_off + 4 * (int64_t)kp;
+    const double* ik = ws + pairs[q.pk].info_off + 4 * (int64_t)kq;
+    const double zp = ib[0], zq = ik[0];
+    const double X = ib[1] - ik[1], Y = ib[2] - ik[2], Z = ib[3] - ik[3];
+    const double rho = zp * zq / (zp + zq);
+    double F[LTOT + 1];
+    boys_eval(q.L, rho * (X * X + Y * Y + Z * Z), F);
+    const double pref = 2.0 * PI * PI * sqrt(PI) / (zp * zq * sqrt(zp + zq));
+    double* out = ws + q.rr_off + (int64_t)it.a * q.nr;
+    double h = 1.0, l = 0.0;
+    for (int m = 0; m <= q.L; ++m) {
+        const double pw = h + l;
+        out[m] = F[m] * ((m & 1) ? -pref * pw : pref * pw);
+        power_step(2.0 * rho, h, l);
+    }
+}
+
+// One single-warp CTA per primitive quartet: item.q = quartet, item.a = kpq = kp * kket + kq.  Its
+// [0]^(m) are the first L + 1 entries of its [r]^(0) on entry.
 __global__ void __launch_bounds__(32) boys_r_kernel(const DQuartet* __restrict__ qd, const DPair* __restrict__ pairs,
-                                                    const WorkItem* __restrict__ items, double* __restrict__ ws,
-                                                    unsigned* status) {
+                                                    const WorkItem* __restrict__ items, double* __restrict__ ws) {
     extern __shared__ double smem[];
     const int lane = threadIdx.x & 31;
     const WorkItem it = items[blockIdx.x];
@@ -110,30 +150,16 @@ __global__ void __launch_bounds__(32) boys_r_kernel(const DQuartet* __restrict__
     const int nr = q.nr;
     double* R = smem;
     double* B = R + nr;
+    double* out = ws + q.rr_off + (int64_t)kpq * nr;
+    if (lane <= q.L) B[lane] = out[lane];
     const int kp = kpq / q.kket, kq = kpq - kp * q.kket;
     const DPair pb = pairs[q.pb], pk = pairs[q.pk];
     const double* ib = ws + pb.info_off + 4 * (int64_t)kp;
     const double* ik = ws + pk.info_off + 4 * (int64_t)kq;
-    const double zp = ib[0], zq = ik[0];
     const double X = ib[1] - ik[1], Y = ib[2] - ik[2], Z = ib[3] - ik[3];
-    const double rho = zp * zq / (zp + zq);
-    const double T = rho * (X * X + Y * Y + Z * Z);
-    if (lane == 0) boys_eval(q.L, T, B);
-    __syncwarp();
-    // [0]^(m) = (-2 rho)^m 2 pi^{5/2} / (zeta_p zeta_q sqrt(zeta_p + zeta_q)) F_m(T), one m per lane
-    scale_base(q.L, rho, 2.0 * PI * PI * sqrt(PI) / (zp * zq * sqrt(zp + zq)), B, lane);
     __syncwarp();
     hermite_r_warp(q.L, X, Y, Z, B, R, lane);
-    double* out = ws + q.rr_off + (int64_t)kpq * nr;
     for (int r = lane; r < nr; r += 32) out[r] = R[r];
-}
-
-// One more power: (h, l) = x^n as an unevaluated sum -> x^(n+1), so that the chain rounds once, at
-// h + l.
-__device__ inline void power_step(double x, double& h, double& l) {
-    const double p = h * x;
-    l = (__double2hiint(p) & 0x7FF00000) == 0x7FF00000 ? 0.0 : fma(l, x, fma(h, x, -p));
-    h = p;
 }
 
 // Axial form (lx_axial.cu): 8 lanes per primitive quartet (item.q, item.a = kp kket + kq) write
@@ -315,11 +341,14 @@ cudaError_t init_boys_table(const double* host_table) {
 }
 
 cudaError_t launch_boys_r(const DQuartet* qd, const DPair* pairs, const WorkItem* items, int nitems, int lmax,
-                          double* ws, unsigned* status, cudaStream_t st) {
+                          double* ws, cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
     if (lmax < 0 || lmax > LTOT) return cudaErrorInvalidValue;
+    boys_base_kernel<<<(nitems + BASE_THREADS - 1) / BASE_THREADS, BASE_THREADS, 0, st>>>(qd, pairs, items, nitems, ws);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     const size_t smem = sizeof(double) * (pyr(lmax) + LTOT + 1);
-    boys_r_kernel<<<nitems, 32, smem, st>>>(qd, pairs, items, ws, status);
+    boys_r_kernel<<<nitems, 32, smem, st>>>(qd, pairs, items, ws);
     return cudaGetLastError();
 }
 

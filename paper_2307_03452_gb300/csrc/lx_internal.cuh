@@ -102,7 +102,7 @@ cudaError_t launch_jk_direct(const DQuartet* qd, const DPair* pairs, const DShel
                              double* K, cudaStream_t st);
 cudaError_t init_jk_kernels();
 cudaError_t launch_boys_r(const DQuartet* qd, const DPair* pairs, const WorkItem* items, int nitems, int lmax,
-                          double* ws, unsigned* status, cudaStream_t st);  // lmax: largest L of the items
+                          double* ws, cudaStream_t st);  // lmax: largest L of the items
 // items grouped by tile shape: counts[v] items of shape v, in shape order; counters[v] is the
 // zero-initialised work counter of shape v's launch
 cudaError_t launch_gemm1(const DQuartet* qd, const DPair* pairs, const WorkItem* items, const int* counts, double* ws,

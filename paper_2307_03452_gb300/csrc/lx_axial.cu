@@ -58,10 +58,11 @@ __constant__ AxDev c_ax;
 // Real rotation blocks of a rotation about y by beta, (c, s) = (cos, sin) of the angle of
 // R = [[c, 0, s], [0, 1, 0], [-s, 0, c]] (Y_l(R v) = D Y_l(v)), for l <= lmax: C[ax_co(l) + m'(l+1) + m]
 // between cosine and S[ax_so(l) + (m'-1) l + m-1] between sine functions.  One chain in l per
-// (m' >= m >= 0), spread over `step` threads; pw: 4 AX_LP + 2 doubles of shared scratch, filled here.
-// The caller synchronises before pw is reused.
-template <typename Sync>
-__device__ void wigner_y(int lmax, double c, double s, double* C, double* S, double* pw, int t0, int step, Sync sync) {
+// (m' >= m >= 0), from the powers pw of cos and sin of the half angle.
+constexpr int WIG_NP = 2 * AX_LP + 1;
+__host__ __device__ inline int wigner_chains(int lmax) { return (lmax + 1) * (lmax + 2) / 2; }
+// Powers 0 .. 2 lmax of the half angle's cos (which = 0) or sin (1) into pw[which WIG_NP ...], one thread.
+__device__ inline void wigner_powers(int lmax, double c, double s, int which, double* pw) {
     double ch = sqrt(fmax(0.0, 0.5 * (1.0 + c))), sh;
     if (ch > 0.5) {
         sh = s / (2.0 * ch);
@@ -69,71 +70,65 @@ __device__ void wigner_y(int lmax, double c, double s, double* C, double* S, dou
         sh = sqrt(fmax(0.0, 0.5 * (1.0 - c)));
         ch = s / (2.0 * sh);
     }
-    constexpr int NP = 2 * AX_LP + 1;
-    if (t0 < 2) {  // powers of cos, sin of the half angle
-        const double b = t0 ? sh : ch;
-        double p = 1.0;
-        for (int i = 0; i <= 2 * lmax; ++i) {
-            pw[t0 * NP + i] = p;
-            p *= b;
-        }
+    const double b = which ? sh : ch;
+    double p = 1.0;
+    for (int i = 0; i <= 2 * lmax; ++i) {
+        pw[which * WIG_NP + i] = p;
+        p *= b;
     }
-    sync();
-    const int nch = (lmax + 1) * (lmax + 2) / 2;
-    for (int i = t0; i < nch; i += step) {
-        int mp = (int)((sqrtf(8.0f * i + 1.0f) - 1.0f) * 0.5f);
-        while ((mp + 1) * (mp + 2) / 2 <= i) ++mp;
-        while (mp * (mp + 1) / 2 > i) --mp;
-        const int m = i - mp * (mp + 1) / 2;
-        const double w0 = __ldg(c_ax.wig0 + i);
-        // (-1)^(m' + m) d_{m',m} and (-1)^(m' + m) d_{m',-m}
-        double x = w0 * pw[mp + m] * pw[NP + mp - m], y = w0 * pw[mp - m] * pw[NP + mp + m], xp = 0.0, yp = 0.0;
-        const double flip = (mp + m) & 1 ? -1.0 : 1.0, par = m & 1 ? -1.0 : 1.0;
-        const double* w = c_ax.wig + (size_t)i * AX_NL * 3;
-        for (int l = mp; l <= lmax; ++l) {
-            double vc, vs = 0.0;
-            if (m) {
-                vc = fma(par, y, x);
-                vs = fma(-par, y, x);
-            } else {
-                vc = mp ? 1.4142135623730951 * x : x;
-            }
-            double* Cl = C + ax_co(l);
-            Cl[mp * (l + 1) + m] = vc;
-            Cl[m * (l + 1) + mp] = mp == m ? vc : flip * vc;
-            if (m) {
-                double* Sl = S + ax_so(l);
-                Sl[(mp - 1) * l + m - 1] = vs;
-                Sl[(m - 1) * l + mp - 1] = mp == m ? vs : flip * vs;
-            }
-            const double a = __ldg(w + 3 * l), b = __ldg(w + 3 * l + 1), cc = __ldg(w + 3 * l + 2);
-            const double xn = fma(a * (c - b), x, -cc * xp), yn = fma(a * (c + b), y, -cc * yp);
-            xp = x;
-            yp = y;
-            x = xn;
-            y = yn;
+}
+__device__ inline void wigner_chain(int i, int lmax, double c, const double* pw, double* C, double* S) {
+    int mp = (int)((sqrtf(8.0f * i + 1.0f) - 1.0f) * 0.5f);
+    while ((mp + 1) * (mp + 2) / 2 <= i) ++mp;
+    while (mp * (mp + 1) / 2 > i) --mp;
+    const int m = i - mp * (mp + 1) / 2;
+    const double w0 = __ldg(c_ax.wig0 + i);
+    // (-1)^(m' + m) d_{m',m} and (-1)^(m' + m) d_{m',-m}
+    double x = w0 * pw[mp + m] * pw[WIG_NP + mp - m], y = w0 * pw[mp - m] * pw[WIG_NP + mp + m], xp = 0.0, yp = 0.0;
+    const double flip = (mp + m) & 1 ? -1.0 : 1.0, par = m & 1 ? -1.0 : 1.0;
+    const double* w = c_ax.wig + (size_t)i * AX_NL * 3;
+    for (int l = mp; l <= lmax; ++l) {
+        double vc, vs = 0.0;
+        if (m) {
+            vc = fma(par, y, x);
+            vs = fma(-par, y, x);
+        } else {
+            vc = mp ? 1.4142135623730951 * x : x;
         }
+        double* Cl = C + ax_co(l);
+        Cl[mp * (l + 1) + m] = vc;
+        Cl[m * (l + 1) + mp] = mp == m ? vc : flip * vc;
+        if (m) {
+            double* Sl = S + ax_so(l);
+            Sl[(mp - 1) * l + m - 1] = vs;
+            Sl[(m - 1) * l + mp - 1] = mp == m ? vs : flip * vs;
+        }
+        const double a = __ldg(w + 3 * l), b = __ldg(w + 3 * l + 1), cc = __ldg(w + 3 * l + 2);
+        const double xn = fma(a * (c - b), x, -cc * xp), yn = fma(a * (c + b), y, -cc * yp);
+        xp = x;
+        yp = y;
+        x = xn;
+        y = yn;
     }
 }
 
 // Full blocks (2l+1)^2, l <= L, of the rotation Rz(a) Ry Rz(b): pa, pb = cos, sin of m a, m b; C, S the
-// Y blocks; D[ax_do(l) + (l + m')(2l+1) + l + m], sine functions at m < 0.  Spread over `step` threads.
+// Y blocks; D[ax_do(l) + (l + m')(2l+1) + l + m], sine functions at m < 0.  The entries of all blocks
+// are spread over `step` threads.
 __device__ __forceinline__ void full_blocks(int L, const double* pa, const double* pb, const double* C,
                                             const double* S, double* D, int t0, int step) {
-    for (int l = 0; l <= L; ++l) {
-        const int w = 2 * l + 1;
+    int l = 0;
+    for (int i = t0; i < ax_co(L + 1); i += step) {
+        while (i >= ax_co(l + 1)) ++l;
+        const int w = 2 * l + 1, e = i - ax_co(l), mp = e / (l + 1), m = e - mp * (l + 1);
         double* Dl = D + ax_do(l);
-        const double *Cl = C + ax_co(l), *Sl = S + ax_so(l);
-        for (int e = t0; e < (l + 1) * (l + 1); e += step) {
-            const int mp = e / (l + 1), m = e - mp * (l + 1);
-            const double c = Cl[e], s = mp && m ? Sl[(mp - 1) * l + m - 1] : 0.0;
-            const double ca = pa[2 * mp], sa = pa[2 * mp + 1], cb = pb[2 * m], sb = pb[2 * m + 1];
-            const double cc = c * cb, cs = c * sb, sc = -s * sb, ss = s * cb;
-            Dl[(l + mp) * w + l + m] = ca * cc + sa * sc;
-            if (m) Dl[(l + mp) * w + l - m] = ca * cs + sa * ss;
-            if (mp) Dl[(l - mp) * w + l + m] = ca * sc - sa * cc;
-            if (mp && m) Dl[(l - mp) * w + l - m] = ca * ss - sa * cs;
-        }
+        const double c = C[i], s = mp && m ? S[ax_so(l) + (mp - 1) * l + m - 1] : 0.0;
+        const double ca = pa[2 * mp], sa = pa[2 * mp + 1], cb = pb[2 * m], sb = pb[2 * m + 1];
+        const double cc = c * cb, cs = c * sb, sc = -s * sb, ss = s * cb;
+        Dl[(l + mp) * w + l + m] = ca * cc + sa * sc;
+        if (m) Dl[(l + mp) * w + l - m] = ca * cs + sa * ss;
+        if (mp) Dl[(l - mp) * w + l + m] = ca * sc - sa * cc;
+        if (mp && m) Dl[(l - mp) * w + l - m] = ca * ss - sa * cs;
     }
 }
 
@@ -195,8 +190,10 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
                 c = cn;
             }
         }
-        wigner_y(lm, n[2], -st, rot + AX_ROT_C, rot + AX_ROT_C + ax_co(lm + 1), pw, tid, AXP_THREADS,
-                 [] { __syncthreads(); });
+        if (tid < 2) wigner_powers(lm, n[2], -st, tid, pw);
+        __syncthreads();
+        for (int i = tid; i < wigner_chains(lm); i += AXP_THREADS)
+            wigner_chain(i, lm, n[2], pw, rot + AX_ROT_C, rot + AX_ROT_C + ax_co(lm + 1));
     }
     // z expansion, one warp, lanes over v
     if (warp == 0) {
@@ -280,24 +277,28 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
 
 // ------------------------------------------------------------------ rotation blocks
 
-// One CTA of two warps per primitive quartet (item.q, item.a = kp kket + kq): from the angles of
-// the table, cos and sin of M gamma and the Y blocks of the bra rotation (warp 0), the Y blocks of
-// the rotation PQ -> CD (warp 1), then the latter's full blocks (or its factors).
-constexpr int AXW_THREADS = 64;
-__global__ void __launch_bounds__(AXW_THREADS) axial_wigner_kernel(const AxQuartet* __restrict__ qd,
-                                                                   const WorkItem* __restrict__ items, int lmax,
-                                                                   double* __restrict__ ws) {
+// One CTA per primitive quartet (item.q, item.a = kp kket + kq): from the angles of the table, cos
+// and sin of M gamma, the Y blocks of the bra rotation and of the rotation PQ -> CD, whose chains
+// share the lanes, then the latter's full blocks (or its factors).  One warp where it holds all
+// chains at once (L <= 4 on both sides), else two: latency of a few dependent steps bounds it (tables
+// of 1,024 contracted (ff|ff), K = 5, 2.61 ms with two warps whose sides took turns, 2.13 so).
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) axial_wigner_kernel(const AxQuartet* __restrict__ qd,
+                                                               const WorkItem* __restrict__ items, int lmax,
+                                                               double* __restrict__ ws) {
     extern __shared__ double sm[];
-    __shared__ double pw[2][4 * AX_LP + 2], ph[4 * AX_NL];  // ph: cos, sin of m a, then of m b: 4 (Lk + 1)
+    __shared__ double pw[2][2 * WIG_NP], ph[4 * AX_NL];  // ph: cos, sin of m a, then of m b: 4 (Lk + 1)
     double* C = sm;
     double* S = C + ax_co(lmax + 1);
     const WorkItem it = items[blockIdx.x];
     const AxQuartet q = qd[it.q];
     double* tab = ws + q.tab_off + (int64_t)it.a * q.tab_stride;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, Lb = q.Lb, Lk = q.Lk;
-    auto sync = [] { __syncwarp(); };
-    if (tid == 31 || tid >= 62) {  // phases: gamma (thread 31), a and b of the ket rotation
-        const int w = tid == 31 ? 0 : tid - 61;
+    const int tid = threadIdx.x, Lb = q.Lb, Lk = q.Lk;
+    if (tid < 4) {  // powers for the bra (0, 1) and ket rotation (2, 3)
+        const int side = tid >> 1;
+        wigner_powers(side ? Lk : Lb, tab[4 * side], -tab[4 * side + 1], tid & 1, pw[side]);
+    } else if (tid < 7) {  // phases: gamma, then a and b of the ket rotation
+        const int w = tid - 4;
         const double c0 = tab[w == 0 ? 2 : 4 + 2 * w], s0 = tab[w == 0 ? 3 : 5 + 2 * w];
         double* o = w == 0 ? tab + ax_t_cg(Lb, Lk) : ph + 2 * (Lk + 1) * (w - 1);
         const int n = w == 0 ? Lb : Lk;
@@ -310,21 +311,23 @@ __global__ void __launch_bounds__(AXW_THREADS) axial_wigner_kernel(const AxQuart
             c = cn;
         }
     }
-    if (warp == 0) {
-        double* tc = tab + ax_t_c(Lb, Lk);
-        wigner_y(Lb, tab[0], -tab[1], tc, tc + ax_co(Lb + 1), pw[0], lane, 32, sync);
-    } else {
-        wigner_y(Lk, tab[4], -tab[5], C, S, pw[1], lane, 32, sync);
+    __syncthreads();
+    const int nb = wigner_chains(Lb), nk = wigner_chains(Lk);
+    double* tc = tab + ax_t_c(Lb, Lk);
+    for (int i = tid; i < nb + nk; i += THREADS) {
+        const bool ket = i >= nb;
+        wigner_chain(ket ? i - nb : i, ket ? Lk : Lb, tab[ket ? 4 : 0], pw[ket], ket ? C : tc,
+                     ket ? S : tc + ax_co(Lb + 1));
     }
     __syncthreads();
     double* D = tab + ax_t_d(Lb, Lk);
     if (q.full) {
-        full_blocks(Lk, ph, ph + 2 * (Lk + 1), C, S, D, tid, AXW_THREADS);
+        full_blocks(Lk, ph, ph + 2 * (Lk + 1), C, S, D, tid, THREADS);
     } else {
         const int nc = ax_co(Lk + 1), ns = ax_so(Lk + 1), np = 4 * (Lk + 1);
-        for (int i = tid; i < np; i += AXW_THREADS) D[i] = ph[i];
-        for (int i = tid; i < nc; i += AXW_THREADS) D[np + i] = C[i];
-        for (int i = tid; i < ns; i += AXW_THREADS) D[np + nc + i] = S[i];
+        for (int i = tid; i < np; i += THREADS) D[i] = ph[i];
+        for (int i = tid; i < nc; i += THREADS) D[np + i] = C[i];
+        for (int i = tid; i < ns; i += THREADS) D[np + nc + i] = S[i];
     }
 }
 
@@ -844,7 +847,10 @@ cudaError_t launch_axial_wigner(const AxQuartet* qd, const WorkItem* items, int 
                                 cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
     const size_t smem = sizeof(double) * (size_t)(ax_co(lmax + 1) + ax_so(lmax + 1));
-    axial_wigner_kernel<<<nitems, AXW_THREADS, smem, st>>>(qd, items, lmax, ws);
+    if (2 * wigner_chains(lmax) <= 32)
+        axial_wigner_kernel<32><<<nitems, 32, smem, st>>>(qd, items, lmax, ws);
+    else
+        axial_wigner_kernel<64><<<nitems, 64, smem, st>>>(qd, items, lmax, ws);
     return cudaGetLastError();
 }
 

@@ -314,6 +314,7 @@ size_t axial_quartet_bytes(const lx_shell* sh, const lx_quartet& q, int flags, b
 }
 
 // Parts of the ket primitives (AX_PART), as many as the quartet's room allows.
+size_t axial_room(const lx_shell* sh, const lx_quartet& q, int flags);
 int axial_split(const lx_shell* sh, const lx_quartet& q, int flags, bool full) {
     const lx_shell &a = sh[q.s[0]], &b = sh[q.s[1]], &c = sh[q.s[2]], &d = sh[q.s[3]];
     const bool solid = flags & LX_SOLID;
@@ -321,7 +322,7 @@ int axial_split(const lx_shell* sh, const lx_quartet& q, int flags, bool full) {
     const size_t block = 8 * (size_t)nfun(a.l, solid) * nfun(b.l, solid) * nfun(c.l, solid) * nfun(d.l, solid);
     const size_t nhalf = axial_tables().cls[ax_class_id(a.l, b.l, solid)].nhalf;
     const size_t per = block + (nhalf + AX_NR - 1) / AX_NR * sizeof(WorkItem);
-    const size_t room = quartet_bytes(sh, q, flags), used = axial_quartet_bytes(sh, q, flags, full) + 256;
+    const size_t room = axial_room(sh, q, flags), used = axial_quartet_bytes(sh, q, flags, full) + 256;
     const int want = std::min(kket, (prim + AX_PART - 1) / AX_PART);
     return used >= room ? 1 : std::max(1, std::min<int>(want, 1 + (int)((room - used) / per)));
 }
@@ -333,23 +334,30 @@ size_t axial_pair_bytes(const lx_shell* sh, int sa, int sb, int flags) {
     return sizeof(AxPair) + kab * sizeof(WorkItem) + 8 * (kab * (4 + c.nh) + ax_rot_size(std::max(a.l, b.l))) + 512;
 }
 
+// Workspace that a quartet's own data may take in the axial form: what the matrix form takes for it
+// and for its pairs, less the axial form's pairs (0 if they alone take more).
+size_t axial_room(const lx_shell* sh, const lx_quartet& q, int flags) {
+    const size_t has = quartet_bytes(sh, q, flags) + pair_bytes(sh, q.s[0], q.s[1], flags) + pair_bytes(sh, q.s[2], q.s[3], flags);
+    const size_t pairs = axial_pair_bytes(sh, q.s[0], q.s[1], flags) + axial_pair_bytes(sh, q.s[2], q.s[3], flags);
+    return has > pairs ? has - pairs : 0;
+}
+
 // How a quartet of the FP64 path is evaluated: 0 = matrix form, 1 = axial form with the
 // factors of the ket blocks in its tables, 2 = axial form with the full blocks.  A rule on its
 // class and contraction degrees alone, so that results do not depend on the batch, the chunk
 // or the workspace.  The matrix form stays for small classes, where it is the faster one
 // (AX_MIN_FMA), and where the axial form's tables (one per primitive quartet) would need more
-// workspace than the matrix form's [r]^(0) and [ab|q], which the workspace sizes are stated for.
+// workspace than the matrix form, which the workspace sizes are stated for.
 int axial_route(const lx_shell* sh, const lx_quartet& q, int flags) {
     if (flags & LX_PATH_SPLIT) return 0;
     const bool solid = flags & LX_SOLID;
     const int Lb = sh[q.s[0]].l + sh[q.s[1]].l, Lk = sh[q.s[2]].l + sh[q.s[3]].l;
     const int64_t nab = (int64_t)nfun(sh[q.s[0]].l, solid) * nfun(sh[q.s[1]].l, solid),
                   ncd = (int64_t)nfun(sh[q.s[2]].l, solid) * nfun(sh[q.s[3]].l, solid);
-    if (nab * pyr(Lk) * (pyr(Lb) + ncd) < (nab < AX_FEW_ROWS ? AX_MIN_FMA_FEW : AX_MIN_FMA)) return 0;
-    if (axial_pair_bytes(sh, q.s[0], q.s[1], flags) > pair_bytes(sh, q.s[0], q.s[1], flags) ||
-        axial_pair_bytes(sh, q.s[2], q.s[3], flags) > pair_bytes(sh, q.s[2], q.s[3], flags))
-        return 0;
-    const size_t room = quartet_bytes(sh, q, flags);
+    const int prim = sh[q.s[0]].nprim * sh[q.s[1]].nprim * sh[q.s[2]].nprim * sh[q.s[3]].nprim;
+    const bool few = nab < AX_FEW_ROWS || prim < AX_FEW_PRIM;
+    if (nab * pyr(Lk) * (pyr(Lb) + ncd) < (few ? AX_MIN_FMA : AX_MIN_FMA_K)) return 0;
+    const size_t room = axial_room(sh, q, flags);
     return axial_quartet_bytes(sh, q, flags, true) <= room ? 2 : axial_quartet_bytes(sh, q, flags, false) <= room;
 }
 
@@ -990,8 +998,9 @@ int plan_batch(const lx_shell* shells, int32_t nshell, const double* exps, const
         B.chunks.emplace_back();
         build_chunk(shells, quartets, chunks[c], pflags, B.head, shapes, pid, apid, B.chunks.back(), ov);
         if (B.head + B.chunks.back().total <= workspace_bytes) continue;
-        // a pair used by matrix-form and by axial quartets of one chunk is stored in both forms,
-        // which plan_chunks does not count: halve such a chunk
+        // plan_chunks counts the matrix form with every pair once: a pair stored in both forms, or
+        // tables that take the room of pairs which quartets share, may not fit.  Halve such a chunk
+        // (one quartet always fits)
         Chunk half = chunks[c];
         if (half.q_end - half.q_begin < 2) return LX_ERR_WORKSPACE;
         half.q_begin += (half.q_end - half.q_begin) / 2;

@@ -51,6 +51,15 @@ def test_classes(cls, solid):
 
 
 @pytest.mark.parametrize("solid", [True, False])
+@pytest.mark.parametrize("cls", [(2, 2, 2, 2), (3, 2, 2, 1), (3, 1, 3, 1), (2, 2, 2, 1), (2, 1, 3, 3), (5, 0, 4, 1)])
+def test_contracted_classes_near_the_line(cls, solid):
+    # K = 1..5: quartets of one batch on both sides of the line between the two forms, which share pairs
+    basis, quartets = inputs.uniform_class(cls, 6, 65, cube=1.5, exps=(0.2, 5.0), kmin=1, kmax=5)
+    q = np.asarray(quartets)
+    check(basis, np.concatenate([q, np.hstack([q[:, :2], np.roll(q[:, 2:], 1, 0)])]), solid)
+
+
+@pytest.mark.parametrize("solid", [True, False])
 def test_directions_without_azimuth(solid):
     # A, B, C, D on the z axis (either order), on the x axis, bra along z and ket along x, tiny
     # tilts of 1e-9 and 1e-170, A = B, C = D, all coincident, P = Q with A != B

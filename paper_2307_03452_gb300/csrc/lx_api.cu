@@ -765,7 +765,7 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
             // columns scaled into (-1, 1): one pass, e = 0 per row
             P.srd.push_back(
                 SplitRowsDesc{0, 0, 0, 0, k, pr.nrow, k, tb, split_nkb(k), -1, 1, 0, nd, split_trim(pr.nrow)});
-            // digit kernels: one item (a CTA) per 64 consecutive rows, written up to nrow rounded
+            // digit kernels: one item (a CTA) per SPLIT_ITEM_ROWS rows, written up to nrow rounded
             // to 8 (the GEMMs drop the output columns of B rows past nrow)
             for (int row = 0; row < pr.nrow; row += SPLIT_ITEM_ROWS) P.items_sB.push_back({p, row, 0, 0});
         }

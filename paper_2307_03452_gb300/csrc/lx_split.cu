@@ -10,8 +10,8 @@
 // accumulator, drained into 64-bit integers every SPLIT_SEG_KB K blocks so that every FP32
 // partial sum stays an integer of magnitude <= 2^24 (exact), and the 64-bit sum is converted
 // to FP64 once (the lowest BETA bits of the last diagonal are rounded off to keep the sum
-// clear of 64-bit overflow).  FP64 arithmetic, which is scarce on this GPU, is used for none
-// of it: the splitting works on the bit patterns of the FP64 inputs.
+// clear of 64-bit overflow).  FP64 arithmetic, which is scarce on this GPU, is used for one
+// instruction per value, which rounds it to its fixed-point place.
 //
 // Kernels:
 //   split_operands_kernel  rows q of the [p|q] operand gathered from [r]^(0), and the H
@@ -161,9 +161,6 @@ __device__ inline void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.alig
 
 // ------------------------------------------------------------------ splitting
 
-// Biased exponent field of an FP64 value (0 for zero / subnormal).
-__device__ inline int exp_field(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); }
-
 // x * 2^s by exponent arithmetic (exact; underflow to zero).
 __device__ inline double scale2(double x, int s) {
     const long long bits = __double_as_longlong(x);
@@ -176,19 +173,18 @@ __device__ inline double scale2(double x, int s) {
 }
 
 // Biased exponent field of x 2^s: 0 if x is zero or subnormal or x 2^s underflows the normal
-// range (the value scale2 would give), capped at 2047.
+// range, capped at 2047.
 __device__ inline int exp_field_scaled(double x, int s) {
-    const int ex = exp_field(x);
+    const int ex = (__double2hiint(x) >> 20) & 0x7FF;
     return ex > 0 ? min(max(ex + s, 0), 2047) : 0;
 }
 
-// q = round(x 2^s 2^(W - e)) for |x 2^s| < 2^e, from the bit pattern (no FP64 arithmetic);
-// equal to the rounding of scale2(x, s), so a scaled value that underflows gives 0.
+// q = round(x 2^s 2^(W - e)), ties away from zero, for |x 2^s| < 2^e, from the bit pattern (no FP64
+// arithmetic); 0 where x or x 2^s is below the normal range.
 __device__ inline long long fixed_of(double x, int s, int e) {
     const long long bits = __double_as_longlong(x);
-    const int ex = (int)((bits >> 52) & 0x7FF);
-    const int ne = ex + s;
-    if (ex == 0 || ne <= 0) return 0;  // zero or subnormal: below any row scale that matters
+    const int ex = (int)((bits >> 52) & 0x7FF), ne = ex + s;
+    if (ex == 0 || ne <= 0) return 0;  // below any row scale that matters
     const long long mant = (bits & 0xFFFFFFFFFFFFFll) | (1ll << 52);
     const int rs = 1075 - ne - SPLIT_W + e;  // right shift, >= 53 - W > 0
     long long q = 0;
@@ -197,257 +193,275 @@ __device__ inline long long fixed_of(double x, int s, int e) {
 }
 
 // The digits of q (|q| <= 2^48), most significant first, balanced: |d_0| <= 2^BETA and
-// -2^(BETA-1) <= d_s < 2^(BETA-1) for s > 0.  Adding B = 2^(BETA-1) (1 + 256 + ... + 256^4)
-// makes the five low digits plain bytes: byte j of y = q + B is d_(5-j) + 128, with every
-// carry done by the one 64-bit add, and d_0 = floor(y / 2^40).  Each byte becomes an FP32 bit
+// -2^(BETA-1) <= d_s < 2^(BETA-1) for s > 0.  `bits` are those of q + B + 1.5 2^52 with B = 2^(BETA-1)
+// (1 + 256 + ... + 256^4): byte j of q + B is d_(5-j) + 128, with every carry done by the one
+// addition, and d_0 = floor((q + B) / 2^40).  Each byte becomes an FP32 bit
 // pattern with one byte permute: [byte, 0, 0x40, 0x4B] is the FP32 number 1.5 2^23 + byte,
 // so subtracting 1.5 2^23 + 128 leaves d exactly.  A digit has at most 8 significant bits,
 // so its BF16 pattern is the upper half of its FP32 pattern.
 static_assert(SPLIT_NSLICE == 6 && SPLIT_BETA == 8, "digit extraction assumes 6 digits of 8 bits");
-__device__ inline void digits_of(long long q, uint32_t (&f)[SPLIT_NSLICE]) {
-    const long long y = q + 0x8080808080ll;
-    const uint32_t lo = (uint32_t)y;
-    const int hi = (int)(y >> 32);
+constexpr long long DIGIT_BIAS = 0x4338008080808080ll;  // the bits of B + 1.5 2^52
+__device__ inline void digits_of(long long bits, uint32_t (&f)[SPLIT_NSLICE]) {
+    const uint32_t lo = (uint32_t)bits, hi = (uint32_t)(bits >> 32);
     constexpr uint32_t MAGIC = 0x4B400000u;  // 1.5 2^23
     constexpr float BIAS = 12582912.0f + 128.0f;
     f[5] = __float_as_uint(__uint_as_float(__byte_perm(lo, MAGIC, 0x7650)) - BIAS);
     f[4] = __float_as_uint(__uint_as_float(__byte_perm(lo, MAGIC, 0x7651)) - BIAS);
     f[3] = __float_as_uint(__uint_as_float(__byte_perm(lo, MAGIC, 0x7652)) - BIAS);
     f[2] = __float_as_uint(__uint_as_float(__byte_perm(lo, MAGIC, 0x7653)) - BIAS);
-    f[1] = __float_as_uint(__uint_as_float(__byte_perm((uint32_t)hi, MAGIC, 0x7650)) - BIAS);
-    f[0] = __float_as_uint(__int_as_float((int)MAGIC + (hi >> 8)) - 12582912.0f);
+    f[1] = __float_as_uint(__uint_as_float(__byte_perm(hi, MAGIC, 0x7650)) - BIAS);
+    f[0] = __float_as_uint(__int_as_float((int)MAGIC - 0x433800 + (int)(hi >> 8)) - 12582912.0f);
 }
 
-// Digits of 8 consecutive values (k0 .. k0+7, k0 a multiple of 8) of one row, written as one
-// 16-byte store per slice (one row of a core matrix), for the first nd slices.
-__device__ inline int64_t dig_index(int row, int k, int s, int T, int nkb, int trim);
-__device__ inline void store_digit_group(__nv_bfloat16* dig, int row, int k0, int T, int nkb, int trim,
-                                         const long long (&q)[8], int nd) {
+// Digits of 8 consecutive values v (scaled by 2^sh, then below 2^e) of one row, written as one 16-byte
+// store per slice (one row of a core matrix), `slice` elements apart, for the first nd slices.
+// q = fixed_of(v, sh, e) comes from one fused multiply-add, which rounds v 2^(sh + W - e) into the low
+// bits of B + 1.5 2^52, for some 20 integer instructions (digit stages of 4,096 (ii|ii): 6.24 against
+// 6.70 ms).  It is the same q for every v: setting v's lowest bit (the scaled value drops at least
+// 53 - W = 5 bits) makes the hardware's ties to even ties away from zero.  Near the ends of the
+// exponent range, where zeros and subnormal or non-finite values would differ, all take the
+// integer form.
+__device__ __forceinline__ void store_digit_group(const double (&v)[8], const int (&sh)[8], int e,
+                                                  __nv_bfloat16* at, int slice, int nd) {
+    const int t = 1023 + SPLIT_W - e;  // t + sh: the exponent field of 2^(sh + W - e)
+    unsigned far = abs(e) < 900 ? 0u : ~0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) far |= (unsigned)(t + sh[i] - 512);
     // w[s][i]: BF16 pair of slice s, element 2i in the low half and 2i + 1 in the high half
     uint32_t w[SPLIT_NSLICE][4];
+    auto pairs = [&](auto bits) {
 #pragma unroll
-    for (int j = 0; j < 8; j += 2) {
-        uint32_t f0[SPLIT_NSLICE], f1[SPLIT_NSLICE];
-        digits_of(q[j], f0);
-        digits_of(q[j + 1], f1);
+        for (int j = 0; j < 8; j += 2) {
+            uint32_t f0[SPLIT_NSLICE], f1[SPLIT_NSLICE];
+            digits_of(bits(j), f0);
+            digits_of(bits(j + 1), f1);
 #pragma unroll
-        for (int s = 0; s < SPLIT_NSLICE; ++s) w[s][j >> 1] = __byte_perm(f0[s], f1[s], 0x7632);
-    }
+            for (int s = 0; s < SPLIT_NSLICE; ++s) w[s][j >> 1] = __byte_perm(f0[s], f1[s], 0x7632);
+        }
+    };
+    if (far < 1024u)
+        pairs([&](int i) {
+            const double x = __longlong_as_double(__double_as_longlong(v[i]) | 1ll);
+            return __double_as_longlong(fma(x, __hiloint2double((t + sh[i]) << 20, 0), __longlong_as_double(DIGIT_BIAS)));
+        });
+    else
+        pairs([&](int i) { return fixed_of(v[i], sh[i], e) + DIGIT_BIAS; });
 #pragma unroll
     for (int s = 0; s < SPLIT_NSLICE; ++s)  // slices past nd are never read
         if (s < nd)
-            *reinterpret_cast<uint4*>(dig + dig_index(row, k0, s, T, nkb, trim)) =
-                make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+            *reinterpret_cast<uint4*>(at + s * slice) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
 }
 
-// Offset (in BF16 elements) of element (row, k) of slice s inside an operand stored as
+// Offset (in BF16 elements) of element (row, k), k < SPLIT_KB, of slice 0 inside an operand stored as
 // row tiles of T rows (the last one trimmed) and K blocks of SPLIT_KB: block (rt, kb) holds NSLICE
-// slice-blocks of T x KB elements, each in core matrices (8 rows x 8 elements) ordered (row/8, k/8).
-__device__ inline int64_t dig_index(int row, int k, int s, int T, int nkb, int trim) {
-    const int rt = row / T, r = row - rt * T, kb = k / SPLIT_KB, kk = k - kb * SPLIT_KB;
-    const int64_t tile = (int64_t)rt * nkb * SPLIT_NSLICE * (T * SPLIT_KB);
-    return tile + (int64_t)(kb * SPLIT_NSLICE + s) * (min(T, trim - rt * T) * SPLIT_KB) +
-           ((r >> 3) * (SPLIT_KB / 8) + (kk >> 3)) * 64 + (r & 7) * 8 + (kk & 7);
+// slice-blocks of T x KB elements (slice: their size), each in core matrices (8 rows x 8 elements)
+// ordered (row/8, k/8).
+__device__ inline int64_t dig_index(int row, int k, int T, int nkb, int trim, int& slice) {
+    const int rt = row / T, r = row - rt * T;
+    slice = min(T, trim - rt * T) * SPLIT_KB;
+    return (int64_t)rt * nkb * SPLIT_NSLICE * (T * SPLIT_KB) + ((r >> 3) * (SPLIT_KB / 8) + (k >> 3)) * 64 + (r & 7) * 8;
 }
 
 constexpr int DIGIT_THREADS = 4 * SPLIT_ITEM_ROWS;  // a warp per 8 rows
+// A warp's values of one pass, [K block][row][column], and the columns' shifts.  Row r keeps column k of a
+// group of 8 in place k ^ r, so that reading a row and reading one column of 8 rows and two groups
+// meet no bank twice.
+struct DigitWarp {
+    double x[SPLIT_SEG_KB * 8 * SPLIT_KB];
+    int sh[SPLIT_SEG_KB * SPLIT_KB];
+};
 
-// split_rows_kernel gives one warp 8 consecutive rows r0 .. r0+7 (r0 a multiple of 8), taken
-// as four pairs.  For a pair, lane (rr, c) = (lane / 16, lane % 16) handles row r0 + 2i + rr and
-// the 8-column groups c, c + 16, c + 32, ... (columns 128 j + 8c .. 128 j + 8c + 7).  A pair is
-// read twice, once for its exponent and once for its digits; the two reads are close enough
-// in time that the second comes from L1 or L2.  The two rows of a pair are adjacent in every
-// core matrix, so each 32-byte sector of the digit planes is written whole.
-
-// Largest exponent field over the 16 lanes of a row.
-__device__ inline int row_max16(int mx) {
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    return mx;
-}
-
-// Split 8 rows (4 pairs) through value(row, k0, v[8], sh[8]) (values and the powers of two
-// they are scaled by; zeros outside the matrix): digit planes of row tile T with nkb K blocks
-// and one int exponent per row (the modes of SplitRowsDesc::fixed).
-template <bool SEGMENTS, typename Value>
+// One warp splits 8 consecutive rows r0 .. r0+7 (r0 a multiple of 8) of an operand whose
+// values and column shifts src gives: digit planes of row tile T with nkb K blocks, and one int exponent
+// per row or segment (the modes of SplitRowsDesc::fixed).  Passes of 128 columns: lanes over
+// consecutive columns of one row after another load the values (and find the row's exponent), so that
+// a load touches few cache lines; then, through shared memory, lane (c, rr) = (lane / 8, lane % 8)
+// makes the digits of row r0 + rr, columns 8c .. 8c+7 of every K block, so that 8 lanes store one
+// core matrix, a whole line.  The L1's wavefronts bound this (lanes that loaded 8 columns each and
+// wrote two rows of a core matrix took 2.5 times as many): digit stages of 4,096 (ii|ii) 8.65 ->
+// 6.24 ms.
+template <typename Src>
 __device__ __forceinline__ void split_8rows(int r0, int nkb, int T, int trim, int fixed, int nseg, int nd,
-                                            __nv_bfloat16* __restrict__ dig, int* __restrict__ exps, Value value) {
-    const int lane = threadIdx.x & 31, c8 = 8 * (lane & 15);
-    static_assert(SPLIT_SEG_KB * SPLIT_KB == 128, "one pass of a row pair covers one segment");
-    for (int pr = 0; pr < 4; ++pr) {
-        const int row = r0 + 2 * pr + (lane >> 4);
-        if (SEGMENTS && fixed == 2) {
-            // one exponent per segment of 128 columns: one pass of the row's 16 lanes covers a
-            // segment (every lane takes every pass, for the shuffles; columns past the K blocks
-            // read as zeros and are not stored)
-            for (int sg = 0; sg < nseg; ++sg) {
-                const int k0 = 128 * sg + c8;
-                double v[8];
-                int sh[8];
-                value(row, k0, v, sh);
-                int mx = 0;
+                                            __nv_bfloat16* __restrict__ dig, int* __restrict__ exps, const Src& src,
+                                            DigitWarp& wm) {
+    const int lane = threadIdx.x & 31, rr = lane & 7, c = lane >> 3, row = r0 + rr;
+    const int npass = split_nseg(nkb);
+    double* put = wm.x + 8 * c;                            // + row, column rr ^ row
+    const double* get = wm.x + SPLIT_KB * rr + 8 * c;  // + column i ^ rr
+    int slice;
+    __nv_bfloat16* at = dig + dig_index(row, 8 * c, T, nkb, trim, slice);
+    using Col = typename Src::Col;
+    auto columns = [&](int sg, Col (&col)[SPLIT_SEG_KB]) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) mx = max(mx, exp_field_scaled(v[i], sh[i]));
-                mx = row_max16(mx);
-                const int e = mx > 0 ? mx - 1022 : SPLIT_EXP_NONE;
-                if (k0 < nkb * SPLIT_KB) {
-                    long long q[8];
+        for (int j = 0; j < SPLIT_SEG_KB; ++j) col[j] = src.col(SPLIT_KB * (SPLIT_SEG_KB * sg + j) + lane);
+    };
+    // largest exponent field of a row's values in this pass
+    auto row_exp = [&](const double (&x)[SPLIT_SEG_KB], const Col (&col)[SPLIT_SEG_KB]) {
+        int m = 0;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) q[i] = mx > 0 ? fixed_of(v[i], sh[i], e) : 0ll;
-                    store_digit_group(dig, row, k0, T, nkb, trim, q, nd);
-                }
-                if ((lane & 15) == 0) exps[(int64_t)row * nseg + sg] = e;
+        for (int j = 0; j < SPLIT_SEG_KB; ++j) m = max(m, exp_field_scaled(x[j], col[j].sh));
+        return (int)__reduce_max_sync(0xffffffffu, (unsigned)m);
+    };
+    int mx = 0;  // largest exponent field of row rr (fixed = 1: values in (-1, 1))
+    if (fixed == 0)
+        for (int sg = 0; sg < npass; ++sg) {
+            Col col[SPLIT_SEG_KB];
+            columns(sg, col);
+#pragma unroll 4
+            for (int r = 0; r < 8; ++r) {
+                double x[SPLIT_SEG_KB];
+                src.load(r, col, x);
+                const int m = row_exp(x, col);
+                if (r == rr) mx = max(mx, m);
             }
-            continue;
         }
-        int mx = fixed == 1 ? 1022 : 0;  // 1022: the exponent field bound of values in (-1, 1)
-        if (fixed == 0) {
-            for (int k0 = c8; k0 < nkb * SPLIT_KB; k0 += 128) {
-                double v[8];
-                int sh[8];
-                value(row, k0, v, sh);
+    for (int sg = 0; sg < npass; ++sg) {
+        Col col[SPLIT_SEG_KB];
+        columns(sg, col);
+        __syncwarp();  // the last pass's values have been read
 #pragma unroll
-                for (int i = 0; i < 8; ++i) mx = max(mx, exp_field_scaled(v[i], sh[i]));
+        for (int j = 0; j < SPLIT_SEG_KB; ++j) wm.sh[SPLIT_KB * j + lane] = col[j].sh;
+#pragma unroll 4
+        for (int r = 0; r < 8; ++r) {
+            double x[SPLIT_SEG_KB];
+            src.load(r, col, x);
+            if (fixed == 2) {
+                const int m = row_exp(x, col);
+                if (r == rr) mx = m;
             }
-            mx = row_max16(mx);
+#pragma unroll
+            for (int j = 0; j < SPLIT_SEG_KB; ++j) put[(8 * j + r) * SPLIT_KB + (rr ^ r)] = x[j];
         }
-        const int e = mx > 0 ? mx - 1022 : 0;  // |x| < 2^e over the row
-        for (int k0 = c8; k0 < nkb * SPLIT_KB; k0 += 128) {
+        __syncwarp();
+        const int e = mx > 0 ? mx - 1022 : 0;  // |x| < 2^e; no value of a zero row reaches a digit of e = 0
+        if (c == 0) {
+            if (fixed == 2)
+                exps[(int64_t)row * nseg + sg] = mx > 0 ? e : SPLIT_EXP_NONE;
+            else if (sg == 0)
+                exps[row] = e;
+        }
+#pragma unroll 1
+        for (int j = 0; j < SPLIT_SEG_KB; ++j) {
+            if (SPLIT_SEG_KB * sg + j == nkb) break;
             double v[8];
             int sh[8];
-            value(row, k0, v, sh);
-            long long q[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) q[i] = mx > 0 ? fixed_of(v[i], sh[i], e) : 0ll;
-            store_digit_group(dig, row, k0, T, nkb, trim, q, nd);
+            for (int i = 0; i < 8; ++i) v[i] = get[8 * SPLIT_KB * j + (i ^ rr)];
+            const int4 sa = *reinterpret_cast<const int4*>(wm.sh + SPLIT_KB * j + 8 * c);
+            const int4 sb = *reinterpret_cast<const int4*>(wm.sh + SPLIT_KB * j + 8 * c + 4);
+            sh[0] = sa.x, sh[1] = sa.y, sh[2] = sa.z, sh[3] = sa.w;
+            sh[4] = sb.x, sh[5] = sb.y, sh[6] = sb.z, sh[7] = sb.w;
+            store_digit_group(v, sh, e, at, slice, nd);
+            at += SPLIT_NSLICE * slice;
         }
-        if ((lane & 15) == 0) exps[row] = e;
     }
 }
 
-// One warp's 8 rows from r0 = item.a + 8 warp of a split_rows item (item.q = descriptor; SEGMENTS:
-// fixed = 2 may occur).
-template <bool SEGMENTS>
-__device__ __forceinline__ void split_rows_item(const SplitRowsDesc* __restrict__ descs, const WorkItem& it,
-                                                const double* __restrict__ src_base, char* __restrict__ ws) {
-    const SplitRowsDesc d = descs[it.q];
-    const int r0 = it.a + 8 * (threadIdx.x >> 5);
-    if (r0 >= d.rows) return;
-    const double* src = src_base + d.src_off;
-    const int* shift = d.shift_off >= 0 ? reinterpret_cast<const int*>(ws + d.shift_off) : nullptr;
-    split_8rows<SEGMENTS>(r0, d.nkb, d.T, d.trim, d.fixed, d.nseg, d.nd, reinterpret_cast<__nv_bfloat16*>(ws + d.dig_off),
-                reinterpret_cast<int*>(ws + d.exp_off), [&](int row, int k0, double (&v)[8], int (&sh)[8]) {
-                    const bool live = row < d.rows;
-                    const double* sr = src + (int64_t)row * d.ld;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int k = k0 + i;
-                        const bool in = live && k < d.K;
-                        v[i] = in ? sr[k] : 0.0;
-                        sh[i] = in && shift ? d.shift_sign * shift[k] : 0;
-                    }
-                });
+// x, or zero bits if the value is outside the matrix (the loads are clamped into it)
+__device__ __forceinline__ double keep_if(double x, unsigned a, unsigned b) {
+    return __hiloint2double(__double2hiint(x) & a & b, __double2loint(x) & a & b);
 }
 
-__global__ void __launch_bounds__(DIGIT_THREADS) split_rows_kernel(const SplitRowsDesc* __restrict__ descs,
-                                                         const WorkItem* __restrict__ items, int nitems,
-                                                         const double* __restrict__ src_base, char* __restrict__ ws) {
-    if (blockIdx.x < nitems) split_rows_item<true>(descs, items[blockIdx.x], src_base, ws);
+// Rows of an FP64 matrix, column k scaled by 2^(shift_sign * shift[k]).
+struct MatrixRows {
+    const double* src;
+    const int* shift;
+    int r0, rows, K, ld, sign;
+    struct Col {
+        const double* x;
+        unsigned in;
+        int sh;
+    };
+    __device__ Col col(int k) const {
+        const int kc = min(k, K - 1);
+        return {src + kc, k < K ? ~0u : 0u, k < K && shift ? sign * shift[kc] : 0};
+    }
+    __device__ void load(int r, const Col (&col)[SPLIT_SEG_KB], double (&x)[SPLIT_SEG_KB]) const {
+        const int64_t at = (int64_t)min(r0 + r, rows - 1) * ld;
+        const unsigned live = r0 + r < rows ? ~0u : 0u;
+#pragma unroll
+        for (int j = 0; j < SPLIT_SEG_KB; ++j) x[j] = keep_if(col[j].x[at], col[j].in, live);
+    }
+};
+
+// One warp's 8 rows from r0 = item.a + 8 warp of a split_rows item (item.q = descriptor).
+__device__ __forceinline__ void split_rows_item(const SplitRowsDesc* __restrict__ descs, const WorkItem& it,
+                                                const double* __restrict__ src_base, char* __restrict__ ws,
+                                                DigitWarp& wm) {
+    const SplitRowsDesc& d = descs[it.q];
+    const int r0 = it.a + 8 * (threadIdx.x >> 5);
+    if (r0 >= d.rows) return;
+    const MatrixRows src{src_base + d.src_off, d.shift_off >= 0 ? reinterpret_cast<const int*>(ws + d.shift_off) : nullptr,
+                         r0, d.rows, d.K, d.ld, d.shift_sign};
+    split_8rows(r0, d.nkb, d.T, d.trim, d.fixed, d.nseg, d.nd, reinterpret_cast<__nv_bfloat16*>(ws + d.dig_off),
+                reinterpret_cast<int*>(ws + d.exp_off), src, wm);
+}
+
+__global__ void __launch_bounds__(DIGIT_THREADS, 5) split_rows_kernel(const SplitRowsDesc* __restrict__ descs,
+                                                                   const WorkItem* __restrict__ items, int nitems,
+                                                                   const double* __restrict__ src_base,
+                                                                   char* __restrict__ ws) {
+    __shared__ __align__(16) DigitWarp wm[DIGIT_THREADS / 32];
+    if (blockIdx.x < nitems) split_rows_item(descs, items[blockIdx.x], src_base, ws, wm[threadIdx.x >> 5]);
 }
 
 // Rows q of the GEMM1 A operand: A[q][k] = [p+q]^(0) of primitive quartet (kp, kq) with
-// k = kp*Np + p, q = kq*Nq + qq, scaled by 2^c1[k].  item.q = quartet, item.a = r0.  Here
-// the 8 rows are processed at once: lane (rr, c) = (lane / 4, lane % 4) handles row r0 + rr
-// and columns 8c .. 8c+7 of every K block, so the gathers of neighbouring rows (neighbouring
-// Hermite indices) fall close together; the rows are gathered twice, once for the exponent.
-// The position of [p+q]^(0) in [r]^(0) comes from the class's index table (gidx_offset): 8
-// consecutive p of one primitive pair are one 16-byte load when they start on a multiple of 8
-// within the pair's block, which every group does when K_bra = 1.
+// k = kp*Np + p, q = kq*Nq + qq, scaled by 2^c1[k].  item.q = quartet, item.a = r0.  The position of
+// [p+q]^(0) in [r]^(0) comes from the class's index table (gidx_offset); consecutive p at one q lie
+// in runs of consecutive positions.  The rows are gathered twice, once for the exponent.
 __device__ const uint16_t* g_gidx;
+
+struct HankelRows {
+    const double* Rr;  // [r]^(0) of the quartet's first primitive quartet
+    const uint16_t* G;
+    const int* c1;
+    int64_t kp_stride;
+    int K, np;
+    unsigned r_off, g_off, live;  // of row lane % 8: its kq's [r]^(0), its q's positions
+    struct Col {
+        const double* R;
+        const uint16_t* G;
+        unsigned in;
+        int sh;
+    };
+    __device__ Col col(int k) const {
+        const int kc = min(k, K - 1), kp = kc / np;
+        return {Rr + kp * kp_stride, G + (kc - kp * np), k < K ? ~0u : 0u, k < K ? c1[kc] : 0};
+    }
+    __device__ void load(int r, const Col (&col)[SPLIT_SEG_KB], double (&x)[SPLIT_SEG_KB]) const {
+        const unsigned ro = __shfl_sync(0xffffffffu, r_off, r), go = __shfl_sync(0xffffffffu, g_off, r);
+        const unsigned lv = __shfl_sync(0xffffffffu, live, r);
+#pragma unroll
+        for (int j = 0; j < SPLIT_SEG_KB; ++j) x[j] = keep_if(col[j].R[ro + __ldg(col[j].G + go)], col[j].in, lv);
+    }
+};
 
 // One warp's 8 rows from item.a + 8 warp of a split_r item (item.q = quartet).
 __device__ __forceinline__ void split_r_item(const DQuartet* __restrict__ qd, const SplitQuartet* __restrict__ sq,
                                              const WorkItem& it, const double* __restrict__ wsd,
-                                             char* __restrict__ ws) {
-    const int lane = threadIdx.x & 31;
-    const DQuartet q = qd[it.q];
-    const SplitQuartet s = sq[it.q];
-    const int r0 = it.a + 8 * (threadIdx.x >> 5), row = r0 + (lane >> 2), c8 = 8 * (lane & 3);
-    const int nrow = q.kket * q.nq, K = q.kbra * q.np;
+                                             char* __restrict__ ws, DigitWarp& wm) {
+    const DQuartet& q = qd[it.q];
+    const SplitQuartet& s = sq[it.q];
+    const int r0 = it.a + 8 * (threadIdx.x >> 5), nq = q.nq, nrow = q.kket * nq, np = q.np;
     if (r0 >= nrow) return;
-    const bool live = row < nrow;
-    const int kq = live ? row / q.nq : 0;
-    const double* Rr = wsd + q.rr_off + (int64_t)kq * q.nr;
-    const int64_t kp_stride = (int64_t)q.kket * q.nr;
-    const int* c1 = reinterpret_cast<const int*>(ws + s.c1_off);
-    // this row's positions hidx(p + q) for p < Np
-    const uint16_t* G = g_gidx + s.gidx_off + (int64_t)(row - kq * q.nq) * ((q.np + 7) / 8 * 8);
-    // [p+q]^(0) of columns k0 .. k0+7 (unscaled) and their shifts, walking (kp, p)
-    auto group = [&](int k0, double (&v)[8], int (&sh)[8]) {
-        int kp = k0 / q.np, p = k0 - kp * q.np;
-        if (live && (p & 7) == 0 && p + 8 <= q.np && k0 + 8 <= K) {
-            // one primitive pair, 16-byte aligned: vector loads of positions and shifts
-            const uint4 g = *reinterpret_cast<const uint4*>(G + p);
-            const int4 ca = *reinterpret_cast<const int4*>(c1 + k0);
-            const int4 cb = *reinterpret_cast<const int4*>(c1 + k0 + 4);
-            const double* Rk = Rr + kp * kp_stride;
-            v[0] = Rk[g.x & 0xFFFF], v[1] = Rk[g.x >> 16], v[2] = Rk[g.y & 0xFFFF], v[3] = Rk[g.y >> 16];
-            v[4] = Rk[g.z & 0xFFFF], v[5] = Rk[g.z >> 16], v[6] = Rk[g.w & 0xFFFF], v[7] = Rk[g.w >> 16];
-            sh[0] = ca.x, sh[1] = ca.y, sh[2] = ca.z, sh[3] = ca.w;
-            sh[4] = cb.x, sh[5] = cb.y, sh[6] = cb.z, sh[7] = cb.w;
-            return;
-        }
-        int k = k0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i, ++k) {
-            double x = 0.0;
-            int h = 0;
-            if (live && k < K) {
-                x = Rr[kp * kp_stride + G[p]];
-                h = c1[k];
-            }
-            v[i] = x;
-            sh[i] = h;
-            if (++p == q.np) {
-                p = 0;
-                ++kp;
-            }
-        }
-    };
-    // exponent pass: the exponent field of x 2^c1 is that of x plus c1 (zeros stay zero)
-    int mx = 0;
-    for (int kb = 0; kb < s.nkb1; ++kb) {
-        double v[8];
-        int sh[8];
-        group(SPLIT_KB * kb + c8, v, sh);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) mx = max(mx, exp_field_scaled(v[i], sh[i]));
-    }
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const int e = mx > 0 ? mx - 1022 : 0;
-    __nv_bfloat16* dig = reinterpret_cast<__nv_bfloat16*>(ws + s.a1_dig);
-    for (int kb = 0; kb < s.nkb1; ++kb) {
-        double v[8];
-        int sh[8];
-        group(SPLIT_KB * kb + c8, v, sh);
-        long long qv[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) qv[i] = mx > 0 ? fixed_of(v[i], sh[i], e) : 0ll;
-        store_digit_group(dig, row, SPLIT_KB * kb + c8, SPLIT_TA, s.nkb1, SPLIT_NO_TRIM, qv, s.nd);
-    }
-    if ((lane & 3) == 0) reinterpret_cast<int*>(ws + s.a1_exp)[row] = e;
+    const int row = r0 + (threadIdx.x & 7), rc = min(row, nrow - 1), kq = rc / nq;
+    const HankelRows src{wsd + q.rr_off, g_gidx + s.gidx_off, reinterpret_cast<const int*>(ws + s.c1_off),
+                         (int64_t)q.kket * q.nr, q.kbra * np, np, (unsigned)(kq * q.nr),
+                         (unsigned)((rc - kq * nq) * ((np + 7) / 8 * 8)), row < nrow ? ~0u : 0u};
+    split_8rows(r0, s.nkb1, SPLIT_TA, SPLIT_NO_TRIM, 0, 0, s.nd, reinterpret_cast<__nv_bfloat16*>(ws + s.a1_dig),
+                reinterpret_cast<int*>(ws + s.a1_exp), src, wm);
 }
 
 // The operands of GEMM1 and the H operand of GEMM2 in one launch: split_r items ([p|q]^T rows,
 // issue-bound gathers) and split_rows items (H rows, load-latency bound) in alternating blocks,
 // so that the two kinds share the SMs.  One item per block.
-__global__ void __launch_bounds__(DIGIT_THREADS, 8) split_operands_kernel(const DQuartet* __restrict__ qd,
+__global__ void __launch_bounds__(DIGIT_THREADS, 5) split_operands_kernel(const DQuartet* __restrict__ qd,
                                                              const SplitQuartet* __restrict__ sq,
                                                              const WorkItem* __restrict__ items_r, int n_r,
                                                              const SplitRowsDesc* __restrict__ descs,
                                                              const WorkItem* __restrict__ items_w, int n_w,
                                                              const double* __restrict__ wsd, char* __restrict__ ws) {
+    __shared__ __align__(16) DigitWarp wm[DIGIT_THREADS / 32];
     const int m = min(n_r, n_w);
     const int b = blockIdx.x;
     int kind, idx;  // kind 0: split_r, 1: split_rows
@@ -459,9 +473,9 @@ __global__ void __launch_bounds__(DIGIT_THREADS, 8) split_operands_kernel(const 
         idx = m + (b - 2 * m);
     }
     if (kind == 0)
-        split_r_item(qd, sq, items_r[idx], wsd, ws);
+        split_r_item(qd, sq, items_r[idx], wsd, ws, wm[threadIdx.x >> 5]);
     else
-        split_rows_item<false>(descs, items_w[idx], wsd, ws);  // H rows: fixed = 1
+        split_rows_item(descs, items_w[idx], wsd, ws, wm[threadIdx.x >> 5]);
 }
 
 // ------------------------------------------------------------------ tcgen05 GEMM

@@ -152,3 +152,31 @@ def test_split_and_routed_on_degenerate_geometry():
         got = out.cpu().numpy()
         assert np.all(np.isfinite(got))
         assert np.abs(got - ref).max() <= 1e-10, f"{path}: {np.abs(got - ref).max():.3e}"
+
+
+@pytest.mark.parametrize("e", [0, 1, 500, -500, 899, -899, 900, -900, 950, -950])
+def test_digits_round_ties_away(e):
+    # B = the identity with 1 - 2^-53 for 1: its fixed-point value is 2^48, one digit, so that C is A
+    # rounded to 48 bits below 2^e exactly, ties away from zero; values from the top of the row down
+    # to 60 bits below it, ties at every depth, zeros, and subnormal numbers (which round to zero)
+    rng = np.random.default_rng(e + 1000)
+    M, K = 70, 130
+    m = rng.integers(1 << 52, 1 << 53, (M, K))
+    drop = rng.integers(0, 60, (M, K))  # bits below the row's top
+    drop[:, 0] = 0
+    tie = rng.random((M, K)) < 0.5
+    low = np.minimum(5 + drop, 53)  # bits of m below the last one kept
+    m = np.where(tie, (m >> low << low) + (np.int64(1) << (low - 1)), m)
+    A = np.ldexp(m.astype(np.float64), e - 53 - drop) * rng.choice([-1.0, 1.0], (M, K))
+    A[rng.random((M, K)) < 0.05] = 0.0
+    A[:, 0] = np.ldexp(m[:, 0].astype(np.float64), e - 53)
+    if e <= 0:
+        A[:, 5] = 5e-324
+    B = np.eye(K) * (1.0 - 2.0 ** -53)
+    C = lx.split_gemm(torch.tensor(A, device="cuda"), torch.tensor(B, device="cuda")).cpu().numpy()
+    mant, ex = np.frexp(np.abs(A))
+    units = (mant * 2.0 ** 53).astype(np.int64)  # |A| = units 2^(ex - 53)
+    down = np.clip(e - ex + 5, 0, 62)  # bits dropped, >= 5
+    q = np.where(A == 0, 0, (units + (np.int64(1) << np.maximum(down - 1, 0))) >> down)
+    ref = np.sign(A) * np.ldexp(q.astype(np.float64), e - 48)
+    assert np.array_equal(C, ref)

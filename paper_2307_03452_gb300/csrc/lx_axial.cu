@@ -61,19 +61,11 @@ __constant__ AxDev c_ax;
 // (m' >= m >= 0), from the powers pw of cos and sin of the half angle.
 constexpr int WIG_NP = 2 * AX_LP + 1;
 __host__ __device__ inline int wigner_chains(int lmax) { return (lmax + 1) * (lmax + 2) / 2; }
-// Powers 0 .. 2 lmax of the half angle's cos (which = 0) or sin (1) into pw[which WIG_NP ...], one thread.
-__device__ inline void wigner_powers(int lmax, double c, double s, int which, double* pw) {
-    double ch = sqrt(fmax(0.0, 0.5 * (1.0 + c))), sh;
-    if (ch > 0.5) {
-        sh = s / (2.0 * ch);
-    } else {
-        sh = sqrt(fmax(0.0, 0.5 * (1.0 - c)));
-        ch = s / (2.0 * sh);
-    }
-    const double b = which ? sh : ch;
+// Powers 0 .. 2 lmax of b, the half angle's cos or sin, one thread.
+__device__ inline void wigner_powers(int lmax, double b, double* pw) {
     double p = 1.0;
     for (int i = 0; i <= 2 * lmax; ++i) {
-        pw[which * WIG_NP + i] = p;
+        pw[i] = p;
         p *= b;
     }
 }
@@ -151,7 +143,7 @@ constexpr int AXP_NV = AX_NL;  // z-derivative orders of a pair
 // and across it Laguerre's: g[q][v] = sum_{ja, jb} a_ja a_jb tau(M, s, q) zeta^-(s+q+M) E[l_a - m_a - 2 ja]
 // [l_b - m_b - 2 jb][v], s = ja + jb (+ min(m_a, m_b) for the order |m_a - m_b|); the (q, v) of one
 // degree n then go over to (k, l = n - 2k).  One warp per half row.  About 7e4 FP64 operations per
-// (ii) pair against 3.5e5 for the matrix form's H: 3.5 -> 1.4 ms for 4,096 pairs.
+// (ii) pair against 3.5e5 for the matrix form's H: 7.0 -> 1.36 ms for 8,192 pairs.
 __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* __restrict__ pairs,
                                                                  const WorkItem* __restrict__ items,
                                                                  const DShell* __restrict__ sh,
@@ -162,7 +154,8 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
     __shared__ double zpow[32];
     __shared__ double g[AXP_THREADS / 32][8][AXP_NV];
     __shared__ double wt[AXP_THREADS / 32][16][8];  // weights of one half row: (ja, jb), q
-    __shared__ double pw[4 * AX_LP + 2];
+    __shared__ double pw[2 * WIG_NP];
+    __shared__ double s_pref;
     const WorkItem it = items[blockIdx.x];
     const AxPair pr = pairs[it.q];
     const DShell sa = sh[pr.sa], sb = sh[pr.sb];
@@ -170,34 +163,12 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
     const int ia = kp / sb.K, ib = kp - ia * sb.K;
     const double za = exps[sa.prim_off + ia], zb = exps[sb.prim_off + ib], zp = za + zb;
     const double AB[3] = {sb.A[0] - sa.A[0], sb.A[1] - sa.A[1], sb.A[2] - sa.A[2]};
-    const double R2 = AB[0] * AB[0] + AB[1] * AB[1] + AB[2] * AB[2];
-    double n[3];
-    const double R = ax_unit3(AB, n);
-    const double pref = exp(-za * zb / zp * R2) * ncoef[sa.prim_off + ia] * ncoef[sb.prim_off + ib];
-    if (kp == 0) {
-        double F[9], cp, sp, st;
-        frame_of(n, F, cp, sp, st);
-        double* rot = ws + pr.rot_off;
-        const int lm = max(la, lb);
-        if (tid == 0) {
-            for (int i = 0; i < 9; ++i) rot[i] = F[i];
-            double c = 1.0, s = 0.0;
-            for (int m = 0; m <= LMAX; ++m) {
-                rot[AX_ROT_CS + 2 * m] = c;
-                rot[AX_ROT_CS + 2 * m + 1] = s;
-                const double cn = c * cp - s * sp;
-                s = c * sp + s * cp;
-                c = cn;
-            }
-        }
-        if (tid < 2) wigner_powers(lm, n[2], -st, tid, pw);
-        __syncthreads();
-        for (int i = tid; i < wigner_chains(lm); i += AXP_THREADS)
-            wigner_chain(i, lm, n[2], pw, rot + AX_ROT_C, rot + AX_ROT_C + ax_co(lm + 1));
-    }
-    // z expansion, one warp, lanes over v
-    if (warp == 0) {
-        const double PA = zb * R / zp, PB = -za * R / zp, oo2p = 0.5 / zp;
+    // Each of the serial preparations in a warp of its own: in all four they took half of the FP64
+    // issues of a (dd) pair (36,697 primitive pairs 1.54 -> 0.71 ms)
+    if (warp == 0) {  // z expansion, lanes over v
+        double n[3];
+        const double R = ax_unit3(AB, n), oz = 1.0 / zp;
+        const double PA = zb * R * oz, PB = -za * R * oz, oo2p = 0.5 * oz;
         const int v = lane;
         if (v <= L + 1) E[0][min(v, AXP_NV)] = v == 0 ? 1.0 : 0.0;
         __syncwarp();
@@ -214,21 +185,48 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
                 __syncwarp();
             }
     } else if (warp == 1) {
-        if (lane == 0) {
-            double* info = ws + pr.info_off + 4 * (int64_t)kp;
+        double* info = ws + pr.info_off + 4 * (int64_t)kp;
+        if (lane < 3) {
+            info[1 + lane] = (za * sh[pr.sa].A[lane] + zb * sh[pr.sb].A[lane]) / zp;
+        } else if (lane == 3) {
             info[0] = zp;
-            for (int d = 0; d < 3; ++d) info[1 + d] = (za * sa.A[d] + zb * sb.A[d]) / zp;
-        }
-        const double oz = 1.0 / zp;
-        if (lane == 1) {  // zeta^-(s+q+M), s + q + M <= 3 LMAX
+        } else if (lane == 4) {  // zeta^-(s+q+M), s + q + M <= L
+            const double oz = 1.0 / zp;
             double p = 1.0;
-            for (int i = 0; i < 32; ++i) {
+            for (int i = 0; i <= L; ++i) {
                 zpow[i] = p;
                 p *= oz;
             }
         }
+    } else if (warp == 2) {
+        const double R2 = AB[0] * AB[0] + AB[1] * AB[1] + AB[2] * AB[2];
+        if (lane == 0) s_pref = exp(-za * zb / zp * R2) * ncoef[sa.prim_off + ia] * ncoef[sb.prim_off + ib];
+    } else if (kp == 0) {  // the pair's rotations
+        double n[3], F[9], cp, sp, st, h[2];
+        ax_unit3(AB, n);
+        frame_of(n, F, cp, sp, st);
+        double* rot = ws + pr.rot_off;
+        const int lm = max(la, lb);
+        ax_half(n[2], -st, h[0], h[1]);
+        if (lane < 2) {
+            wigner_powers(lm, lane ? h[1] : h[0], pw + lane * WIG_NP);
+        } else if (lane == 2) {
+            for (int i = 0; i < 9; ++i) rot[i] = F[i];
+            double c = 1.0, s = 0.0;
+            for (int m = 0; m <= LMAX; ++m) {
+                rot[AX_ROT_CS + 2 * m] = c;
+                rot[AX_ROT_CS + 2 * m + 1] = s;
+                const double cn = c * cp - s * sp;
+                s = c * sp + s * cp;
+                c = cn;
+            }
+        }
+        __syncwarp();
+        for (int i = lane; i < wigner_chains(lm); i += 32)
+            wigner_chain(i, lm, n[2], pw, rot + AX_ROT_C, rot + AX_ROT_C + ax_co(lm + 1));
     }
     __syncthreads();
+    const double pref = s_pref;
     const AxClass cl = c_ax.cls[pr.cls];
     const AxFn* fa0 = c_ax.fns + c_ax.shell[la][solid].fn0;
     const AxFn* fb0 = c_ax.fns + c_ax.shell[lb][solid].fn0;
@@ -277,11 +275,12 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
 
 // ------------------------------------------------------------------ rotation blocks
 
-// One CTA per primitive quartet (item.q, item.a = kp kket + kq): from the angles of the table, cos
+// One CTA per primitive quartet (item.q, item.a = kp kket + kq): from the angles of the table (those
+// about y halved), cos
 // and sin of M gamma, the Y blocks of the bra rotation and of the rotation PQ -> CD, whose chains
 // share the lanes, then the latter's full blocks (or its factors).  One warp where it holds all
-// chains at once (L <= 4 on both sides), else two: latency of a few dependent steps bounds it (tables
-// of 1,024 contracted (ff|ff), K = 5, 2.61 ms with two warps whose sides took turns, 2.13 so).
+// chains at once (L <= 4 on both sides), else two: latency of a few dependent steps bounds it (Boys
+// values and tables of 1,024 contracted (ff|ff), K = 5, 2.61 ms with two warps whose sides took turns, 2.13 so).
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS) axial_wigner_kernel(const AxQuartet* __restrict__ qd,
                                                                const WorkItem* __restrict__ items, int lmax,
@@ -296,7 +295,7 @@ __global__ void __launch_bounds__(THREADS) axial_wigner_kernel(const AxQuartet* 
     const int tid = threadIdx.x, Lb = q.Lb, Lk = q.Lk;
     if (tid < 4) {  // powers for the bra (0, 1) and ket rotation (2, 3)
         const int side = tid >> 1;
-        wigner_powers(side ? Lk : Lb, tab[4 * side], -tab[4 * side + 1], tid & 1, pw[side]);
+        wigner_powers(side ? Lk : Lb, tab[4 * side + (tid & 1)], pw[side] + (tid & 1) * WIG_NP);
     } else if (tid < 7) {  // phases: gamma, then a and b of the ket rotation
         const int w = tid - 4;
         const double c0 = tab[w == 0 ? 2 : 4 + 2 * w], s0 = tab[w == 0 ? 3 : 5 + 2 * w];
@@ -316,7 +315,8 @@ __global__ void __launch_bounds__(THREADS) axial_wigner_kernel(const AxQuartet* 
     double* tc = tab + ax_t_c(Lb, Lk);
     for (int i = tid; i < nb + nk; i += THREADS) {
         const bool ket = i >= nb;
-        wigner_chain(ket ? i - nb : i, ket ? Lk : Lb, tab[ket ? 4 : 0], pw[ket], ket ? C : tc,
+        const double ch = tab[ket ? 4 : 0], sh = tab[ket ? 5 : 1];
+        wigner_chain(ket ? i - nb : i, ket ? Lk : Lb, (ch - sh) * (ch + sh), pw[ket], ket ? C : tc,
                      ket ? S : tc + ax_co(Lb + 1));
     }
     __syncthreads();

@@ -120,6 +120,17 @@ __device__ inline double ax_unit3(const double v[3], double n[3]) {
     return m * len;
 }
 
+// cos and sin of half the angle of (c, s).
+__device__ inline void ax_half(double c, double s, double& ch, double& sh) {
+    ch = sqrt(fmax(0.0, 0.5 * (1.0 + c)));
+    if (ch > 0.5) {
+        sh = s / (2.0 * ch);
+    } else {
+        sh = sqrt(fmax(0.0, 0.5 * (1.0 - c)));
+        ch = s / (2.0 * sh);
+    }
+}
+
 struct AxHost {
     std::vector<double> g;         // axial products G(l, l', M, L), l <= l'
     std::vector<double> vinv;      // cylindrical -> spherical operators of degree n, order M

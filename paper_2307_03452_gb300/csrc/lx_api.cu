@@ -313,7 +313,7 @@ size_t axial_quartet_bytes(const lx_shell* sh, const lx_quartet& q, int flags, b
     return bytes;
 }
 
-// Parts of the ket primitives (AX_PART), as many as the quartet's room allows.
+// Parts of the ket primitives (ax_part), as many as the quartet's room allows.
 size_t axial_room(const lx_shell* sh, const lx_quartet& q, int flags);
 int axial_split(const lx_shell* sh, const lx_quartet& q, int flags, bool full) {
     const lx_shell &a = sh[q.s[0]], &b = sh[q.s[1]], &c = sh[q.s[2]], &d = sh[q.s[3]];
@@ -323,7 +323,7 @@ int axial_split(const lx_shell* sh, const lx_quartet& q, int flags, bool full) {
     const size_t nhalf = axial_tables().cls[ax_class_id(a.l, b.l, solid)].nhalf;
     const size_t per = block + (nhalf + AX_NR - 1) / AX_NR * sizeof(WorkItem);
     const size_t room = axial_room(sh, q, flags), used = axial_quartet_bytes(sh, q, flags, full) + 256;
-    const int want = std::min(kket, (prim + AX_PART - 1) / AX_PART);
+    const int part = ax_part(a.l + b.l, c.l + d.l), want = std::min(kket, (prim + part - 1) / part);
     return used >= room ? 1 : std::max(1, std::min<int>(want, 1 + (int)((room - used) / per)));
 }
 

@@ -66,8 +66,15 @@ struct AxQuartet {
 };
 // Primitive quartets per part: a CTA of the main kernel takes one part of one quartet, and with
 // K = 5 on every shell (625 primitive quartets) one CTA would outlast the rest of a batch of some
-// hundred quartets.
-constexpr int AX_PART = 16;
+// hundred quartets; of the largest classes 16 would.  So a part has as many as AX_PART_OPS, in units of
+// pyr(Lk) (Lb + 1), about a primitive quartet's work in one CTA, and at most AX_PART.  Seven mixed
+// Cartesian quartets, K = 1..2: main kernel 0.77 ms with 16 in every part, 0.46 so (0.53 at 12,000, 0.52 at
+// 8,000); 200 mixed solid ones 17.4 -> 16.6.
+constexpr int AX_PART = 16, AX_PART_OPS = 16000;
+inline int ax_part(int Lb, int Lk) {
+    const int ops = pyr(Lk) * (Lb + 1), n = AX_PART_OPS / ops;
+    return n < 1 ? 1 : n < AX_PART ? n : AX_PART;
+}
 
 // Offsets of the l blocks: cosine blocks (l+1)^2, sine blocks l^2, full blocks (2l+1)^2.
 __host__ __device__ inline int ax_co(int l) { return l * (l + 1) * (2 * l + 1) / 6; }

@@ -480,6 +480,8 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
     __shared__ unsigned farw[LX_KMAX * LX_KMAX / 32];  // far flags of the primitives of one kq
     __shared__ double cg[AX_NR][2];
     __shared__ AxHalf hr[AX_NR];
+    // the next group's launch (launch_axial_main) may fill the SMs once every CTA of this one runs
+    asm volatile("griddepcontrol.launch_dependents;");
     const WorkItem it = items[blockIdx.x];
     const AxQuartet q = qd[it.q];
     const AxPair pb = pairs[q.pb], pk = pairs[q.pk];
@@ -659,6 +661,8 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
         __syncthreads();
         if (tid == 0) ctr[2] = 0;
     }
+    // ends after the groups before it, so that what follows in the stream sees them all
+    if (tid == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ------------------------------------------------------------------ to the lab frame
@@ -854,21 +858,43 @@ cudaError_t launch_axial_wigner(const AxQuartet* qd, const WorkItem* items, int 
     return cudaGetLastError();
 }
 
+// One launch per group of shared-memory sizes.  The groups read what earlier kernels wrote and
+// write apart, so a group need not wait for the one before it: it is launched to start once all of
+// that one's CTAs run, and fills the SMs that its last, longest CTAs leave idle (7 mixed Cartesian
+// quartets, K = 1..2, 0.46 -> 0.35 ms; 200 mixed ones 16.6 -> 16.3).
+template <int THREADS, int MINB, int KM>
+cudaError_t launch_group(int n, size_t smem, bool overlap, const AxQuartet* qd, const AxPair* pairs, const WorkItem* items,
+                         double* ws, double* out, cudaStream_t st) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(n);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, axial_main_kernel<THREADS, MINB, KM>, qd, pairs, items, (const double*)ws, ws, out);
+}
+
 cudaError_t launch_axial_main(const AxQuartet* qd, const AxPair* pairs, const WorkItem* items, const int* counts,
                               const size_t* smem, double* ws, double* out, cudaStream_t st) {
+    bool overlap = false;
     for (int b = 0; b < AX_NBIN; ++b) {
         const int n = counts[b];
         if (n <= 0) continue;
+        cudaError_t e;
         switch (b) {
-            case 0: axial_main_kernel<512, 1, 8><<<n, 512, smem[b], st>>>(qd, pairs, items, ws, ws, out); break;
-            case 1: axial_main_kernel<256, 2, 7><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, ws, out); break;
-            case 2: axial_main_kernel<256, 3, 6><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, ws, out); break;
-            case 3: axial_main_kernel<256, 4, 5><<<n, 256, smem[b], st>>>(qd, pairs, items, ws, ws, out); break;
-            default: axial_main_kernel<128, 8, 4><<<n, 128, smem[b], st>>>(qd, pairs, items, ws, ws, out); break;
+            case 0: e = launch_group<512, 1, 8>(n, smem[b], overlap, qd, pairs, items, ws, out, st); break;
+            case 1: e = launch_group<256, 2, 7>(n, smem[b], overlap, qd, pairs, items, ws, out, st); break;
+            case 2: e = launch_group<256, 3, 6>(n, smem[b], overlap, qd, pairs, items, ws, out, st); break;
+            case 3: e = launch_group<256, 4, 5>(n, smem[b], overlap, qd, pairs, items, ws, out, st); break;
+            default: e = launch_group<128, 8, 4>(n, smem[b], overlap, qd, pairs, items, ws, out, st); break;
         }
-        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         items += n;
+        overlap = true;
     }
     return cudaSuccess;
 }

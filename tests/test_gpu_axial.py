@@ -127,3 +127,26 @@ def test_near_and_far_primitives():
         sl = slice(off[i], off[i] + int(np.prod(2 * ls[4 * i:4 * i + 4] + 1)))
         noise = np.abs(ref[sl] - ref2[sl]).max()
         assert np.abs(got[sl] - ref[sl]).max() <= TOL * np.abs(ref[sl]).max() + 20 * noise, seps[i]
+
+
+def test_groups_of_one_call_overlap():
+    # classes of every group of the main kernel in one call, whose launches overlap: each quartet
+    # equals its evaluation alone, bit for bit, in repeated calls and in a replayed graph
+    cls = [(7, 7, 7, 7), (6, 6, 6, 6), (5, 5, 5, 5), (4, 4, 4, 4), (3, 3, 3, 3), (4, 3, 7, 7), (7, 6, 2, 1)]
+    basis, quartets = inputs.concat([inputs.uniform_class(c, 2, 66 + i, cube=2.0, exps=(0.2, 5.0), kmin=2, kmax=2)
+                                     for i, c in enumerate(cls)])
+    b = lx.Batch(basis, quartets, True)
+    ws = lx.alloc_workspace(b.workspace_size())
+    one = torch.cat([lx.eri(basis, [q], solid=True)[0] for q in np.asarray(quartets)])
+    out = torch.empty(b.out_size, dtype=torch.float64, device="cuda")
+    for _ in range(3):
+        out.fill_(float("nan"))
+        b.run(out, ws)
+        lx.sync_status()
+        assert torch.equal(out, one)
+    graph = lx.Graph(b, out, ws)
+    for _ in range(3):
+        out.fill_(float("nan"))
+        graph.launch()
+        lx.sync_status()
+        assert torch.equal(out, one)

@@ -346,7 +346,7 @@ size_t axial_room(const lx_shell* sh, const lx_quartet& q, int flags) {
 // factors of the ket blocks in its tables, 2 = axial form with the full blocks.  A rule on its
 // class and contraction degrees alone, so that results do not depend on the batch, the chunk
 // or the workspace.  The matrix form stays for small classes, where it is the faster one
-// (AX_MIN_FMA), and where the axial form's tables (one per primitive quartet) would need more
+// (AX_MIN_FMA_SOLID and so on), and where the axial form's tables (one per primitive quartet) would need more
 // workspace than the matrix form, which the workspace sizes are stated for.
 int axial_route(const lx_shell* sh, const lx_quartet& q, int flags) {
     if (flags & LX_PATH_SPLIT) return 0;
@@ -355,8 +355,8 @@ int axial_route(const lx_shell* sh, const lx_quartet& q, int flags) {
     const int64_t nab = (int64_t)nfun(sh[q.s[0]].l, solid) * nfun(sh[q.s[1]].l, solid),
                   ncd = (int64_t)nfun(sh[q.s[2]].l, solid) * nfun(sh[q.s[3]].l, solid);
     const int prim = sh[q.s[0]].nprim * sh[q.s[1]].nprim * sh[q.s[2]].nprim * sh[q.s[3]].nprim;
-    const bool few = nab < AX_FEW_ROWS || prim < AX_FEW_PRIM;
-    if (nab * pyr(Lk) * (pyr(Lb) + ncd) < (few ? AX_MIN_FMA : AX_MIN_FMA_K)) return 0;
+    const int64_t line = prim >= AX_CONTRACTED ? AX_MIN_FMA_CONTRACTED : solid ? AX_MIN_FMA_SOLID : AX_MIN_FMA_CART;
+    if (nab * pyr(Lk) * (pyr(Lb) + ncd) < line) return 0;
     const size_t room = axial_room(sh, q, flags);
     return axial_quartet_bytes(sh, q, flags, true) <= room ? 2 : axial_quartet_bytes(sh, q, flags, false) <= room;
 }

@@ -11,15 +11,14 @@ namespace lx {
 constexpr int AX_LP = 2 * LMAX;  // largest degree of one pair's operators (14)
 constexpr int AX_NL = AX_LP + 1;
 // Smallest matrix-form transforms, N_ab N_p N_q + N_ab N_q N_cd FMAs per primitive quartet, for
-// which the axial form is taken: a contraction spreads its fixed cost (pairs, rotations), and
-// pairs of few functions leave its lanes idle.  Device times of the classes of s to k pairs near the
-// lines, matrix form against axial form: 1,024 quartets with K = 1, first classes above the line
-// Cartesian (dd|dd) 0.44 against 0.40 ms, (fd|dp) 0.44 against 0.39, below it (fp|fp) 0.30 against
-// 0.35; 256 quartets with K = 1..5, above the line (dd|dd) 3.67 against 2.41, (fd|dp) 5.07 against
-// 1.33, (fp|fp) 3.47 against 1.87; below 21 rows (dp|ff) 3.66 against 1.68 above the line.
-constexpr int AX_FEW_ROWS = 21, AX_FEW_PRIM = 4;
-constexpr int64_t AX_MIN_FMA = 85000, AX_MIN_FMA_K = 38000;  // _K: of at least
-// AX_FEW_ROWS rows and AX_FEW_PRIM primitive quartets
+// which the axial form is taken: uncontracted, by output, and of at least AX_CONTRACTED primitive
+// quartets.  Device times of all classes of s to k pairs near the lines, matrix form against axial
+// form: 1,024 uncontracted quartets, solid, (fp|fs) (the lowest) 0.209 against 0.201 ms, (dd|dd) 0.32
+// against 0.25, Cartesian just above its line (ff|ps) and (fd|pp) 1.2 to 1.5 times faster, just below it
+// (gs|dd) 0.25 against 0.28; 256 quartets with K = 1..5, above the line (dd|dd) 3.7 against 1.9, (fp|fp) 3.5
+// against 1.4, below it (dd|dp) 2.8 against 3.2.
+constexpr int AX_CONTRACTED = 4;
+constexpr int64_t AX_MIN_FMA_SOLID = 16000, AX_MIN_FMA_CART = 38000, AX_MIN_FMA_CONTRACTED = 26000;
 constexpr int AX_NR = 8;         // half rows of one CTA of the main kernel
 
 // One harmonic component group of a shell: Y_lam,m r^(l - lam) for m >= 0 (and its sine partner

@@ -60,6 +60,14 @@ def test_contracted_classes_near_the_line(cls, solid):
 
 
 @pytest.mark.parametrize("solid", [True, False])
+@pytest.mark.parametrize("cls", [(3, 1, 3, 0), (4, 0, 3, 1), (2, 1, 2, 1), (7, 0, 1, 0), (1, 0, 7, 0), (7, 1, 1, 0), (0, 0, 6, 6)])
+def test_small_classes_near_the_line(cls, solid):
+    # uncontracted classes just above and below the line of either output; (dp|dp) lies below both
+    basis, quartets = inputs.uniform_class(cls, 8, 67, cube=1.5, exps=(0.2, 5.0))
+    check(basis, quartets, solid)
+
+
+@pytest.mark.parametrize("solid", [True, False])
 def test_directions_without_azimuth(solid):
     # A, B, C, D on the z axis (either order), on the x axis, bra along z and ket along x, tiny
     # tilts of 1e-9 and 1e-170, A = B, C = D, all coincident, P = Q with A != B

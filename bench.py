@@ -76,22 +76,25 @@ def nfun(l, solid):
     return 2 * l + 1 if solid else (l + 1) * (l + 2) // 2
 
 
-# DRAM bytes per quartet of one launch, from single ncu captures (dram__bytes_read.sum +
-# dram__bytes_write.sum) of these kernels on 256 solid (ii|ii) K = 1 quartets; a launch's
-# traffic grows with its quartet count.  Each figure holds for that workload and for the
-# kernel source it was captured on, named with its sha256: once that file changes, the
-# traffic is reported as unknown (null) until it is captured again.
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) and executed FP64 FLOPs
+# (2 x dfma + dmul thread instructions) per quartet of one launch, from single ncu captures of
+# these kernels on 256 solid (ii|ii) K = 1 quartets; a launch's counts grow with its quartet
+# count.  Each figure holds for that workload and for the kernel source it was captured on,
+# named with its sha256: once that file changes, it is reported as unknown (null) until it is
+# captured again.
 NCU_TRAFFIC = {
-    "gemm1": (311.383296e6 / 256, "paper_2307_03452_gb300/csrc/lx_gemm.cu",
-              "2e31e62d4b0eb5d2d87ec27d9d5e2bf675e0e8eec6d9707d1c2f2df1cb75f841"),
-    "split_gemm1": ((957.045504e6 + 145.702656e6) / 256, "paper_2307_03452_gb300/csrc/lx_split.cu",
-                    "559aa480485e877e1e889fde8c826245b58238bb6559e839d3fb8fb2230d99a4"),
+    "axial_main": ((23.601664e6 + 5.142528e6) / 256, "paper_2307_03452_gb300/csrc/lx_axial.cu",
+                   "74e9046763e84f16c248d33f5e98b6a0376793aad42eba17645265d013920fd5"),
+    "axial_main_flops": ((2 * 369679842 + 29037262) / 256, "paper_2307_03452_gb300/csrc/lx_axial.cu",
+                         "74e9046763e84f16c248d33f5e98b6a0376793aad42eba17645265d013920fd5"),
+    "split_gemm1": ((932.810496e6 + 143.186944e6) / 256, "paper_2307_03452_gb300/csrc/lx_split.cu",
+                    "21ed6dd6f07ed4a70bb609af8012f5fd75e2a8b361be5069a35d5c94f8fcef11"),
 }
 
 
 def ncu_traffic(kernel, nquartet):
-    """DRAM bytes of one launch of `kernel` over nquartet (ii|ii) quartets, or None when its
-    source has changed since the capture."""
+    """The captured count of `kernel` for one launch over nquartet (ii|ii) quartets, or None when
+    its source has changed since the capture."""
     import hashlib
     per, path, sha = NCU_TRAFFIC[kernel]
     try:
@@ -713,23 +716,25 @@ def main(argv=None):
     g1, g2, nint = gemm_flops(basis, quartets, True)
     fp64_tf = world * (g1 + g2) * args.steps / (total_ms * 1e-3) / 1e12
     dominant = max(("gemm1", "gemm2", "pair_h", "boys_r"), key=lambda s: stage_ms[s])
-    dom_flops = {"gemm1": g1, "gemm2": g2}.get(dominant)
+    # (ii|ii) takes the axial form, whose main kernel is the gemm1 stage: its rate counts the FP64
+    # operations it executes, not those of the matrix form's transforms (g1, g2), which fp64_equiv
+    # figures use.  The peak: the measured BF16 tensor peak times the nominal FP64 / BF16 ratio,
+    # or the FP64 rate cuBLAS DGEMM reaches in this run if that is higher (a measured rate is a
+    # lower bound of the true peak, so the fraction cannot pass 1 on a figure the chip was seen to
+    # beat)
+    dom_flops = ncu_traffic("axial_main_flops", nq) if dominant == "gemm1" and default_workload else None
     per_launch_ms = stage_ms[dominant] / max(1, launches[dominant])
-    # the FP64 GEMMs are contractions on the FP64 mma.sync path.  Their peak: the measured BF16
-    # tensor peak times the nominal FP64 / BF16 ratio, or the FP64 rate cuBLAS DGEMM reaches in
-    # this run if that is higher (a measured rate is a lower bound of the true peak, so the
-    # fraction cannot pass 1 on a figure the chip was seen to beat)
     bf16_peak, bf16_src = _bf16_peak_and_source()
     fp64_derived = bf16_peak * NOMINAL_FP64_TFLOPS / NOMINAL_BF16_TFLOPS
     fp64_peak = max(fp64_derived, peak64)
-    roofline = {"bound": "tensor", "kernel": dominant, "unit": "TFLOP/s",
+    roofline = {"bound": "compute", "kernel": "axial_main" if dominant == "gemm1" else dominant, "unit": "TFLOP/s",
                 "achieved": (dom_flops / (per_launch_ms * 1e-3) / 1e12) if dom_flops else None,
                 "peak": fp64_peak,
                 "peak_source": f"max of MEASURED_PEAKS.json bf16_tflops x nominal FP64/BF16 dense ratio "
                                f"({NOMINAL_FP64_TFLOPS} / {NOMINAL_BF16_TFLOPS} TFLOP/s) = {fp64_derived:.4f} "
                                f"(of {bf16_src}) and cuBLAS DGEMM 4096^3 measured in this run = {peak64:.4f}",
                 "cublas_dgemm_tflops": peak64, "dtype": "f64",
-                "traffic": (ncu_traffic("gemm1", nq) if dominant == "gemm1" and default_workload else None),
+                "traffic": (ncu_traffic("axial_main", nq) if dominant == "gemm1" and default_workload else None),
                 "traffic_source": "ncu capture on 256 quartets scaled by quartet count; null if the kernel source "
                                   "changed since"}
     roofline["frac"] = roofline["achieved"] / fp64_peak if roofline["achieved"] else None

@@ -74,23 +74,43 @@ __device__ inline void scale_base(int L, double rho, double pref, double* B, int
     }
 }
 
+// Positions h, h - 32, ..., h - 32 (N - 1) (those >= 1) of one order of Eq. md1: all lanes read their
+// sources, then write.
+template <int N>
+__device__ __forceinline__ void hermite_r_block(int h, double X, double Y, double Z, double* R) {
+    int4 e[N];
+    double a[N], b[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) e[u] = __ldg(&g_rec[max(h - 32 * u, 1)]);
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        a[u] = R[e[u].x & 0x1FFF];
+        b[u] = R[(e[u].x >> 13) & 0x1FFF];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        const int d = e[u].x >> 26;
+        const double xd = d == 0 ? X : (d == 1 ? Y : Z);
+        const double v = fma(__hiloint2double(e[u].w, e[u].z), b[u], xd * a[u]);
+        if (h - 32 * u >= 1) R[h - 32 * u] = v;
+    }
+}
+
 // In-place Eq. md1 on R[pyr(L)] (shared memory), by one warp.  B[m] = [0]^(m), m = 0..L.
-// On return R holds [r]^(0).
+// On return R holds [r]^(0).  A position's sources lie in the two shells below its own, so one
+// order m is done from the last position down, several positions a lane at once (as many as are
+// left fill), and the warp waits once between reading and writing a block.  Bound by the latency of
+// a block's loads at 9 warps per SM (L = 24): with a shell at a time, one position a lane and a fifth of
+// the lanes idle, 0.69 ms for 4,096 (ii|ii), so 0.39.
 __device__ void hermite_r_warp(int L, double X, double Y, double Z, const double* B, double* R, int lane) {
     if (lane == 0) R[0] = B[L];
     __syncwarp();
     for (int m = L - 1; m >= 0; --m) {
-        for (int n = L - m; n >= 1; --n) {
-            const int base = n * (n + 1) * (n + 2) / 6;  // pyr(n-1)
-            const int cnt = (n + 1) * (n + 2) / 2;
-            for (int s = lane; s < cnt; s += 32) {
-                const int4 e = __ldg(&g_rec[base + s]);
-                const int d = e.x >> 26;
-                const double xd = d == 0 ? X : (d == 1 ? Y : Z);
-                R[base + s] = fma(__hiloint2double(e.w, e.z), R[(e.x >> 13) & 0x1FFF], xd * R[e.x & 0x1FFF]);
-            }
-            __syncwarp();
-        }
+        int top = pyr(L - m) - 1;
+        for (; top > 96; top -= 128) hermite_r_block<4>(top - lane, X, Y, Z, R);
+        for (; top > 32; top -= 64) hermite_r_block<2>(top - lane, X, Y, Z, R);
+        if (top >= 1) hermite_r_block<1>(top - lane, X, Y, Z, R);
         if (lane == 0) R[0] = B[m];
         __syncwarp();
     }

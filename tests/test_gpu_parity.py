@@ -300,3 +300,9 @@ def test_full_size_iiii_sampled():
     # tolerance against the class scale of the whole batch
     scale = float(out.abs().max())
     assert np.abs(got - ref).max() <= TOL_ERI * scale
+
+
+@pytest.mark.parametrize("L", [3, 4, 6, 7, 9, 10, 11])
+def test_hermite_R_stage_at_block_edges(L):
+    # orders of 1 to 363 positions besides 0, around the 32, 96 and 128 that the recursion takes at once
+    test_hermite_R_stage_matches_oracle(L)

@@ -276,12 +276,13 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
 
 // ------------------------------------------------------------------ rotation blocks
 
-// One CTA per primitive quartet (item.q, item.a = kp kket + kq): from the angles of the table (those
-// about y halved), cos
-// and sin of M gamma, the Y blocks of the bra rotation and of the rotation PQ -> CD, whose chains
+// One CTA per primitive quartet (item.q, item.a = kp kket + kq): from the half angles about y and the
+// phases of the table, the Y blocks of the bra rotation and of the rotation PQ -> CD, whose chains
 // share the lanes, then the latter's full blocks (or its factors).  One warp where it holds all
-// chains at once (L <= 4 on both sides), else two: latency of a few dependent steps bounds it (Boys
-// values and tables of 1,024 contracted (ff|ff), K = 5, 2.61 ms with two warps whose sides took turns, 2.13 so).
+// chains at once (L <= 4 on both sides), else two.  FP64 issue and the latency of a few dependent steps
+// bound it: Boys values and tables of 1,024 contracted (ff|ff), K = 5, 2.61 ms with two warps whose
+// sides took turns, 2.13 with the chains in one range, 1.56 with the half angles and 1.45 with the phases
+// from axial_boys_kernel.
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS) axial_wigner_kernel(const AxQuartet* __restrict__ qd,
                                                                const WorkItem* __restrict__ items, int lmax,
@@ -297,20 +298,10 @@ __global__ void __launch_bounds__(THREADS) axial_wigner_kernel(const AxQuartet* 
     if (tid < 4) {  // powers for the bra (0, 1) and ket rotation (2, 3)
         const int side = tid >> 1;
         wigner_powers(side ? Lk : Lb, tab[4 * side + (tid & 1)], pw[side] + (tid & 1) * WIG_NP);
-    } else if (tid < 7) {  // phases: gamma, then a and b of the ket rotation
-        const int w = tid - 4;
-        const double c0 = tab[w == 0 ? 2 : 4 + 2 * w], s0 = tab[w == 0 ? 3 : 5 + 2 * w];
-        double* o = w == 0 ? tab + ax_t_cg(Lb, Lk) : ph + 2 * (Lk + 1) * (w - 1);
-        const int n = w == 0 ? Lb : Lk;
-        double c = 1.0, s = 0.0;
-        for (int m = 0; m <= n; ++m) {
-            o[2 * m] = c;
-            o[2 * m + 1] = s;
-            const double cn = c * c0 - s * s0;
-            s = c * s0 + s * c0;
-            c = cn;
-        }
     }
+    double* D = tab + ax_t_d(Lb, Lk);
+    if (q.full)
+        for (int i = tid; i < 4 * (Lk + 1); i += THREADS) ph[i] = D[i];
     __syncthreads();
     const int nb = wigner_chains(Lb), nk = wigner_chains(Lk);
     double* tc = tab + ax_t_c(Lb, Lk);
@@ -321,12 +312,10 @@ __global__ void __launch_bounds__(THREADS) axial_wigner_kernel(const AxQuartet* 
                      ket ? S : tc + ax_co(Lb + 1));
     }
     __syncthreads();
-    double* D = tab + ax_t_d(Lb, Lk);
     if (q.full) {
         full_blocks(Lk, ph, ph + 2 * (Lk + 1), C, S, D, tid, THREADS);
     } else {
         const int nc = ax_co(Lk + 1), ns = ax_so(Lk + 1), np = 4 * (Lk + 1);
-        for (int i = tid; i < np; i += THREADS) D[i] = ph[i];
         for (int i = tid; i < nc; i += THREADS) D[np + i] = C[i];
         for (int i = tid; i < ns; i += THREADS) D[np + nc + i] = S[i];
     }

@@ -85,7 +85,8 @@ __host__ __device__ inline int ax_bz(int N) { return (N - 1) * (N - 1) / 4 + N; 
 // Rotation data of a pair: frame (9), cos and sin of m phi (m = 0..LMAX), Y blocks l = 0..LMAX.
 constexpr int AX_ROT_CS = 10, AX_ROT_C = AX_ROT_CS + 2 * (LMAX + 1);
 __host__ __device__ inline int ax_rot_size(int l) { return AX_ROT_C + ax_co(l + 1) + ax_so(l + 1); }
-// Table of a primitive quartet: angles, a flag (see AX_FAR), B Z^L, cos and sin of M gamma, Y blocks of the bra
+// Table of a primitive quartet: cos and sin of the half angles about y (bra at 0, ket at 4), a flag (see
+// AX_FAR), B Z^L, cos and sin of M gamma, Y blocks of the bra
 // rotation, and of the ket rotation either the full blocks or, at about half the size, their
 // factors: cos and sin of m a, of m b, Y blocks.
 constexpr int AX_T_FAR = 10, AX_T_BZ = 12;
@@ -99,7 +100,9 @@ __host__ __device__ inline int ax_t_cg(int Lb, int Lk) { return AX_T_BZ + ax_bz(
 __host__ __device__ inline int ax_t_c(int Lb, int Lk) { return ax_t_cg(Lb, Lk) + 2 * (Lb + 1); }
 __host__ __device__ inline int ax_t_d(int Lb, int Lk) { return ax_t_c(Lb, Lk) + ax_co(Lb + 1) + ax_so(Lb + 1); }
 __host__ __device__ inline int ax_t_size(int Lb, int Lk, bool full) {
-    return (ax_t_d(Lb, Lk) + (full ? ax_do(Lk + 1) : 4 * (Lk + 1) + ax_co(Lk + 1) + ax_so(Lk + 1)) + 3) / 4 * 4;
+    // full: the phases of the factors stand there first (more than the one block of Lk = 0)
+    const int blocks = full ? ax_do(Lk + 1) : ax_co(Lk + 1) + ax_so(Lk + 1), ph = 4 * (Lk + 1);
+    return (ax_t_d(Lb, Lk) + (full ? (blocks > ph ? blocks : ph) : ph + blocks) + 3) / 4 * 4;
 }
 
 // (c, s) = (x, y) / |(x, y)| and the length; (1, 0) for a null vector.  Scaled by the larger
@@ -135,6 +138,18 @@ __device__ inline void ax_half(double c, double s, double& ch, double& sh) {
     } else {
         sh = sqrt(fmax(0.0, 0.5 * (1.0 - c)));
         ch = s / (2.0 * sh);
+    }
+}
+
+// cos and sin of m times the angle of (c, s), m = 0..n.
+__device__ inline void ax_phases(int n, double c, double s, double* o) {
+    double x = 1.0, y = 0.0;
+    for (int m = 0; m <= n; ++m) {
+        o[2 * m] = x;
+        o[2 * m + 1] = y;
+        const double t = x * c - y * s;
+        y = x * s + y * c;
+        x = t;
     }
 }
 

@@ -183,24 +183,28 @@ __global__ void __launch_bounds__(32) boys_r_kernel(const DQuartet* __restrict__
 }
 
 // Axial form (lx_axial.cu): the angles of each primitive quartet's frames (item.q, item.a = kp kket +
-// kq) and its table B_kappa(L) Z^L.  One warp per `per` of them: first a thread each for geometry and
-// Boys values, some 600 FP64 instructions with their divisions, then 8 lanes each for the table
-// rows.  FP64 issue bounds it (one warp instruction in 20 cycles and SM), so full warps in the first part
-// count: these and the rotation blocks of 165,856 primitive quartets of (dd|dd) 2.77 -> 1.47 ms; `per`
-// = 4 spreads a short list over the SMs (64 of (gg|gg) 60 us against 92; equal at 4,096).  The powers of 2 rho and Z are one chain of products with their errors carried (7 FP64
-// instructions per degree for both; pow takes some 150 per power).
-constexpr int AXB_PER = 32, AXB_PER_FEW = 4, AXB_FEW = 4096;
-__global__ void __launch_bounds__(32) axial_boys_kernel(const AxQuartet* __restrict__ qd,
-                                                        const AxPair* __restrict__ pairs,
-                                                        const WorkItem* __restrict__ items, int nitems, int per,
-                                                        double* __restrict__ ws) {
+// kq), as half angles and phases, and its table B_kappa(L) Z^L.  One CTA per `per` of them: first a
+// thread each, in one warp for the geometry and in the other for the Boys values, some 300 FP64
+// instructions with their divisions either way, then 8 lanes each for the table rows.  FP64 issue
+// bounds it (one warp instruction in 20 cycles and SM), so full warps in the first part count: these and
+// the rotation blocks of 165,856 primitive quartets of (dd|dd) 2.77 ms with 8 lanes doing alike, 1.32 so;
+// `per` = 4 spreads a short list over the SMs (64 of (gg|gg) 52 us).  The
+// powers of 2 rho and Z are one chain of products with their errors carried (7 FP64 instructions per
+// degree for both; pow takes some 150 per power).
+constexpr int AXB_THREADS = 64, AXB_PER = 32, AXB_PER_FEW = 4, AXB_FEW = 4096;
+__global__ void __launch_bounds__(AXB_THREADS) axial_boys_kernel(const AxQuartet* __restrict__ qd,
+                                                                 const AxPair* __restrict__ pairs,
+                                                                 const WorkItem* __restrict__ items, int nitems,
+                                                                 int per, double* __restrict__ ws) {
     // B_0(L), the kappa = 1 row from entry 1, Z^L; the second row of the recursion
-    __shared__ double f_[AXB_PER][LTOT + 1], row_[AXB_PER][LTOT + 1], z_[AXB_PER][LTOT + 1], nxt_[4][LTOT + 1];
+    __shared__ double f_[AXB_PER][LTOT + 1], row_[AXB_PER][LTOT + 1], z_[AXB_PER][LTOT + 1],
+        nxt_[AXB_THREADS / 8][LTOT + 1];
     __shared__ double r2_[AXB_PER];
     __shared__ double* tab_[AXB_PER];
     __shared__ int lt_[AXB_PER];
-    const int lane = threadIdx.x, item = blockIdx.x * per + lane;
-    if (lane < per) lt_[lane] = -1;
+    const int lane = threadIdx.x & 31, item = blockIdx.x * per + lane;
+    const bool boys = threadIdx.x >= 32;
+    if (boys) lt_[lane] = -1;
     if (lane < per && item < nitems) {
         const WorkItem it = items[item];
         const AxQuartet& q = qd[it.q];
@@ -212,69 +216,75 @@ __global__ void __launch_bounds__(32) axial_boys_kernel(const AxQuartet* __restr
         const double zp = ib[0], zq = ik[0];
         const double v[3] = {ib[1] - ik[1], ib[2] - ik[2], ib[3] - ik[3]};
         const double R2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+        double* tab = ws + q.tab_off + (int64_t)it.a * q.tab_stride;
         double n[3];
         const double Z = ax_unit3(v, n);
-        const double rho = zp * zq / (zp + zq), T = rho * R2;
-        const double pref = 2.0 * PI * PI * sqrt(PI) / (zp * zq * sqrt(zp + zq));
-        double* tab = ws + q.tab_off + (int64_t)it.a * q.tab_stride;
-        // bra rotation: PQ in the AB frame (no rotation for P = Q)
-        double c = 1.0, s = 0.0, cg = 1.0, sg = 0.0;
-        if (Z > 0.0) {
-            c = Fb[6] * n[0] + Fb[7] * n[1] + Fb[8] * n[2];
-            s = ax_unit(Fb[0] * n[0] + Fb[1] * n[1] + Fb[2] * n[2], Fb[3] * n[0] + Fb[4] * n[1] + Fb[5] * n[2], cg, sg);
-        }
-        const double nrm = 1.0 / sqrt(c * c + s * s);
-        c *= nrm;
-        s *= nrm;
-        // PQ frame in the lab, and the ket rotation Rm = F_cd F_pq^T = Rz(a) Ry Rz(b)
-        double Fp[9], Rm[9];
+        if (boys) {
+            const double rho = zp * zq / (zp + zq), T = rho * R2;
+            const double pref = 2.0 * PI * PI * sqrt(PI) / (zp * zq * sqrt(zp + zq));
+            double *f = f_[lane], *row = row_[lane], *z = z_[lane];
+            boys_eval(Lt, T, f);
+            const double ex = exp(-T);
+            double ph = 1.0, pl = 0.0, zh = 1.0, zl = 0.0;
+            for (int L = 0; L <= Lt; ++L) {
+                const double pw = (L & 1 ? -pref : pref) * (ph + pl);
+                f[L] *= pw;
+                row[L] = pw * ex;
+                z[L] = zh + zl;
+                power_step(2.0 * rho, ph, pl);
+                power_step(Z, zh, zl);
+            }
+            lt_[lane] = Lt;
+            tab_[lane] = tab;
+            r2_[lane] = fmin(R2, 1e300);
+        } else {
+            // bra rotation: PQ in the AB frame (no rotation for P = Q)
+            double c = 1.0, s = 0.0, cg = 1.0, sg = 0.0;
+            if (Z > 0.0) {
+                c = Fb[6] * n[0] + Fb[7] * n[1] + Fb[8] * n[2];
+                s = ax_unit(Fb[0] * n[0] + Fb[1] * n[1] + Fb[2] * n[2], Fb[3] * n[0] + Fb[4] * n[1] + Fb[5] * n[2], cg, sg);
+            }
+            const double nrm = 1.0 / sqrt(c * c + s * s);
+            c *= nrm;
+            s *= nrm;
+            // PQ frame in the lab, and the ket rotation Rm = F_cd F_pq^T = Rz(a) Ry Rz(b)
+            double Fp[9], Rm[9];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const double r0 = cg * Fb[i] + sg * Fb[3 + i];
-            Fp[i] = c * r0 - s * Fb[6 + i];
-            Fp[3 + i] = cg * Fb[3 + i] - sg * Fb[i];
-            Fp[6 + i] = s * r0 + c * Fb[6 + i];
-        }
+            for (int i = 0; i < 3; ++i) {
+                const double r0 = cg * Fb[i] + sg * Fb[3 + i];
+                Fp[i] = c * r0 - s * Fb[6 + i];
+                Fp[3 + i] = cg * Fb[3 + i] - sg * Fb[i];
+                Fp[6 + i] = s * r0 + c * Fb[6 + i];
+            }
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
+            for (int i = 0; i < 3; ++i)
 #pragma unroll
-            for (int j = 0; j < 3; ++j)
-                Rm[3 * i + j] = Fk[3 * i] * Fp[3 * j] + Fk[3 * i + 1] * Fp[3 * j + 1] + Fk[3 * i + 2] * Fp[3 * j + 2];
-        double cb, sb, c2 = Rm[8], s2 = ax_unit(Rm[6], Rm[7], cb, sb);
-        const double nrm2 = 1.0 / sqrt(c2 * c2 + s2 * s2);
-        c2 *= nrm2;
-        s2 *= nrm2;
-        // a from what Rz(b) and Ry leave of Rm, so that a and b stay consistent when s2 is tiny:
-        // row 0 of Rm Rz(b)^T Ry^T with Rz(b)^T = [[cb, -sb], [sb, cb]], Ry^T = [[c2, 0, s2], [0, 1, 0], [-s2, 0, c2]]
-        double ca = c2 * (Rm[0] * cb + Rm[1] * sb) - s2 * Rm[2], sa = Rm[1] * cb - Rm[0] * sb;
-        const double nrm3 = 1.0 / sqrt(ca * ca + sa * sa);
-        ca *= nrm3;
-        sa *= nrm3;
-        ax_half(c, -s, tab[0], tab[1]);
-        tab[2] = cg, tab[3] = sg;
-        ax_half(c2, -s2, tab[4], tab[5]);
-        tab[6] = ca, tab[7] = sa, tab[8] = cb, tab[9] = sb;
-        double *f = f_[lane], *row = row_[lane], *z = z_[lane];
-        boys_eval(Lt, T, f);
-        const double ex = exp(-T);
-        double ph = 1.0, pl = 0.0, zh = 1.0, zl = 0.0;
-        for (int L = 0; L <= Lt; ++L) {
-            const double pw = (L & 1 ? -pref : pref) * (ph + pl);
-            f[L] *= pw;
-            row[L] = pw * ex;
-            z[L] = zh + zl;
-            power_step(2.0 * rho, ph, pl);
-            power_step(Z, zh, zl);
+                for (int j = 0; j < 3; ++j)
+                    Rm[3 * i + j] = Fk[3 * i] * Fp[3 * j] + Fk[3 * i + 1] * Fp[3 * j + 1] + Fk[3 * i + 2] * Fp[3 * j + 2];
+            double cb, sb, c2 = Rm[8], s2 = ax_unit(Rm[6], Rm[7], cb, sb);
+            const double nrm2 = 1.0 / sqrt(c2 * c2 + s2 * s2);
+            c2 *= nrm2;
+            s2 *= nrm2;
+            // a from what Rz(b) and Ry leave of Rm, so that a and b stay consistent when s2 is tiny:
+            // row 0 of Rm Rz(b)^T Ry^T with Rz(b)^T = [[cb, -sb], [sb, cb]], Ry^T = [[c2, 0, s2], [0, 1, 0], [-s2, 0, c2]]
+            double ca = c2 * (Rm[0] * cb + Rm[1] * sb) - s2 * Rm[2], sa = Rm[1] * cb - Rm[0] * sb;
+            const double nrm3 = 1.0 / sqrt(ca * ca + sa * sa);
+            ca *= nrm3;
+            sa *= nrm3;
+            ax_half(c, -s, tab[0], tab[1]);
+            ax_half(c2, -s2, tab[4], tab[5]);
+            // cos and sin of m gamma for the bra; of m a, then m b, where the ket blocks will be
+            ax_phases(q.Lb, cg, sg, tab + ax_t_cg(q.Lb, q.Lk));
+            double* ab = tab + ax_t_d(q.Lb, q.Lk);
+            ax_phases(q.Lk, ca, sa, ab);
+            ax_phases(q.Lk, cb, sb, ab + 2 * (q.Lk + 1));
         }
-        lt_[lane] = Lt;
-        tab_[lane] = tab;
-        r2_[lane] = fmin(R2, 1e300);
     }
-    __syncwarp();
+    __syncthreads();
     // 0 Z^L is taken as 0 and the square of Z kept finite: at separations where F_L underflows
     // the powers of Z may overflow
-    const int sub = lane & 7, g = lane >> 3;
-    for (int i0 = 0; i0 < per && blockIdx.x * per + i0 < nitems; i0 += 4) {
+    const int sub = lane & 7, g = threadIdx.x >> 3;
+    for (int i0 = 0; i0 < per; i0 += AXB_THREADS / 8) {
         const int i = i0 + g, Lt = lt_[i];
         const double* z = z_[i];
         double *f = f_[i], *cur = row_[i] + 1, *nxt = nxt_[g], *tab = tab_[i], *bz = tab + AX_T_BZ;
@@ -387,7 +397,7 @@ cudaError_t launch_axial_boys(const AxQuartet* qd, const AxPair* pairs, const Wo
                               cudaStream_t st) {
     if (nitems <= 0) return cudaSuccess;
     const int per = nitems > AXB_FEW ? AXB_PER : AXB_PER_FEW;
-    axial_boys_kernel<<<(nitems + per - 1) / per, 32, 0, st>>>(qd, pairs, items, nitems, per, ws);
+    axial_boys_kernel<<<(nitems + per - 1) / per, AXB_THREADS, 0, st>>>(qd, pairs, items, nitems, per, ws);
     return cudaGetLastError();
 }
 

@@ -158,3 +158,11 @@ def test_groups_of_one_call_overlap():
         graph.launch()
         lx.sync_status()
         assert torch.equal(out, one)
+
+
+@pytest.mark.parametrize("solid", [True, False])
+@pytest.mark.parametrize("cls", [(6, 6, 0, 0), (0, 0, 6, 6), (7, 5, 0, 0), (7, 5, 1, 0)])
+def test_a_side_of_s_functions(cls, solid):
+    # l = 0 alone on one side: tables whose ket blocks are the smallest, several in a row
+    basis, quartets = inputs.uniform_class(cls, 5, 68, cube=1.5, exps=(0.2, 5.0), kmin=1, kmax=3)
+    check(basis, quartets, solid)

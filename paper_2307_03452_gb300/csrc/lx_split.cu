@@ -174,8 +174,8 @@ __device__ inline double scale2(double x, int s) {
 
 // Biased exponent field of x 2^s: 0 if x is zero or subnormal or x 2^s underflows the normal
 // range, capped at 2047.
-__device__ inline int exp_field_scaled(double x, int s) {
-    const int ex = (__double2hiint(x) >> 20) & 0x7FF;
+__device__ inline int exp_field_scaled(int hi, int s) {  // hi: the upper word of x
+    const int ex = (hi >> 20) & 0x7FF;
     return ex > 0 ? min(max(ex + s, 0), 2047) : 0;
 }
 
@@ -279,7 +279,7 @@ struct DigitWarp {
 // makes the digits of row r0 + rr, columns 8c .. 8c+7 of every K block, so that 8 lanes store one
 // core matrix, a whole line.  The L1's wavefronts bound this (lanes that loaded 8 columns each and
 // wrote two rows of a core matrix took 2.5 times as many): digit stages of 4,096 (ii|ii) 8.65 ->
-// 6.24 ms.
+// 6.24 ms; 6.16 with the exponent pass of fixed = 0 on upper words, all 32 loads of a pass in flight.
 template <typename Src>
 __device__ __forceinline__ void split_8rows(int r0, int nkb, int T, int trim, int fixed, int nseg, int nd,
                                             __nv_bfloat16* __restrict__ dig, int* __restrict__ exps, const Src& src,
@@ -296,10 +296,10 @@ __device__ __forceinline__ void split_8rows(int r0, int nkb, int T, int trim, in
         for (int j = 0; j < SPLIT_SEG_KB; ++j) col[j] = src.col(SPLIT_KB * (SPLIT_SEG_KB * sg + j) + lane);
     };
     // largest exponent field of a row's values in this pass
-    auto row_exp = [&](const double (&x)[SPLIT_SEG_KB], const Col (&col)[SPLIT_SEG_KB]) {
+    auto row_exp = [&](const int (&hi)[SPLIT_SEG_KB], const Col (&col)[SPLIT_SEG_KB]) {
         int m = 0;
 #pragma unroll
-        for (int j = 0; j < SPLIT_SEG_KB; ++j) m = max(m, exp_field_scaled(x[j], col[j].sh));
+        for (int j = 0; j < SPLIT_SEG_KB; ++j) m = max(m, exp_field_scaled(hi[j], col[j].sh));
         return (int)__reduce_max_sync(0xffffffffu, (unsigned)m);
     };
     int mx = 0;  // largest exponent field of row rr (fixed = 1: values in (-1, 1))
@@ -307,11 +307,11 @@ __device__ __forceinline__ void split_8rows(int r0, int nkb, int T, int trim, in
         for (int sg = 0; sg < npass; ++sg) {
             Col col[SPLIT_SEG_KB];
             columns(sg, col);
-#pragma unroll 4
+#pragma unroll
             for (int r = 0; r < 8; ++r) {
-                double x[SPLIT_SEG_KB];
-                src.load(r, col, x);
-                const int m = row_exp(x, col);
+                int hi[SPLIT_SEG_KB];
+                src.load_hi(r, col, hi);
+                const int m = row_exp(hi, col);
                 if (r == rr) mx = max(mx, m);
             }
         }
@@ -326,7 +326,10 @@ __device__ __forceinline__ void split_8rows(int r0, int nkb, int T, int trim, in
             double x[SPLIT_SEG_KB];
             src.load(r, col, x);
             if (fixed == 2) {
-                const int m = row_exp(x, col);
+                int hi[SPLIT_SEG_KB];
+#pragma unroll
+                for (int j = 0; j < SPLIT_SEG_KB; ++j) hi[j] = __double2hiint(x[j]);
+                const int m = row_exp(hi, col);
                 if (r == rr) mx = m;
             }
 #pragma unroll
@@ -362,6 +365,9 @@ __device__ __forceinline__ double keep_if(double x, unsigned a, unsigned b) {
     return __hiloint2double(__double2hiint(x) & a & b, __double2loint(x) & a & b);
 }
 
+// The word of *p that holds its exponent.
+__device__ __forceinline__ int upper_word(const double* p) { return reinterpret_cast<const int*>(p)[1]; }
+
 // Rows of an FP64 matrix, column k scaled by 2^(shift_sign * shift[k]).
 struct MatrixRows {
     const double* src;
@@ -381,6 +387,12 @@ struct MatrixRows {
         const unsigned live = r0 + r < rows ? ~0u : 0u;
 #pragma unroll
         for (int j = 0; j < SPLIT_SEG_KB; ++j) x[j] = keep_if(col[j].x[at], col[j].in, live);
+    }
+    __device__ void load_hi(int r, const Col (&col)[SPLIT_SEG_KB], int (&hi)[SPLIT_SEG_KB]) const {
+        const int64_t at = (int64_t)min(r0 + r, rows - 1) * ld;
+        const unsigned live = r0 + r < rows ? ~0u : 0u;
+#pragma unroll
+        for (int j = 0; j < SPLIT_SEG_KB; ++j) hi[j] = upper_word(col[j].x + at) & col[j].in & live;
     }
 };
 
@@ -433,6 +445,13 @@ struct HankelRows {
         const unsigned lv = __shfl_sync(0xffffffffu, live, r);
 #pragma unroll
         for (int j = 0; j < SPLIT_SEG_KB; ++j) x[j] = keep_if(col[j].R[ro + __ldg(col[j].G + go)], col[j].in, lv);
+    }
+    __device__ void load_hi(int r, const Col (&col)[SPLIT_SEG_KB], int (&hi)[SPLIT_SEG_KB]) const {
+        const unsigned ro = __shfl_sync(0xffffffffu, r_off, r), go = __shfl_sync(0xffffffffu, g_off, r);
+        const unsigned lv = __shfl_sync(0xffffffffu, live, r);
+#pragma unroll
+        for (int j = 0; j < SPLIT_SEG_KB; ++j)
+            hi[j] = upper_word(col[j].R + (ro + __ldg(col[j].G + go))) & col[j].in & lv;
     }
 };
 

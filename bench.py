@@ -84,9 +84,9 @@ def nfun(l, solid):
 # captured again.
 NCU_TRAFFIC = {
     "axial_main": ((23.603968e6 + 5.128960e6) / 256, "paper_2307_03452_gb300/csrc/lx_axial.cu",
-                   "d26c84c84f3ba1448b77f5247dbd9176969dbab9722e8c199d8a8d7f62615082"),
+                   "90fc98fb32eb74991708d847d0ba3ee93c1fc766179ad36d84fcb47c3f187435"),
     "axial_main_flops": ((2 * 369679842 + 29037262) / 256, "paper_2307_03452_gb300/csrc/lx_axial.cu",
-                         "d26c84c84f3ba1448b77f5247dbd9176969dbab9722e8c199d8a8d7f62615082"),
+                         "90fc98fb32eb74991708d847d0ba3ee93c1fc766179ad36d84fcb47c3f187435"),
     "split_gemm1": ((932.808960e6 + 139.972608e6) / 256, "paper_2307_03452_gb300/csrc/lx_split.cu",
                     "5de22ce9fdf3d9152351ae56c6097075c27336080eeb27cd667ba8dcde5d60da"),
 }

@@ -454,8 +454,8 @@ __device__ __forceinline__ void r_far(int l, int mm, int mtop, int nk, bool firs
 // the 8 half rows (then the 16 rows: cosine, sine), so every table value is a broadcast and
 // every operand row one conflict-free shared access; groups of tasks are taken from shared
 // counters, the longest first.  Every stage is bound by the FP64 pipe: 87,300 warp FMAs per
-// (ii|ii) quartet, at the 20 cycles each that a plain FMA loop reaches 843 us of one SM; measured
-// 934 us (12.6 ms for 2,048 quartets).
+// (ii|ii) quartet, at the 20 cycles each that a plain FMA loop reaches 843 us of one SM (11.4 ms for 2,048
+// quartets); measured 11.1 ms within 6 bohr, where few are far, and 8.4 ms in a 20-bohr cube.
 // KM: the largest k range, Lk / 2 + 1, that the group's shared memory admits.
 template <int THREADS, int MINB, int KM>
 __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuartet* __restrict__ qd,

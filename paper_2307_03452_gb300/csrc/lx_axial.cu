@@ -287,7 +287,7 @@ template <int THREADS>
 __global__ void __launch_bounds__(THREADS) axial_wigner_kernel(const AxQuartet* __restrict__ qd,
                                                                const WorkItem* __restrict__ items, int lmax,
                                                                double* __restrict__ ws) {
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
     __shared__ double pw[2][2 * WIG_NP], ph[4 * AX_NL];  // ph: cos, sin of m a, then of m b: 4 (Lk + 1)
     double* C = sm;
     double* S = C + ax_co(lmax + 1);
@@ -463,7 +463,8 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
                                                                    const WorkItem* __restrict__ items,
                                                                    const double* __restrict__ ws, double* wso,
                                                                    double* out) {
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
+    static_assert(__alignof__(sm) >= alignof(double2), "r_task and r_far take X's entries in pairs");
     __shared__ int tinfo[AX_NL * AX_NL];
     __shared__ int hpre[AX_NL + 1], scp[AX_NL + 1], ssp[AX_NL + 1], xp[AX_NL + 1];
     __shared__ int ctr[3];
@@ -672,7 +673,7 @@ __global__ void __launch_bounds__(THREADS) axial_rotate_kernel(const AxQuartet* 
                                                                    const WorkItem* __restrict__ items, int lanes,
                                                                    const double* __restrict__ ws,
                                                                    double* __restrict__ out, int solid) {
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
     __shared__ double rot[AX_ROT_C + 204 + 140];
     const WorkItem it = items[blockIdx.x];
     const AxQuartet q = qd[it.q];

@@ -193,13 +193,15 @@ struct Overrides {
 // ------------------------------------------------------------------ planning
 
 // Pair ids of one chunk: an open-addressing table keyed by (shells, side), emptied in O(1) by a new
-// generation.  (std::unordered_map took about a third of the planning of small classes.)
+// generation.  (std::unordered_map took about a third of the planning of small classes.)  It starts
+// with room for as many pairs as `nquartet` quartets can have, up to 16,384 (half a MB), and grows with the
+// pairs it holds: a list of n x n quartets has only 2 n.
 inline int64_t pair_key(int sa, int sb, int side) { return ((int64_t)sa << 32 | (uint32_t)sb) * 2 + side; }
 class PairMap {
   public:
     explicit PairMap(int64_t nquartet) {
         size_t n = 64;
-        while (n < 4 * (size_t)std::min<int64_t>(nquartet, 1 << 20)) n *= 2;
+        while (n < 4 * (size_t)std::min<int64_t>(nquartet, 1 << 13)) n *= 2;
         slots_.assign(n, Slot{0, 0, 0});
     }
     void clear() {
@@ -977,7 +979,7 @@ int plan_batch(const lx_shell* shells, int32_t nshell, const double* exps, const
     const int pflags = flags & (LX_SOLID | LX_PATH_SPLIT | JK_DIGEST | LX_SPLIT_DIGITS_MASK);
     std::vector<Chunk> chunks;
     Shapes shapes(shells, pflags);
-    PairMap pid(nquartet), apid(nquartet);
+    PairMap pid(nquartet), apid(flags & LX_PATH_SPLIT ? 0 : nquartet);
     int v = plan_chunks(shapes, quartets, nquartet, workspace_bytes - B.head, pid, chunks);
     if (v != LX_OK) return v;
     B.head_blob.assign(B.head, 0);

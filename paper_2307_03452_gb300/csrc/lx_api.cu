@@ -192,7 +192,7 @@ struct Overrides {
 
 // ------------------------------------------------------------------ planning
 
-// Pair ids of one chunk: an open-addressing table keyed by (shells, side), emptied in O(1) by a new
+// Pairs of one chunk: an open-addressing table keyed by (shells, side), emptied in O(1) by a new
 // generation.  (std::unordered_map took about a third of the planning of small classes.)  It starts
 // with room for as many pairs as `nquartet` quartets can have, up to 16,384 (half a MB), and grows with the
 // pairs it holds: a list of n x n quartets has only 2 n.
@@ -208,23 +208,22 @@ class PairMap {
         ++gen_;
         used_ = 0;
     }
-    // The id stored for k, or `id` after storing it (fresh = true).
-    int get(int64_t k, int id, bool& fresh) {
+    // The value stored for k, or `v` after storing it (fresh = true); valid until the next call.
+    int& get(int64_t k, int v, bool& fresh) {
         if (2 * (used_ + 1) > slots_.size()) grow();
         Slot& s = find(k);
         fresh = s.gen != gen_;
         if (fresh) {
-            s = Slot{k, id, gen_};
+            s = Slot{k, v, gen_};
             ++used_;
         }
-        return s.id;
+        return s.value;
     }
-    bool has(int64_t k) { return find(k).gen == gen_; }
 
   private:
     struct Slot {
         int64_t key;
-        int id;
+        int value;
         unsigned gen;
     };
     Slot& find(int64_t k) {
@@ -240,7 +239,7 @@ class PairMap {
         const unsigned g = gen_;
         gen_ = 1;
         for (const Slot& s : old)
-            if (s.gen == g) find(s.key) = Slot{s.key, s.id, 1};
+            if (s.gen == g) find(s.key) = Slot{s.key, s.value, 1};
     }
     std::vector<Slot> slots_;
     size_t used_ = 0;
@@ -315,15 +314,21 @@ size_t axial_quartet_bytes(const lx_shell* sh, const lx_quartet& q, int flags, b
     return bytes;
 }
 
+// What the parts of the ket primitives beyond the first add: their sums and their main items.
+size_t axial_part_bytes(const lx_shell* sh, const lx_quartet& q, int flags, int nsplit) {
+    const lx_shell &a = sh[q.s[0]], &b = sh[q.s[1]], &c = sh[q.s[2]], &d = sh[q.s[3]];
+    const bool solid = flags & LX_SOLID;
+    const size_t block = 8 * (size_t)nfun(a.l, solid) * nfun(b.l, solid) * nfun(c.l, solid) * nfun(d.l, solid);
+    const size_t nhalf = axial_tables().cls[ax_class_id(a.l, b.l, solid)].nhalf;
+    return nsplit > 1 ? (nsplit - 1) * (block + (nhalf + AX_NR - 1) / AX_NR * sizeof(WorkItem)) + 256 : 0;
+}
+
 // Parts of the ket primitives (ax_part), as many as the quartet's room allows.
 size_t axial_room(const lx_shell* sh, const lx_quartet& q, int flags);
 int axial_split(const lx_shell* sh, const lx_quartet& q, int flags, bool full) {
     const lx_shell &a = sh[q.s[0]], &b = sh[q.s[1]], &c = sh[q.s[2]], &d = sh[q.s[3]];
-    const bool solid = flags & LX_SOLID;
     const int kket = c.nprim * d.nprim, prim = a.nprim * b.nprim * kket;
-    const size_t block = 8 * (size_t)nfun(a.l, solid) * nfun(b.l, solid) * nfun(c.l, solid) * nfun(d.l, solid);
-    const size_t nhalf = axial_tables().cls[ax_class_id(a.l, b.l, solid)].nhalf;
-    const size_t per = block + (nhalf + AX_NR - 1) / AX_NR * sizeof(WorkItem);
+    const size_t per = axial_part_bytes(sh, q, flags, 2) - 256;
     const size_t room = axial_room(sh, q, flags), used = axial_quartet_bytes(sh, q, flags, full) + 256;
     const int part = ax_part(a.l + b.l, c.l + d.l), want = std::min(kket, (prim + part - 1) / part);
     return used >= room ? 1 : std::max(1, std::min<int>(want, 1 + (int)((room - used) / per)));
@@ -349,7 +354,7 @@ size_t axial_room(const lx_shell* sh, const lx_quartet& q, int flags) {
 // class and contraction degrees alone, so that results do not depend on the batch, the chunk
 // or the workspace.  The matrix form stays for small classes, where it is the faster one
 // (AX_MIN_FMA_SOLID and so on), and where the axial form's tables (one per primitive quartet) would need more
-// workspace than the matrix form, which the workspace sizes are stated for.
+// workspace than the matrix form takes for the quartet and its pairs, which lx_eri_workspace_min is stated for.
 int axial_route(const lx_shell* sh, const lx_quartet& q, int flags) {
     if (flags & LX_PATH_SPLIT) return 0;
     const bool solid = flags & LX_SOLID;
@@ -363,16 +368,22 @@ int axial_route(const lx_shell* sh, const lx_quartet& q, int flags) {
     return axial_quartet_bytes(sh, q, flags, true) <= room ? 2 : axial_quartet_bytes(sh, q, flags, false) <= room;
 }
 
+// Workspace bytes of a quartet's own data and of its two pairs.
+struct FormBytes {
+    size_t own = 0, bra = 0, ket = 0;
+};
 // What the planner needs of a quartet that depends on its class and contraction degrees alone,
 // computed once per shape of a batch.
 struct Shape {
-    uint64_t key = ~0ull;
-    size_t qbytes = 0, bra_bytes = 0, ket_bytes = 0;
-    int route = 0, nsplit = 1;
+    uint64_t key = 0;        // 0: empty (a shell has at least one primitive)
+    FormBytes matrix, form;  // in the matrix form, and in the form that it takes
+    int route = 0, nsplit = 0;
 };
 class Shapes {
   public:
-    Shapes(const lx_shell* sh, int flags) : sh_(sh), flags_(flags), cache_(1024) {}
+    // matrix_only: every quartet takes the matrix form
+    Shapes(const lx_shell* sh, int flags, bool matrix_only = false)
+        : sh_(sh), flags_(flags), matrix_only_(matrix_only), cache_(1024) {}
     const Shape& of(const lx_quartet& q) {
         uint64_t k = 0;
         for (int i = 0; i < 4; ++i) k = k << 8 | (uint64_t)(sh_[q.s[i]].l << 5 | sh_[q.s[i]].nprim);
@@ -380,11 +391,14 @@ class Shapes {
         Shape& s = cache_[h >> 54];
         if (s.key != k) {
             s.key = k;
-            s.qbytes = quartet_bytes(sh_, q, flags_);
-            s.bra_bytes = pair_bytes(sh_, q.s[0], q.s[1], flags_);
-            s.ket_bytes = pair_bytes(sh_, q.s[2], q.s[3], flags_);
-            s.route = axial_route(sh_, q, flags_);
+            s.matrix = {quartet_bytes(sh_, q, flags_), pair_bytes(sh_, q.s[0], q.s[1], flags_),
+                        pair_bytes(sh_, q.s[2], q.s[3], flags_)};
+            s.route = matrix_only_ ? 0 : axial_route(sh_, q, flags_);
             s.nsplit = s.route ? axial_split(sh_, q, flags_, s.route == 2) : 1;
+            s.form = s.matrix;
+            if (s.route)
+                s.form = {axial_quartet_bytes(sh_, q, flags_, s.route == 2) + axial_part_bytes(sh_, q, flags_, s.nsplit),
+                          axial_pair_bytes(sh_, q.s[0], q.s[1], flags_), axial_pair_bytes(sh_, q.s[2], q.s[3], flags_)};
         }
         return s;
     }
@@ -392,6 +406,7 @@ class Shapes {
   private:
     const lx_shell* sh_;
     int flags_;
+    bool matrix_only_;
     std::vector<Shape> cache_;
 };
 static_assert(LX_LMAX < 8 && LX_KMAX < 32, "a shell's l and degree fit 8 bits of a shape key");
@@ -402,35 +417,54 @@ size_t head_bytes(int nshell, int nprim) {
     return align256(sizeof(DShell) * (size_t)nshell) + 3 * align256(sizeof(double) * (size_t)nprim);
 }
 
+// Bytes of one chunk of quartets: an upper bound of the layout that build_chunk gives it, each pair
+// counted once per form, and of what the matrix form takes for all of them.  The workspace sizes
+// are the larger: the axial form's tables may take the room of a quartet's matrix-form pairs
+// (axial_room), which quartets that share those pairs have only once, and callers of forced tile
+// shapes and of other paths find what the matrix form needs.
+struct ChunkBytes {
+    size_t matrix = CHUNK_SLACK, form = CHUNK_SLACK;
+    size_t total() const { return std::max(matrix, form); }
+    void add(const lx_quartet& q, const Shape& s, PairMap& seen) {
+        matrix += s.matrix.own;
+        form += s.form.own;
+        pair(seen, pair_key(q.s[0], q.s[1], 0), s.route, s.matrix.bra, s.form.bra);
+        pair(seen, pair_key(q.s[2], q.s[3], 1), s.route, s.matrix.ket, s.form.ket);
+    }
+
+  private:
+    // seen: a bit for each form that holds the pair
+    void pair(PairMap& seen, int64_t key, int route, size_t in_matrix, size_t in_form) {
+        bool fresh;
+        int& forms = seen.get(key, 0, fresh);
+        const int bit = route ? 2 : 1;
+        if (fresh) matrix += in_matrix;
+        if (!(forms & bit)) form += in_form;
+        forms |= bit;
+    }
+};
+
 // Greedy chunking of the quartet list so that each chunk fits `budget` bytes.
 int plan_chunks(Shapes& shapes, const lx_quartet* qs, int64_t nq, size_t budget, PairMap& seen,
                 std::vector<Chunk>& chunks) {
     chunks.clear();
     seen.clear();
-    size_t used = CHUNK_SLACK;
+    ChunkBytes used;
     Chunk cur;
-    cur.q_begin = 0;
     for (int64_t i = 0; i < nq; ++i) {
-        const lx_quartet& q = qs[i];
-        const Shape& s = shapes.of(q);
-        const int64_t kb = pair_key(q.s[0], q.s[1], 0), kk = pair_key(q.s[2], q.s[3], 1);
-        size_t add = s.qbytes;
-        if (!seen.has(kb)) add += s.bra_bytes;
-        if (!seen.has(kk)) add += s.ket_bytes;
-        if (used + add > budget) {
+        ChunkBytes next = used;
+        next.add(qs[i], shapes.of(qs[i]), seen);
+        if (next.total() > budget) {
             if (i == cur.q_begin) return LX_ERR_WORKSPACE;  // one quartet does not fit
             cur.q_end = i;
             chunks.push_back(cur);
             cur.q_begin = i;
+            used = ChunkBytes();
             seen.clear();
-            used = CHUNK_SLACK;
-            --i;  // retry this quartet in the new chunk
+            --i;
             continue;
         }
-        used += add;
-        bool fresh;
-        seen.get(kb, 0, fresh);
-        seen.get(kk, 0, fresh);
+        used = next;
     }
     cur.q_end = nq;
     if (nq > 0) chunks.push_back(cur);
@@ -564,7 +598,7 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
         size_t nax = 0, prims = 0, nmatrix = 0;
         for (int64_t i = ch.q_begin; i < ch.q_end; ++i) {
             const lx_quartet& q = qs[i];
-            if (ov.v1 < 0 && shapes.of(q).route) ++nax;
+            if (shapes.of(q).route) ++nax;
             else ++nmatrix;
             prims += (size_t)sh[q.s[0]].nprim * sh[q.s[1]].nprim * sh[q.s[2]].nprim * sh[q.s[3]].nprim;
         }
@@ -575,7 +609,7 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
     }
     for (int64_t i = ch.q_begin; i < ch.q_end; ++i) {
         const lx_quartet& q = qs[i];
-        const int route = ov.v1 < 0 ? shapes.of(q).route : 0;
+        const int route = shapes.of(q).route;
         if (route) {
             const lx_shell &a = sh[q.s[0]], &b = sh[q.s[1]], &c = sh[q.s[2]], &dd = sh[q.s[3]];
             AxQuartet x{};
@@ -932,22 +966,12 @@ void build_chunk(const lx_shell* sh, const lx_quartet* qs, const Chunk& ch, int 
     P.total = (size_t)dw * 8 - chunk_base;
 }
 
-// Workspace bytes that plan_chunks needs to keep quartets [b, e) in one chunk (an upper
-// bound of the exact layout built by build_chunk).
+// Workspace bytes that plan_chunks needs to keep quartets [b, e) in one chunk.
 size_t chunk_estimate(Shapes& shapes, const lx_quartet* qs, int64_t b, int64_t e, PairMap& seen) {
     seen.clear();
-    size_t used = CHUNK_SLACK;
-    for (int64_t i = b; i < e; ++i) {
-        const lx_quartet& q = qs[i];
-        const Shape& s = shapes.of(q);
-        bool fresh;
-        used += s.qbytes;
-        seen.get(pair_key(q.s[0], q.s[1], 0), 0, fresh);
-        if (fresh) used += s.bra_bytes;
-        seen.get(pair_key(q.s[2], q.s[3], 1), 0, fresh);
-        if (fresh) used += s.ket_bytes;
-    }
-    return used;
+    ChunkBytes used;
+    for (int64_t i = b; i < e; ++i) used.add(qs[i], shapes.of(qs[i]), seen);
+    return used.total();
 }
 
 int64_t prim_count(const lx_shell* sh, int32_t nshell) {
@@ -978,7 +1002,7 @@ int plan_batch(const lx_shell* shells, int32_t nshell, const double* exps, const
     if (workspace_bytes < B.head + CHUNK_SLACK) return LX_ERR_WORKSPACE;
     const int pflags = flags & (LX_SOLID | LX_PATH_SPLIT | JK_DIGEST | LX_SPLIT_DIGITS_MASK);
     std::vector<Chunk> chunks;
-    Shapes shapes(shells, pflags);
+    Shapes shapes(shells, pflags, ov.v1 >= 0);
     PairMap pid(nquartet), apid(flags & LX_PATH_SPLIT ? 0 : nquartet);
     int v = plan_chunks(shapes, quartets, nquartet, workspace_bytes - B.head, pid, chunks);
     if (v != LX_OK) return v;
@@ -1001,20 +1025,10 @@ int plan_batch(const lx_shell* shells, int32_t nshell, const double* exps, const
         std::memcpy(B.head_blob.data() + B.o_exps, exps, sizeof(double) * (size_t)nprim_total);
         std::memcpy(B.head_blob.data() + B.o_coefs, coefs, sizeof(double) * (size_t)nprim_total);
     }
+    B.chunks.resize(chunks.size());
     for (size_t c = 0; c < chunks.size(); ++c) {
-        B.chunks.emplace_back();
-        build_chunk(shells, quartets, chunks[c], pflags, B.head, shapes, pid, apid, B.chunks.back(), ov);
-        if (B.head + B.chunks.back().total <= workspace_bytes) continue;
-        // plan_chunks counts the matrix form with every pair once: a pair stored in both forms, or
-        // tables that take the room of pairs which quartets share, may not fit.  Halve such a chunk
-        // (one quartet always fits)
-        Chunk half = chunks[c];
-        if (half.q_end - half.q_begin < 2) return LX_ERR_WORKSPACE;
-        half.q_begin += (half.q_end - half.q_begin) / 2;
-        chunks[c].q_end = half.q_begin;
-        chunks.insert(chunks.begin() + c + 1, half);
-        B.chunks.pop_back();
-        --c;
+        build_chunk(shells, quartets, chunks[c], pflags, B.head, shapes, pid, apid, B.chunks[c], ov);
+        if (B.head + B.chunks[c].total > workspace_bytes) return LX_ERR_WORKSPACE;
     }
     return LX_OK;
 }

@@ -258,8 +258,10 @@ int lx_eri_graph_destroy(void* handle);
  * output kind): for each of the `max_keys` costliest keys of the batch, up to `samples` of its
  * quartets are evaluated with every tile shape (32x64, 64x32, 32x32, 64x64) and the fastest,
  * timed with CUDA events on cuda_stream, is recorded in the library's tuning table, which the
- * planner consults for every later call (for the quartets that take the GEMMs).  out (DEVICE, out_doubles long) and workspace are
- * scratch.  Synchronises cuda_stream.  The split path has a single tile shape: no-op.
+ * planner consults for every later call.  Only quartets that take the GEMMs use it: keys of the
+ * axial form are passed over, unless the batch has no others.  out (DEVICE, out_doubles long)
+ * and workspace are scratch.  Synchronises cuda_stream.  The split path has a single tile shape:
+ * no-op.
  */
 int lx_eri_autotune(const lx_shell* shells, int32_t nshell, const double* exps, const double* coefs,
                     int32_t nprim_total, const lx_quartet* quartets, int64_t nquartet, int32_t flags, double* out,

@@ -1693,10 +1693,17 @@ int lx_eri_autotune(const lx_shell* shells, int32_t nshell, const double* exps, 
     if ((v = ensure_device(&status)) != LX_OK) return v;
     const bool solid = flags & LX_SOLID;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    // Only quartets that take the matrix form, in lx_eri_batch or in lx_eri_jk, look at the table: the
+    // other keys are left out (timing them took most of the call, and they used up max_keys).  A batch
+    // of nothing else has its costliest keys timed and recorded all the same.
+    Shapes batch_shapes(shells, flags & LX_SOLID), jk_shapes(shells, (flags & LX_SOLID) | JK_DIGEST);
+    auto takes_gemms = [&](const lx_quartet& q) { return !batch_shapes.of(q).route || !jk_shapes.of(q).route; };
+    const bool some = std::any_of(quartets, quartets + nquartet, takes_gemms);
     // group by key; the costliest keys (total GEMM1 work) first
     std::map<TuneKey, std::vector<int64_t>> groups;
     std::map<TuneKey, double> cost;
     for (int64_t i = 0; i < nquartet; ++i) {
+        if (some && !takes_gemms(quartets[i])) continue;
         const TuneKey k = tune_key(shells, quartets[i], solid);
         groups[k].push_back(i);
         cost[k] += (double)nfun(k.la, solid) * nfun(k.lb, solid) * k.kbra * pyr(k.la + k.lb) * k.kket * pyr(k.lc + k.ld);

@@ -234,6 +234,12 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
     double* h = ws + pr.h_off + (int64_t)kp * cl.nh;
     for (int r = blockIdx.y * (AXP_THREADS / 32) + warp; r < cl.nhalf; r += gridDim.y * (AXP_THREADS / 32)) {
         const AxHalf hr = c_ax.halves[cl.half0 + r];
+        const int cnt = (r + 1 < cl.nhalf ? c_ax.halves[cl.half0 + r + 1].hoff : cl.nh) - hr.hoff;
+        double* hp = h + hr.hoff;
+        if (pref == 0.0) {  // centers so far apart that powers of R may have overflowed: 0 times them is 0
+            for (int e = lane; e < cnt; e += 32) hp[e] = 0.0;
+            continue;
+        }
         const AxFn &fa = fa0[hr.fa], &fb = fb0[hr.fb];
         const int ma = fa.m, mb = fb.m, M = hr.M;
         const int na = (la - ma) / 2, nb = (lb - mb) / 2, s0 = hr.slot ? min(ma, mb) : 0;
@@ -259,8 +265,6 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
         }
         __syncwarp();
         // entries (l, k), l = M .. L, k = 0 .. (L - l) / 2, of degree n = 2k + l
-        double* hp = h + hr.hoff;
-        const int cnt = (r + 1 < cl.nhalf ? c_ax.halves[cl.half0 + r + 1].hoff : cl.nh) - hr.hoff;
         for (int e = lane; e < cnt; e += 32) {
             int l = M, k = e;
             for (int nk; k >= (nk = (L - l) / 2 + 1); ++l) k -= nk;

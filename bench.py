@@ -11,7 +11,9 @@ GEMM1 and GEMM2 (every row of the hot path).
 
 Multi-GPU: one process per GPU under torchrun, each evaluating its own replica of the
 batch (quartets are independent: weak scaling, no data-path collective); the timing is
-the max over ranks.  Rank 0 prints one JSON line.
+the max over ranks.  Rank 0 prints one JSON line, short enough (about 2.5 kB) to be read whole by a
+caller that keeps only the end of the output; before it, the full record of every leg (stages, errors per
+class, notes) goes to stderr as one JSON line.
 """
 from __future__ import annotations
 
@@ -438,6 +440,35 @@ def run_reference(args):
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
     print(json.dumps(line), flush=True)
     return 0
+
+
+# What the printed line keeps of each leg, and of each arm of one.
+LEG_KEYS = ("quartets_per_s", "ms_per_step", "max_abs_diff_vs_fp64_path", "split_max_abs_diff_vs_fp64_on_sample",
+            "max_abs_err_vs_fp64_path_on_sample", "routed_quartets_per_s",
+            "split_only_quartets_per_s", "fp64_only_quartets_per_s", "routed_max_abs_err_vs_fp64_on_sample")
+LEGS = ("cartesian", "split", "mixed", "split_config", "routed", "pairs", "jk")
+PART_KEYS = {"roofline": ("bound", "kernel", "unit", "achieved", "peak", "frac", "cublas_dgemm_tflops", "traffic"),
+             "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"),
+             "cpu_baseline": ("value", "unit", "cores", "kind")}
+
+
+def headline(record):
+    """The printed line: the record's own figures, and of its legs the rates and largest errors, to 6 digits."""
+    def short(d, keys):
+        return {k: float(f"{d[k]:.6g}") if isinstance(d[k], float) else d[k] for k in keys if d.get(k) is not None}
+
+    line = {k: v for k, v in record.items() if k not in LEGS and k not in PART_KEYS and k != "sweep"}
+    line["stage_ms_per_step"] = short(record["stage_ms_per_step"], record["stage_ms_per_step"])
+    for part, keys in PART_KEYS.items():
+        line[part] = {k: record[part].get(k) for k in keys} if record.get(part) else None
+    for leg in LEGS:
+        if not record.get(leg):
+            continue
+        line[leg] = short(record[leg], LEG_KEYS)
+        for arm in ("fp64", "split"):
+            if isinstance(record[leg].get(arm), dict):
+                line[leg][arm] = short(record[leg][arm], LEG_KEYS)
+    return line
 
 
 SWEEP_CLASSES = [(2, 2, 2, 2), (3, 3, 3, 3), (4, 4, 4, 4), (5, 5, 5, 5), (6, 6, 6, 6), (7, 7, 7, 7)]
@@ -956,7 +987,7 @@ def main(argv=None):
         cpu["oracle_checks_s"] = checks.run()
 
     if rank == 0:
-        line = {
+        record = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
@@ -970,7 +1001,8 @@ def main(argv=None):
             "sweep": sweep,
             "gpu_launches": int(sum(launches.values())),
         }
-        print(json.dumps(line), flush=True)
+        print(json.dumps(record), file=sys.stderr, flush=True)
+        print(json.dumps(headline(record)), flush=True)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()

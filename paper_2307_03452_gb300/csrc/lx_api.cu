@@ -379,35 +379,53 @@ struct Shape {
     FormBytes matrix, form;  // in the matrix form, and in the form that it takes
     int route = 0, nsplit = 0;
 };
+// An open-addressing table that grows with the shapes it holds (K = 1..5 on every shell of one class
+// makes 625 of them, more than a table that forgets on a collision kept).
 class Shapes {
   public:
     // matrix_only: every quartet takes the matrix form
     Shapes(const lx_shell* sh, int flags, bool matrix_only = false)
-        : sh_(sh), flags_(flags), matrix_only_(matrix_only), cache_(1024) {}
+        : sh_(sh), flags_(flags), matrix_only_(matrix_only), slots_(64) {}
+    // valid until the next call
     const Shape& of(const lx_quartet& q) {
         uint64_t k = 0;
         for (int i = 0; i < 4; ++i) k = k << 8 | (uint64_t)(sh_[q.s[i]].l << 5 | sh_[q.s[i]].nprim);
-        uint64_t h = k * 0x9E3779B97F4A7C15ull;
-        Shape& s = cache_[h >> 54];
-        if (s.key != k) {
-            s.key = k;
-            s.matrix = {quartet_bytes(sh_, q, flags_), pair_bytes(sh_, q.s[0], q.s[1], flags_),
-                        pair_bytes(sh_, q.s[2], q.s[3], flags_)};
-            s.route = matrix_only_ ? 0 : axial_route(sh_, q, flags_);
-            s.nsplit = s.route ? axial_split(sh_, q, flags_, s.route == 2) : 1;
-            s.form = s.matrix;
-            if (s.route)
-                s.form = {axial_quartet_bytes(sh_, q, flags_, s.route == 2) + axial_part_bytes(sh_, q, flags_, s.nsplit),
-                          axial_pair_bytes(sh_, q.s[0], q.s[1], flags_), axial_pair_bytes(sh_, q.s[2], q.s[3], flags_)};
+        Shape* s = &find(k);
+        if (s->key == k) return *s;
+        if (2 * (used_ + 1) > slots_.size()) {
+            grow();
+            s = &find(k);
         }
-        return s;
+        ++used_;
+        s->key = k;
+        s->matrix = {quartet_bytes(sh_, q, flags_), pair_bytes(sh_, q.s[0], q.s[1], flags_),
+                     pair_bytes(sh_, q.s[2], q.s[3], flags_)};
+        s->route = matrix_only_ ? 0 : axial_route(sh_, q, flags_);
+        s->nsplit = s->route ? axial_split(sh_, q, flags_, s->route == 2) : 1;
+        s->form = s->matrix;
+        if (s->route)
+            s->form = {axial_quartet_bytes(sh_, q, flags_, s->route == 2) + axial_part_bytes(sh_, q, flags_, s->nsplit),
+                       axial_pair_bytes(sh_, q.s[0], q.s[1], flags_), axial_pair_bytes(sh_, q.s[2], q.s[3], flags_)};
+        return *s;
     }
 
   private:
+    Shape& find(uint64_t k) {
+        size_t i = (size_t)(k * 0x9E3779B97F4A7C15ull >> 32) & (slots_.size() - 1);
+        while (slots_[i].key && slots_[i].key != k) i = (i + 1) & (slots_.size() - 1);
+        return slots_[i];
+    }
+    void grow() {
+        std::vector<Shape> old(4 * slots_.size());
+        old.swap(slots_);
+        for (const Shape& s : old)
+            if (s.key) find(s.key) = s;
+    }
     const lx_shell* sh_;
     int flags_;
     bool matrix_only_;
-    std::vector<Shape> cache_;
+    std::vector<Shape> slots_;
+    size_t used_ = 0;
 };
 static_assert(LX_LMAX < 8 && LX_KMAX < 32, "a shell's l and degree fit 8 bits of a shape key");
 

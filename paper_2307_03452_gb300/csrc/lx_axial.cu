@@ -168,7 +168,9 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
     // issues of a (dd) pair (36,697 primitive pairs 1.54 -> 0.71 ms)
     if (warp == 0) {  // z expansion, lanes over v
         double n[3];
-        const double R = ax_unit3(AB, n), oz = 1.0 / zp;
+        const double oz = 1.0 / zp;
+        double R = ax_unit3(AB, n);
+        if (za * zb * oz * R * R > 800.0) R = 0.0;  // the prefactor is 0: no power of R may make that NaN
         const double PA = zb * R * oz, PB = -za * R * oz, oo2p = 0.5 * oz;
         const int v = lane;
         if (v <= L + 1) E[0][min(v, AXP_NV)] = v == 0 ? 1.0 : 0.0;
@@ -234,12 +236,6 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
     double* h = ws + pr.h_off + (int64_t)kp * cl.nh;
     for (int r = blockIdx.y * (AXP_THREADS / 32) + warp; r < cl.nhalf; r += gridDim.y * (AXP_THREADS / 32)) {
         const AxHalf hr = c_ax.halves[cl.half0 + r];
-        const int cnt = (r + 1 < cl.nhalf ? c_ax.halves[cl.half0 + r + 1].hoff : cl.nh) - hr.hoff;
-        double* hp = h + hr.hoff;
-        if (pref == 0.0) {  // centers so far apart that powers of R may have overflowed: 0 times them is 0
-            for (int e = lane; e < cnt; e += 32) hp[e] = 0.0;
-            continue;
-        }
         const AxFn &fa = fa0[hr.fa], &fb = fb0[hr.fb];
         const int ma = fa.m, mb = fb.m, M = hr.M;
         const int na = (la - ma) / 2, nb = (lb - mb) / 2, s0 = hr.slot ? min(ma, mb) : 0;
@@ -265,6 +261,8 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
         }
         __syncwarp();
         // entries (l, k), l = M .. L, k = 0 .. (L - l) / 2, of degree n = 2k + l
+        double* hp = h + hr.hoff;
+        const int cnt = (r + 1 < cl.nhalf ? c_ax.halves[cl.half0 + r + 1].hoff : cl.nh) - hr.hoff;
         for (int e = lane; e < cnt; e += 32) {
             int l = M, k = e;
             for (int nk; k >= (nk = (L - l) / 2 + 1); ++l) k -= nk;

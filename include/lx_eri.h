@@ -77,8 +77,10 @@ typedef struct {
                               log10 of the split path's error on the quartet (its output 1); the
                               quartet takes the split path with the fewest digits (4, 5, 6) whose
                               threshold lies above that prediction, else LX_PATH_FP64.  Quartets
-                              whose two transforms need fewer than LX_ROUTE_SPLIT_MIN_FLOP FLOPs
-                              (too small for the split path to be faster) take LX_PATH_FP64.
+                              whose two transforms need fewer than LX_ROUTE_SPLIT_MIN_FLOP FLOPs in
+                              matrix form take LX_PATH_FP64 (too small for the split path to be
+                              faster; so are some above that line, (ff|ff) with K = 1 and deep
+                              contractions at 6 digits, where it stands for the results' sake).
                               lx_eri_batch then waits for the stream once, to read the predictions
                               back.  Not with LX_PATH_SPLIT; not for lx_eri_graph_create,
                               lx_eri_autotune or lx_eri_batch_static */

@@ -14,12 +14,13 @@
 //      B_kappa+1(L) = (2L + 3) B_kappa(L + 1) + Z^2 B_kappa(L + 2)
 //    (d^2 f is a Gaussian, so kappa >= 1 needs no difference of Boys functions);
 //  * CD: as AB, for the ket.
-// Rotations between the frames act on each l block alone (Wigner functions).  Per primitive
-// quartet of (ii|ii) in solid functions the bra rotation, T and the ket rotation take about
-// 1.4e6 FMAs where H_ab [p+q] takes 3.5e7, and the ket transform 7e5 where the second transform takes
-// 1.3e7; what remains is 1e6 FMAs per quartet to rotate the functions to the lab frame.  No
-// step leaves FP64.  2,048 (ii|ii) quartets, solid, K = 1: 194.4 -> 14.2 ms; 200 Cartesian ones 169.1 -> 24.8 ms;
-// against 80-bit arithmetic the axial form's errors are at or below the matrix form's.
+// Rotations between the frames act on each l block alone (Wigner functions).  An uncontracted
+// (ii|ii) quartet in solid functions executes 2.3e6 FMAs for the bra rotation, T, the ket rotation
+// and the ket transform (1.4e6 on average in a 20-bohr cube, where half of the primitive quartets are far) and
+// 0.8e6 to rotate its functions to the lab frame; H_ab [p+q] takes 3.5e7 and the second transform
+// 1.3e7.  No step leaves FP64.  2,048 (ii|ii) quartets, solid, K = 1: 194.4 -> 13.6 ms; 200 Cartesian ones
+// 169.1 -> 24.7 ms.  Against extended precision the two forms' errors are of one size (the largest 2e-15 to
+// 1e-14 of the largest integral, up to 2.4 times the matrix form's where they are greater).
 //
 // Rows and columns are kept by half rows (AxHalf): the product of functions of orders m_a, m_b >= 0
 // has orders m_a + m_b and |m_a - m_b|, each with a cosine and a sine member whose coefficients
@@ -137,13 +138,13 @@ __device__ inline void frame_of(const double n[3], double F[9], double& cp, doub
 
 constexpr int AXP_THREADS = 128;
 constexpr int AXP_NV = AX_NL;  // z-derivative orders of a pair
-constexpr int AXP_SPREAD = 608;  // CTAs of a short list
+constexpr int AXP_SPREAD = 4 * AX_SMS;  // CTAs of a short list
 
 // One CTA per primitive pair (item.q = pair, item.a = primitive pair kp).  With A and B on the z
 // axis the expansion along z is the E recursion with P - A = zeta_b R / zeta, P - B = -zeta_a R / zeta,
 // and across it Laguerre's: g[q][v] = sum_{ja, jb} a_ja a_jb tau(M, s, q) zeta^-(s+q+M) E[l_a - m_a - 2 ja]
 // [l_b - m_b - 2 jb][v], s = ja + jb (+ min(m_a, m_b) for the order |m_a - m_b|); the (q, v) of one
-// degree n then go over to (k, l = n - 2k).  One warp per half row.  About 7e4 FP64 operations per
+// degree n then go over to (k, l = n - 2k).  One warp per half row.  3.8e4 FP64 instructions per
 // (ii) pair against 3.5e5 for the matrix form's H: 7.0 -> 1.36 ms for 8,192 pairs.
 __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* __restrict__ pairs,
                                                                  const WorkItem* __restrict__ items,
@@ -282,9 +283,9 @@ __global__ void __launch_bounds__(AXP_THREADS) axial_pair_kernel(const AxPair* _
 // phases of the table, the Y blocks of the bra rotation and of the rotation PQ -> CD, whose chains
 // share the lanes, then the latter's full blocks (or its factors).  One warp where it holds all
 // chains at once (L <= 4 on both sides), else two.  FP64 issue and the latency of a few dependent steps
-// bound it: Boys values and tables of 1,024 contracted (ff|ff), K = 5, 2.61 ms with two warps whose
-// sides took turns, 2.13 with the chains in one range, 1.56 with the half angles and 1.45 with the phases
-// from axial_boys_kernel.
+// bound it: Boys values and tables of 1,024 contracted (ff|ff), K = 1..5 (85,000 primitive quartets), 2.61 ms
+// with two warps whose sides took turns, 2.13 with the chains in one range, 1.56 with the half angles and
+// 1.44 with the phases from axial_boys_kernel.
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS) axial_wigner_kernel(const AxQuartet* __restrict__ qd,
                                                                const WorkItem* __restrict__ items, int lmax,
@@ -413,7 +414,7 @@ __device__ __forceinline__ void r_task(int l, int mm, int mtop, bool first, doub
 // The same for a far primitive quartet (AX_FAR): k = k' = 0, 3 FMAs per (l, l', M') instead of
 // (nk + 2) nk'.  With centers in a 20-bohr cube and exponents of 0.05 to 20 half of the primitive
 // quartets are far: main kernel 12.5 -> 9.65 ms for 2,048 (ii|ii), 72.0 -> 45.4 ms for 200 mixed
-// quartets with K = 1..5; within 6 bohr 6.21 -> 6.14 ms.
+// quartets with K = 1..5; within 6 bohr, where few are far, it costs nothing.
 __device__ __forceinline__ void t_far(int lp, int Mp, int Lb, int lo, int M, const double* __restrict__ hs,
                                       const int* __restrict__ hpre, const int* __restrict__ tinfo,
                                       const double* __restrict__ T, const double* __restrict__ tc, double* __restrict__ sc_out,
@@ -455,9 +456,10 @@ __device__ __forceinline__ void r_far(int l, int mm, int mtop, int nk, bool firs
 // of the ket primitives; 200 mixed quartets with K = 1..5: 42.9 -> 19.6 ms with the parts).  Lanes are
 // the 8 half rows (then the 16 rows: cosine, sine), so every table value is a broadcast and
 // every operand row one conflict-free shared access; groups of tasks are taken from shared
-// counters, the longest first.  Every stage is bound by the FP64 pipe: 87,300 warp FMAs per
-// (ii|ii) quartet, at the 20 cycles each that a plain FMA loop reaches 843 us of one SM (11.4 ms for 2,048
-// quartets); measured 11.1 ms within 6 bohr, where few are far, and 8.4 ms in a 20-bohr cube.
+// counters, the longest first.  Every stage is bound by the FP64 pipe, which takes a warp instruction
+// in 16 cycles: 100,000 of them per (ii|ii) quartet within 2 bohr, where none is far, 773 us of one SM or
+// 10.4 ms for 2,048 quartets (measured 11.3, with 24 of 32 lanes filled), and 70,600 in a 20-bohr cube,
+// 7.4 ms (8.4, with 22).
 // KM: the largest k range, Lk / 2 + 1, that the group's shared memory admits.
 template <int THREADS, int MINB, int KM>
 __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuartet* __restrict__ qd,
@@ -664,8 +666,8 @@ __global__ void __launch_bounds__(THREADS, MINB) axial_main_kernel(const AxQuart
 // half rows are combined into products of functions, each index is rotated from the pair's
 // frame to the lab (transposed Y, then z) and, for Cartesian output, expanded over monomials.
 // SIDE = 1: ket indices, `lanes` rows from item.a; SIDE = 0: bra indices, `lanes` columns from item.a.
-// Bound by the FP64 pipe (32,800 warp FMAs per (ii|ii) quartet for both sides, 317 us of one SM;
-// measured 315 us, 4.24 ms for 2,048 quartets; 200 Cartesian (ii|ii) 14.0 ms).  Neighbouring tasks of
+// Bound by the FP64 pipe: 37,000 warp instructions per (ii|ii) quartet for both sides, 286 us of one SM
+// or 3.85 ms for 2,048 quartets (measured 4.23, with 27 of 32 lanes filled; 200 Cartesian ones 14.0).  Neighbouring tasks of
 // a warp take the same function of neighbouring lines, so that loop lengths do not differ within a
 // warp (4.47 and 20.2 ms with neighbouring functions of one line); a tile of 16 lanes keeps the
 // accesses of a half warp in 128 bytes and four CTAs on an SM (32 lanes: 5.64 ms).
@@ -793,12 +795,15 @@ size_t axial_main_smem(int Lb, int Lk) {
 
 // The groups by shared memory: 1, 2, 3, 4 and 8 CTAs per SM of 512, 256, 256, 256 and 128 threads
 // (CTAs that share an SM fill one another's gaps at barriers and table loads; small classes, with
-// short stages, want the most warps).  (ii|ii) needs 113,896 bytes, two per SM with the bra blocks
-// left in global memory: its main kernel 9.65 -> 8.46 ms for 2,048 quartets against one CTA of 512
-// threads; (gg|gg) with 256 threads 4.41 ms for 8,192, with 128 5.34.
+// short stages, want the most warps).  n CTAs fit an SM's 228 KB if each takes 1,024 reserved bytes, 1,456 of
+// static arrays and no more than the rest; the other limits are whole KB below that.  (ii|ii) needs
+// 113,896 bytes, two per SM with the bra blocks left in global memory: its main kernel 9.65 -> 8.46 ms
+// for 2,048 quartets against one CTA of 512 threads; (gg|gg) with 256 threads 4.41 ms for 8,192, with
+// 128 5.34.
 int axial_bin(int Lb, int Lk) {
     const size_t s = axial_main_smem(Lb, Lk);
-    const int bin = s <= 25 * 1024 ? 4 : s <= 54 * 1024 ? 3 : s <= 73 * 1024 ? 2 : s <= 113900 ? 1 : 0;
+    constexpr size_t two = 228 * 1024 / 2 - 1024 - 1456;
+    const int bin = s <= 25 * 1024 ? 4 : s <= 54 * 1024 ? 3 : s <= 73 * 1024 ? 2 : s <= two ? 1 : 0;
     return std::min(bin, 8 - (Lk / 2 + 1));  // group b's kernel takes k ranges up to 8 - b
 }
 

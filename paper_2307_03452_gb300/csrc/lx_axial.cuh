@@ -19,7 +19,8 @@ constexpr int AX_NL = AX_LP + 1;
 // against 1.4, below it (dd|dp) 2.8 against 3.2.
 constexpr int AX_CONTRACTED = 4;
 constexpr int64_t AX_MIN_FMA_SOLID = 16000, AX_MIN_FMA_CART = 38000, AX_MIN_FMA_CONTRACTED = 26000;
-constexpr int AX_ONE_WAVE = 608;  // main items that run at once, four to an SM
+constexpr int AX_SMS = 152;      // SMs of a GB300
+constexpr int AX_ONE_WAVE = 4 * AX_SMS;  // main items that run at once, four to an SM
 constexpr int AX_NR = 8;         // half rows of one CTA of the main kernel
 
 // One harmonic component group of a shell: Y_lam,m r^(l - lam) for m >= 0 (and its sine partner

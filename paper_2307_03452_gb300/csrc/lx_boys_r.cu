@@ -7,8 +7,9 @@
 //
 // R: one warp per primitive quartet evaluates [r]^(m) for m = L-1 down to 0 in one shared
 // array of pyr(L) doubles, overwriting [r]^(m+1) with [r]^(m) (the paper's in-place
-// scheme, Section 3): within level m the totals n = |r| are processed from L-m down
-// to 1, so the inputs at totals n-1 and n-2 still hold level m+1 when they are read.
+// scheme, Section 3).  A position's inputs, at totals n-1 and n-2 of its n = |r|, lie below it, and
+// within level m the positions are processed from the last down to the first: those below a block of
+// positions still hold level m+1, and within a block every lane has read before any lane writes.
 // In the batch kernel each CTA is that one warp, with shared memory for the chunk's
 // largest L, so that as many quartets as shared memory allows run side by side.
 #include <cmath>
@@ -186,7 +187,7 @@ __global__ void __launch_bounds__(32) boys_r_kernel(const DQuartet* __restrict__
 // kq), as half angles and phases, and its table B_kappa(L) Z^L.  One CTA per `per` of them: first a
 // thread each, in one warp for the geometry and in the other for the Boys values, some 300 FP64
 // instructions with their divisions either way, then 8 lanes each for the table rows.  FP64 issue
-// bounds it (one warp instruction in 20 cycles and SM), so full warps in the first part count: these and
+// bounds it (one warp instruction in 16 cycles and SM), so full warps in the first part count: these and
 // the rotation blocks of 165,856 primitive quartets of (dd|dd) 2.77 ms with 8 lanes doing alike, 1.32 so;
 // `per` = 4 spreads a short list over the SMs (64 of (gg|gg) 52 us).  The
 // powers of 2 rho and Z are one chain of products with their errors carried (7 FP64 instructions per

@@ -59,7 +59,7 @@ __device__ inline double prim_norm(int l, double z) {
 // unit-normalised: sum_ij c'_i c'_j (2l-1)!! / (2(z_i+z_j))^l (pi/(z_i+z_j))^{3/2} = 1.  Each
 // primitive's normaliser is computed once and the K^2 overlaps are spread over the lanes, with
 // square roots and short products for the half-integer powers (pow takes some 150 FP64
-// instructions, which this GPU issues at one per 20 cycles and SM); blocks of one warp
+// instructions, which this GPU issues at one per 16 cycles and SM); blocks of one warp
 // spread small batches over the SMs.
 constexpr int NORM_THREADS = 32;
 template <int G>
